@@ -237,7 +237,8 @@ int sl_field_load(const char *path, void *field, int ndim, const int64_t dims[3]
  * gives bitwise the same results:
  *   SL_KERNEL_CEC_FAST     persistent FP32 split CEC kernel (32 x 32 column
  *                          tiles): CTAs per SM, 1 or 2.
- *   SL_KERNEL_CEC_SPLIT    generic split CEC kernel: planes per work item.
+ *   SL_KERNEL_CEC_SPLIT    generic split CEC kernel: planes per work item, or for
+ *                          SL_F64 and SL_F32_D64 in 3D persistent equal shares.
  *   SL_KERNEL_CIR_GROUPS   FP32 CIR kernel on four-cell groups: tile height
  *                          16 or 32, planes per work item.
  *   SL_KERNEL_UNSPLIT      generic CIR / FEC / BEC kernel: tile height 8, 16 or
@@ -383,7 +384,8 @@ int sl_tuning_clear(void);
 
 /*
  * Former interface, kept: sl_autotune_scheme for SL_CEC; *tile_z receives the
- * chosen planes per work item of the generic kernel, or the chosen CTA count
+ * chosen planes per work item of the generic kernel (0: equal shares, chosen only
+ * for SL_F64 and SL_F32_D64), or the chosen CTA count
  * (CTAs per SM times SMs) of the persistent FP32 kernel (used when dims[0] and
  * dims[1] are multiples of 32, dims[0] >= 64, dims[2] >= 8 and the buffers are
  * 16-byte aligned).

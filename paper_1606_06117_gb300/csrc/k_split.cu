@@ -541,26 +541,13 @@ cudaError_t launch_split_cec(int dtype, const void *in, void *out, const void *v
     g.chunks = (g.nz + g.tz - 1) / g.tz;
     g.tiles_x = (g.nx + TX - 1) / TX;
     const bool has_z = ndim == 3;
-    if (dtype == 1) {   // SL_F64
-        constexpr int TY = 16;
-        g.tiles_y = (g.ny + TY - 1) / TY;
-        const bool vec = lc.aligned && g.nx % 2 == 0;
-        if (has_z)
-            return vec ? dispatch_order<double, double, TX, TY, true, true>(parity, g, lc.grid, in, out, vel, fs, st)
-                       : dispatch_order<double, double, TX, TY, true, false>(parity, g, lc.grid, in, out, vel, fs, st);
-        return vec ? dispatch_order<double, double, TX, TY, false, true>(parity, g, lc.grid, in, out, vel, fs, st)
-                   : dispatch_order<double, double, TX, TY, false, false>(parity, g, lc.grid, in, out, vel, fs, st);
+    if (dtype != 0) {   // SL_F64, SL_F32_D64
+        g.tz = ndim == 3 && lc.tz > 0 ? g.tz : 0;   // default: equal shares
+        return launch_split_cec64(dtype == 2, g, parity, lc, has_z, in, out, vel, fs, st);
     }
     constexpr int TY = 32;
     g.tiles_y = (g.ny + TY - 1) / TY;
     const bool vec = lc.aligned && g.nx % 4 == 0;
-    if (dtype == 2) {   // SL_F32_D64
-        if (has_z)
-            return vec ? dispatch_order<float, double, TX, TY, true, true>(parity, g, lc.grid, in, out, vel, fs, st)
-                       : dispatch_order<float, double, TX, TY, true, false>(parity, g, lc.grid, in, out, vel, fs, st);
-        return vec ? dispatch_order<float, double, TX, TY, false, true>(parity, g, lc.grid, in, out, vel, fs, st)
-                   : dispatch_order<float, double, TX, TY, false, false>(parity, g, lc.grid, in, out, vel, fs, st);
-    }
     if (has_z)
         return vec ? dispatch_order<float, float, TX, TY, true, true>(parity, g, lc.grid, in, out, vel, fs, st)
                    : dispatch_order<float, float, TX, TY, true, false>(parity, g, lc.grid, in, out, vel, fs, st);

@@ -812,6 +812,7 @@ int sl_autotune_scheme(void *out, const void *in, const void *vel, int ndim, con
         const int occ = std::max(1, fast_grid(0) / c->num_sms);
         for (int k = 1; k <= std::min(occ, 2); ++k) cands.push_back({0, 0, k});
     } else if (fam == SL_KERNEL_CEC_SPLIT) {
+        if (dtype != SL_F32 && ndim == 3) cands.push_back({0, 0, 0});   // equal shares
         for (int tz : tzs) cands.push_back({0, tz, 0});
     } else if (fam == SL_KERNEL_CIR_GROUPS) {
         for (int ty : {16, 32})

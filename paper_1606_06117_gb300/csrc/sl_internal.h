@@ -43,6 +43,11 @@ struct FieldSet {
 cudaError_t launch_split_cec(int dtype, const void *in, void *out, const void *vel, int ndim,
                              const int64_t dims[3], const double s[3], int parity,
                              Launch lc, unsigned *status, cudaStream_t st, FieldSet fs = FieldSet());
+// The same with double arithmetic (SL_F64, or float storage for SL_F32_D64);
+// g carries the sizes, Courant factors and planes per work item (tz = 0: equal
+// shares), its tiles are set by the launch (k_split64.cu).
+cudaError_t launch_split_cec64(bool f32_storage, Geo g, int parity, Launch lc, bool has_z, const void *in, void *out,
+                               const void *vel, const FieldSet &fs, cudaStream_t st);
 cudaError_t launch_unsplit(int dtype, int scheme, const void *in, void *out, const void *vel,
                            int ndim, const int64_t dims[3], const double s[3], Launch lc,
                            unsigned *status, cudaStream_t st, FieldSet fs = FieldSet());
