@@ -24,7 +24,6 @@ namespace {
 
 template <typename T, int TX, int TY>
 struct Shape {
-    static constexpr int V = 16 / sizeof(T);             // elements per 16-byte copy
     static constexpr int HW = TX + 8;                    // staged x in [-4, TX+4)
     static constexpr int PW = HW + (sizeof(T) == 4 ? 4 : 2);   // row stride
     static constexpr int PH = TY + 6;                    // staged y in [-3, TY+3)
@@ -66,54 +65,49 @@ __device__ __forceinline__ void sts_vec(T *dst, const T (&src)[N])
 }
 
 // Stages a rectangle of rows [r0, r0+NR) (relative to the tile origin) and
-// staged columns [-4, -4 + NC) of one plane into shared memory with row
-// stride LD.  Vector path: NC multiple of V and nx multiple of V, so every
-// 16-byte copy lies inside one period.  Offsets are per-thread and
-// precomputed per work item.
+// columns [c0, c0 + NC) of one plane into shared memory with row stride LD.
+// VEC: 16-byte copies (NC and nx multiples of V, so every copy lies inside one
+// period).  Otherwise 4-byte copies of whole shared rows (all LD columns: the
+// destination of a thread's k-th copy is then tid + k NT elements in, with no
+// row arithmetic).  The periodic wrap is in per-thread source offsets, computed
+// once per work item; wrapping every element of every plane again took most of
+// the time on grids whose rows are no multiple of 16 bytes (187 x 150 x 131,
+// x,y,z / z,y,x: 123 / 173 us before, 55 / 79 now; 46 / 69 us with rows of 188).
 template <typename T, int NT, int NR, int NC, int LD, bool VEC>
 struct Stager {
-    static constexpr int V = 16 / sizeof(T);
-    static constexpr int CPR = NC / V;
+    static constexpr int V = VEC ? 16 / sizeof(T) : 1;
+    static constexpr int CPR = VEC ? NC / V : LD;
     static constexpr int N = NR * CPR;
-    static constexpr int K = VEC ? (N + NT - 1) / NT : 1;
+    static constexpr int K = (N + NT - 1) / NT;
     int off[K];
 
     __device__ __forceinline__ void setup(int tid, int x0, int y0, int r0, int c0, int nx, int ny)
     {
-        if constexpr (VEC) {
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const int idx = tid + k * NT;
-                if (idx < N) {
-                    const int row = idx / CPR, cc = idx - (idx / CPR) * CPR;
-                    const int gy = wrapi(y0 + r0 + row, ny);
-                    const int gx = wrapi(x0 + c0 + cc * V, nx);
-                    off[k] = gy * nx + gx;
-                } else {
-                    off[k] = -1;
-                }
+        for (int k = 0; k < K; ++k) {
+            const int idx = tid + k * NT;
+            if (idx < N) {
+                const int row = idx / CPR, cc = idx - (idx / CPR) * CPR;
+                const int gy = wrapi(y0 + r0 + row, ny);
+                const int gx = wrapi(x0 + c0 + cc * V, nx);
+                off[k] = gy * nx + gx;
+            } else {
+                off[k] = -1;
             }
         }
     }
 
-    __device__ __forceinline__ void issue(int tid, T *dst, const T *src, int x0, int y0, int r0, int c0, int nx,
-                                          int ny) const
+    __device__ __forceinline__ void issue(int tid, T *dst, const T *src) const
     {
-        if constexpr (VEC) {
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const int idx = tid + k * NT;
-                if (off[k] >= 0) {
-                    const int row = idx / CPR, cc = idx - (idx / CPR) * CPR;
-                    cp_async16(dst + row * LD + cc * V, src + off[k]);
-                }
-            }
-        } else {
-            for (int idx = tid; idx < NR * NC; idx += NT) {
-                const int row = idx / NC, col = idx - (idx / NC) * NC;
-                const int gy = wrapi(y0 + r0 + row, ny);
-                const int gx = wrapi(x0 + c0 + col, nx);
-                cp_async_elem(dst + row * LD + col, src + (int64_t)gy * nx + gx);
+        for (int k = 0; k < K; ++k) {
+            const int idx = tid + k * NT;
+            if (off[k] < 0) continue;
+            if constexpr (VEC) {
+                const int row = idx / CPR, cc = idx - (idx / CPR) * CPR;
+                cp_async16(dst + row * LD + cc * V, src + off[k]);
+            } else {
+                cp_async_elem(dst + idx, src + off[k]);
             }
         }
     }
@@ -176,12 +170,12 @@ __device__ __forceinline__ void xyz_item(const Geo &g, int item, const T *__rest
     const int plast = HAS_Z ? z1 + 2 : 0;
     auto issue = [&](int p, int slot) {
         const int64_t base = (int64_t)wrapi(p, g.nz) * g.plane;
-        stPhi.issue(tid, sPhi + slot * K::SZ_PHI, in + base, x0, y0, -3, -4, g.nx, g.ny);
-        stPhi.issue(tid, sCx + slot * K::SZ_PHI, vel + base, x0, y0, -3, -4, g.nx, g.ny);
-        stCy.issue(tid, sCy + slot * K::SZ_CY, vel + g.ncell + base, x0, y0, -2, 0, g.nx, g.ny);
+        stPhi.issue(tid, sPhi + slot * K::SZ_PHI, in + base);
+        stPhi.issue(tid, sCx + slot * K::SZ_PHI, vel + base);
+        stCy.issue(tid, sCy + slot * K::SZ_CY, vel + g.ncell + base);
         if constexpr (HAS_Z) {
             const int64_t bz = (int64_t)wrapi(p - 1, g.nz) * g.plane;
-            stCz.issue(tid, sCz + slot * K::SZ_CZ, vel + 2 * g.ncell + bz, x0, y0, 0, 0, g.nx, g.ny);
+            stCz.issue(tid, sCz + slot * K::SZ_CZ, vel + 2 * g.ncell + bz);
         }
         cp_async_commit();
     };
@@ -323,15 +317,15 @@ __device__ __forceinline__ void zyx_item(const Geo &g, int item, const T *__rest
     const int plast = HAS_Z ? z1 + 2 : 0;
     auto issue = [&](int p, int slot) {
         const int64_t base = (int64_t)wrapi(p, g.nz) * g.plane;
-        stPhi.issue(tid, sPhi + slot * K::SZ_PHI, in + base, x0, y0, -3, -4, g.nx, g.ny);
+        stPhi.issue(tid, sPhi + slot * K::SZ_PHI, in + base);
         int64_t bk = base;
         if constexpr (HAS_Z) {
             const int64_t bz = (int64_t)wrapi(p - 1, g.nz) * g.plane;
-            stPhi.issue(tid, sCz + slot * K::SZ_CZ, vel + 2 * g.ncell + bz, x0, y0, -3, -4, g.nx, g.ny);
+            stPhi.issue(tid, sCz + slot * K::SZ_CZ, vel + 2 * g.ncell + bz);
             bk = (int64_t)wrapi(p - 3, g.nz) * g.plane;
         }
-        stCy.issue(tid, sCy + slot * K::SZ_CY, vel + g.ncell + bk, x0, y0, -2, -4, g.nx, g.ny);
-        stCx.issue(tid, sCx + slot * K::SZ_CX, vel + bk, x0, y0, 0, -4, g.nx, g.ny);
+        stCy.issue(tid, sCy + slot * K::SZ_CY, vel + g.ncell + bk);
+        stCx.issue(tid, sCx + slot * K::SZ_CX, vel + bk);
         cp_async_commit();
     };
 
