@@ -400,11 +400,11 @@ cudaError_t go(Geo g, int grid, const void *in, void *out, const void *vel, cons
     const int64_t total = tiles * (g.tz > 0 ? g.chunks : g.nz);
     int64_t gr = total;
     if (HAS_Z && g.tz == 0) {
-        // Equal shares: a share begins with six planes of z warm-up, so no more
-        // CTAs than keep shares of 12 planes or more, and no more than the GPU
-        // holds at a time (all fields together).
+        // Equal shares, of two planes or more, for as many CTAs as the GPU holds
+        // at a time (all fields together): a share begins with six planes of z
+        // warm-up, but a CTA that would otherwise not run costs nothing.
         gr = (resident[dev] + fs.n - 1) / fs.n;
-        if (gr > (total + 11) / 12) gr = (total + 11) / 12;
+        if (gr > (total + 1) / 2) gr = (total + 1) / 2;
     }
     if (grid > 0 && grid < gr) gr = grid;
     if (gr < 1) gr = 1;
