@@ -241,11 +241,11 @@ int sl_field_load(const char *path, void *field, int ndim, const int64_t dims[3]
  *                          SL_F64 and SL_F32_D64 in 3D persistent equal shares.
  *   SL_KERNEL_CIR_GROUPS   FP32 CIR kernel on four-cell groups: tile height
  *                          16 or 32, planes per work item.
- *   SL_KERNEL_UNSPLIT      generic CIR / FEC / BEC kernel: tile height 8, 16 or
- *                          32 (FP32 3D grids with dims[0] % 4 == 0 and aligned
- *                          buffers; otherwise the dtype's fixed height) and
- *                          planes per work item, or for 3D BEC (persistent
- *                          equal shares) CTAs per SM, 1 to 3.
+ *   SL_KERNEL_UNSPLIT      generic CIR / FEC / BEC kernels: on large FP32 3D grids
+ *                          with dims[0] % 4 == 0 and aligned buffers tile height
+ *                          8, 16 or 32 (otherwise a fixed height) and planes per
+ *                          work item, or for 3D BEC and the other FP32 3D grids
+ *                          (persistent equal shares) CTAs per SM.
  * A choice is cached per (dims, scheme, dtype) in the process and used by
  * sl_advect, sl_advect_multi, sl_advect_host and sl_batch_create whenever the
  * request is served by the kernel it was tuned for.

@@ -1,4 +1,5 @@
-// k_unsplit.cu -- fused unsplit CIR / FEC / BEC step.
+// k_unsplit.cu -- fused unsplit CIR / FEC / BEC step (2D, double arithmetic, and
+// large FP32 3D grids of whole 16-byte chunks; k_unsplit32.cu takes the others).
 //
 // The multilinear operator L_U (Sec. 2; eq. CIR2D and its 3D tensor-product
 // analogue) is applied 1, 2 or 3 times (Table 1, "Nb of calls"):
@@ -415,11 +416,19 @@ cudaError_t launch_unsplit(int dtype, int scheme, const void *in, void *out, con
     if (dtype == 1) return by_shape<double, double, 8>(scheme, has_z, lc.aligned && g.nx % 2 == 0, g, lc.grid, in, out, vel, fs, st);
     if (dtype == 2) return by_shape<float, double, 16>(scheme, has_z, lc.aligned && g.nx % 4 == 0, g, lc.grid, in, out, vel, fs, st);
     const bool vec = lc.aligned && g.nx % 4 == 0;
-    // FP32 3D grids with vector staging: tile heights 8 and 32 besides 16 (a
-    // launch-shape choice; a cell's arithmetic does not depend on it)
-    if (has_z && vec && lc.ty == 8) return by_scheme<float, float, 8, true, true>(scheme, g, lc.grid, in, out, vel, fs, st);
-    if (has_z && vec && lc.ty == 32) return by_scheme<float, float, 32, true, true>(scheme, g, lc.grid, in, out, vel, fs, st);
-    return by_shape<float, float, 16>(scheme, has_z, vec, g, lc.grid, in, out, vel, fs, st);
+    if (unsplit32_serves(scheme, ndim, dims, vec)) {
+        g.tz = lc.tz > 0 ? g.tz : 0;   // default: equal shares
+        return launch_unsplit32(scheme, g, lc.grid, in, out, vel, fs, st);
+    }
+    if (has_z) {
+        // tile heights 8 and 32 besides 16 (a launch-shape choice; a cell's
+        // arithmetic does not depend on it)
+        if (lc.ty == 8) return by_scheme<float, float, 8, true, true>(scheme, g, lc.grid, in, out, vel, fs, st);
+        if (lc.ty == 32) return by_scheme<float, float, 32, true, true>(scheme, g, lc.grid, in, out, vel, fs, st);
+        return by_scheme<float, float, 16, true, true>(scheme, g, lc.grid, in, out, vel, fs, st);
+    }
+    return vec ? by_scheme<float, float, 16, false, true>(scheme, g, lc.grid, in, out, vel, fs, st)
+               : by_scheme<float, float, 16, false, false>(scheme, g, lc.grid, in, out, vel, fs, st);
 }
 
 }  // namespace sl

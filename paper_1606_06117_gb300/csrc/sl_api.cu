@@ -819,13 +819,19 @@ int sl_autotune_scheme(void *out, const void *in, const void *vel, int ndim, con
             if (ty == 16 || dims[1] >= 32)
                 for (int tz : tzs) cands.push_back({ty, tz, 0});
     } else {
-        std::vector<int> tys = {0};
-        if (dtype == SL_F32 && ndim == 3 && aligned && dims[0] % 4 == 0) tys = {8, 16, 32};
-        for (int ty : tys) {
-            if (scheme == SL_BEC && ndim == 3)
-                for (int k = 1; k <= 3; ++k) cands.push_back({ty, 0, k});
-            else
-                for (int tz : tzs) cands.push_back({ty, tz, 0});
+        const bool vec = aligned && dims[0] % 4 == 0;
+        if (dtype == SL_F32 && unsplit32_serves(scheme, ndim, dims, vec)) {
+            for (int k = 0; k <= 2; ++k) cands.push_back({0, 0, k});   // equal shares
+            for (int tz : tzs) cands.push_back({0, tz, 0});
+        } else {
+            std::vector<int> tys = {0};
+            if (dtype == SL_F32 && ndim == 3) tys = {8, 16, 32};
+            for (int ty : tys) {
+                if (scheme == SL_BEC && ndim == 3)
+                    for (int k = 1; k <= 3; ++k) cands.push_back({ty, 0, k});
+                else
+                    for (int tz : tzs) cands.push_back({ty, tz, 0});
+            }
         }
     }
 

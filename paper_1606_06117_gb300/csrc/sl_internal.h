@@ -51,6 +51,12 @@ cudaError_t launch_split_cec64(bool f32_storage, Geo g, int parity, Launch lc, b
 cudaError_t launch_unsplit(int dtype, int scheme, const void *in, void *out, const void *vel,
                            int ndim, const int64_t dims[3], const double s[3], Launch lc,
                            unsigned *status, cudaStream_t st, FieldSet fs = FieldSet());
+// The same for FP32 in 3D, any size and alignment (k_unsplit32.cu), and whether it
+// serves a request (vec: 16-byte aligned buffers and rows of whole 16-byte
+// chunks); g as for launch_split_cec64.
+bool unsplit32_serves(int scheme, int ndim, const int64_t dims[3], bool vec);
+cudaError_t launch_unsplit32(int scheme, Geo g, int grid, const void *in, void *out, const void *vel,
+                             const FieldSet &fs, cudaStream_t st);
 // FP32 3D CIR kernel on four-cell groups (k_cir_fast.cu); launch_unsplit routes
 // eligible CIR steps to it.
 bool cir_fast_eligible(int dtype, int ndim, const int64_t dims[3], bool aligned);
