@@ -17,9 +17,12 @@
 //                  number r shifted by m cells (third order); for |C| < 1 it
 //                  is the local CEC.
 //
-// Unfused: one gather kernel per interpolation call, each with the scheme's
-// pointwise combination as its epilogue, and one gather kernel for the CEC
-// correction.  Intermediate fields live in a caller-owned workspace.
+// A CEC sweep whose lines fit in shared memory is one kernel.  Otherwise one
+// gather kernel per interpolation call, each with the scheme's pointwise
+// combination as its epilogue, and one for the CEC correction.  Intermediate
+// fields live in a caller-owned workspace.
+#include <algorithm>
+
 #include "sl_internal.h"
 
 namespace sl {
@@ -212,180 +215,265 @@ dim3 wide_grid(const WideGeo &g)
 // A CEC sweep along AX only reads the line it works on: L_U[Phi] at a cell
 // gathers Phi near the cell's departure point, delta gathers L_U[Phi] near the
 // reversed departure point, and the correction gathers delta near the
-// departure cell.  So a CTA holds W whole lines in shared memory (Phi, then
-// delta in its place; the Courant numbers; L_U[Phi]) and writes the sweep's
-// output: one read of Phi and u_AX and one write per cell (12 B in FP32), in
-// place of the 44 B of the three gathers above.  Lines along x are rows
-// (contiguous); lines along y or z are W adjacent x columns, so that every
-// load and store of a warp is coalesced along x.
-constexpr int kSweepThreads = 256;
-// 24 KB per CTA (8 lines of 256 cells in FP32): measured fastest among 12,
-// 24, 36, 48 and 96 KB, several CTAs per SM hiding each other's barriers
-constexpr size_t kSweepSmem = 24 * 1024;
+// departure cell.  So a CTA holds whole lines in shared memory (Phi, then
+// delta in its place; L_U[Phi]) and writes the sweep's output: one read of Phi
+// and u_AX and one write per cell (12 B in FP32), in place of the 44 B of the
+// three gathers above.  Lines along x are rows (contiguous); lines along y or z
+// are W adjacent x columns, so that every load and store of a warp is coalesced
+// along x; the last column block of a row may be partial.
+//
+// What bounds it: instruction issue, so each cell's departure is worked out
+// once, m = trunc C, r = C - m, and kept in registers with both gather
+// positions.  With lo = i - m - [r > 0] the departure lies between lo and
+// lo + 1 (fraction [r > 0] - r), and these two are also the departure cell and
+// its upwind neighbour, which the correction reads; the reversed departure lies
+// between lo' = i + m - [r < 0] and lo' + 1 (fraction [r < 0] + r).  Positions
+// wrap by an unsigned minimum of p, p + n and p - n, and every line repeats its
+// first element at its end, so that lo + 1 needs no wrap.  Courant numbers of n
+// or more take a remainder first.
+// Measured (256^3 FP32 at CFL 3.64, us per step of three sweeps): 291 with the
+// Courant numbers in shared memory and three separate departure calculations
+// (170-179 instructions per cell and sweep), 178 now.
+// Cells per thread: with 4 a thread keeps to 64 registers, so that 32 warps fit an
+// SM (8 took 98).
+constexpr int kSweepCells = 4;
 
-template <typename T, int AX, int W>
-__global__ void __launch_bounds__(kSweepThreads)
-k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict__ vel, WideGeo g, int64_t nlines)
+// unsigned wrap of p in [-n, 2 n) into [0, n)
+__device__ __forceinline__ int wrap3(int p, int n)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    return (int)min(min((unsigned)p, (unsigned)(p + n)), (unsigned)(p - n));
+}
+
+// r > 0; a double's from its bits, since a double comparison costs as much as a
+// double multiply-add, of which an SM issues two per clock
+__device__ __forceinline__ bool positive(float r) { return r > 0.f; }
+__device__ __forceinline__ bool positive(double r) { return __double_as_longlong(r) > 0; }
+// |c| < n (false for a NaN)
+__device__ __forceinline__ bool below(float c, int n) { return fabsf(c) < (float)n; }
+__device__ __forceinline__ bool below(double c, int n)
+{
+    return (__double_as_longlong(c) & 0x7fffffffffffffffll) < __double_as_longlong((double)n);
+}
+
+// LW: log2 of the columns per tile (AX > 0).  For AX = 0 a tile is `rows` rows.
+// Persistent CTAs; the loads of a CTA's next tile are issued before it works on
+// the current one, so that DRAM latency runs under the three gathers (without
+// that the y and z sweeps stalled on their loads).
+template <typename T, int AX, int LW, int NT>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 1024 / NT : 1)
+k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict__ vel, WideGeo g, T sc, int rows,
+             int tiles)
+{
+    constexpr int E = kSweepCells, W = 1 << LW;
+    // Everything in shared memory is addressed in bytes: Phi, then delta, in lines
+    // of n + 1 and a spare place; then L_U[Phi] the same way.
+    extern __shared__ __align__(16) char sm[];
+    constexpr int B = sizeof(T);
     const int n = g.n[AX];
-    T *S = reinterpret_cast<T *>(smem_raw);   // Phi, then delta
-    T *V = S + (size_t)W * n;                 // Courant numbers along AX
-    T *Lb = V + (size_t)W * n;                // L_U[Phi]
+    const int lines = AX == 0 ? rows : W;
+    const int spare = lines * (n + 1) * B, LB = spare + B;
     const int tid = threadIdx.x;
-    const T sc = T(g.s[AX]);
     bool bad = false;
-    // first element of line w = 0, and the stride along the line
-    int64_t base, stride, row0 = 0;
+    const T *const va = vel + (int64_t)AX * g.ncell;
+    constexpr int step = (AX == 0 ? 1 : W) * B;        // along a line
+    const int period = n * step;
+    const int xt = (g.n[0] + W - 1) >> LW;
+    const int64_t stride = AX == 1 ? g.n[0] : (int64_t)g.n[0] * g.n[1];   // along a line (AX > 0)
+    // Cell k of this thread has flat index e = tid + k NT of the tile: line e / n
+    // and position e mod n of it (AX = 0), or column e mod W and position e / W.
+    // pos: its distance from the line's start (AX = 0) or from column 0; own: its
+    // place.  Cells beyond the tile's lines go to the spare place, and cells of a
+    // partial tile beyond the grid work on zeros in places of their own.
+    const int count = AX == 0 ? rows * n : n << LW;
+    int pos[E], line[E], own[E];
+    bool rep[E];                                       // repeated at its line's end
     if constexpr (AX == 0) {
-        row0 = (int64_t)blockIdx.x * W;
-        base = row0 * g.n[0];
-        stride = 1;
+        int w = tid / n, i = tid - w * n;
+        const int dw = NT / n, di = NT - dw * n;
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const bool in = tid + k * NT < count;
+            pos[k] = in ? i * B : 0;
+            line[k] = in ? w * (n + 1) * B : 0;
+            own[k] = in ? line[k] + pos[k] : spare;
+            rep[k] = in && i == 0;
+            w += dw;
+            i += di;
+            if (i >= n) {
+                i -= n;
+                ++w;
+            }
+        }
     } else {
-        const int xt = g.n[0] / W;
-        const int64_t q = blockIdx.x / xt;                         // z (AX = 1) or y (AX = 2)
-        const int x0 = (int)(blockIdx.x - q * xt) * W;
-        base = (AX == 1 ? q * g.n[0] * (int64_t)g.n[1] : q * g.n[0]) + x0;
-        stride = AX == 1 ? g.n[0] : (int64_t)g.n[0] * g.n[1];
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const int e = tid + k * NT;
+            pos[k] = e < count ? e * B : 0;
+            line[k] = 0;
+            own[k] = e < count ? e * B : spare;
+            rep[k] = k == 0 && tid < W;
+        }
     }
-    auto sidx = [&](int w, int i) { return AX == 0 ? w * n + i : i * W + w; };
-    auto gidx = [&](int w, int i) { return AX == 0 ? base + (int64_t)w * n + i : base + (int64_t)i * stride + w; };
-    // rows of a power-of-two length take one flat loop with shifts
-    const int lg = (n & (n - 1)) == 0 ? __ffs(n) - 1 : -1;
-    const int rows = AX == 0 ? (int)min((int64_t)W, nlines - row0) : W;
-    auto each = [&](auto f) {
+    auto lds = [&](int q) { return *reinterpret_cast<const T *>(sm + q); };
+    auto put = [&](int off, int k, T x) {
+        *reinterpret_cast<T *>(sm + off + own[k]) = x;
+        if ((AX == 0 || k == 0) && rep[k]) *reinterpret_cast<T *>(sm + off + own[k] + period) = x;
+    };
+
+    T v[E], c[E];
+    int64_t q0;        // element of cell 0
+    int limit;         // cells with k NT < limit are inside the grid
+    const int64_t hop = AX == 0 ? NT : (int64_t)(NT >> LW) * stride;   // from cell k to k + 1
+    const int64_t first = AX == 0 ? tid : (int64_t)(tid >> LW) * stride + (tid & (W - 1));
+    auto load = [&](int b) {
         if constexpr (AX == 0) {
-            if (lg >= 0) {
-                for (int e = tid; e < (rows << lg); e += kSweepThreads) f(e >> lg, e & (n - 1));
-            } else {
-                for (int w = 0; w < rows; ++w)
-                    for (int i = tid; i < n; i += kSweepThreads) f(w, i);
-            }
+            const int64_t row0 = (int64_t)b * rows, all = (int64_t)g.n[1] * g.n[2];
+            q0 = row0 * n + first;
+            limit = (int)min((int64_t)rows, all - row0) * n - tid;
         } else {
-            for (int e = tid; e < W * n; e += kSweepThreads) f(e % W, e / W);
+            const int q = b / xt, x0 = (b - q * xt) << LW;   // q: z (AX = 1) or y (AX = 2)
+            q0 = (AX == 1 ? (int64_t)q * g.n[0] * g.n[1] : (int64_t)q * g.n[0]) + x0 + first;
+            limit = x0 + (tid & (W - 1)) < g.n[0] ? count - tid : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const bool ok = k * NT < limit;
+            v[k] = ok ? src[q0 + k * hop] : T(0);
+            c[k] = ok ? va[q0 + k * hop] : T(0);
         }
     };
-    // staging: each thread issues the loads of B elements before storing any,
-    // so that B global loads of Phi and B of u_AX are in flight at once (4
-    // measured fastest of 1, 2, 4, 8 and 16: more costs registers and CTAs)
-    constexpr int B = 4;
-    auto stage = [&](const int (&w)[B], const int (&i)[B], const bool (&ok)[B]) {
-        T a[B], c[B];
+    if (blockIdx.x < (unsigned)tiles) load(blockIdx.x);
+    for (int b = blockIdx.x; b < tiles; b += gridDim.x) {
+        int lo[E], back[E];           // places of the departure and of the reversed departure
+        T r[E], phi[E], L[E];
+        bool far = false;
 #pragma unroll
-        for (int k = 0; k < B; ++k) {
-            const int64_t q = ok[k] ? gidx(w[k], i[k]) : 0;
-            a[k] = ok[k] ? src[q] : T(0);
-            c[k] = ok[k] ? vel[(int64_t)AX * g.ncell + q] * sc : T(0);
+        for (int k = 0; k < E; ++k) {
+            c[k] *= sc;
+            far |= !below(c[k], n);
         }
+        int m[E];
+        if (!__any_sync(0xffffffffu, far)) {
 #pragma unroll
-        for (int k = 0; k < B; ++k) {
-            if (!ok[k]) continue;
-            if (!(fabs(c[k]) < T(1073741824.0))) {
-                bad = true;
-                c[k] = T(0);
+            for (int k = 0; k < E; ++k) {
+                const T f = trunc(c[k]);
+                m[k] = (int)f;
+                r[k] = c[k] - f;
             }
-            S[sidx(w[k], i[k])] = a[k];
-            V[sidx(w[k], i[k])] = c[k];
-        }
-    };
-    if constexpr (AX == 0) {
-        for (int w0 = 0; w0 < W; w0 += B)
-            for (int i0 = tid; i0 < n; i0 += kSweepThreads) {
-                int w[B], i[B];
-                bool ok[B];
+        } else {   // a period or more somewhere, or a number that cannot be used
 #pragma unroll
-                for (int k = 0; k < B; ++k) {
-                    w[k] = w0 + k;
-                    i[k] = i0;
-                    ok[k] = w[k] < W && row0 + w[k] < nlines;
+            for (int k = 0; k < E; ++k) {
+                if (!(fabs(c[k]) < T(1073741824.0))) {
+                    bad = true;
+                    c[k] = T(0);
                 }
-                stage(w, i, ok);
+                const T f = trunc(c[k]);
+                m[k] = (int)f % n;
+                r[k] = c[k] - f;
             }
-    } else {
-        for (int e0 = tid; e0 < W * n; e0 += kSweepThreads * B) {
-            int w[B], i[B];
-            bool ok[B];
+        }
 #pragma unroll
-            for (int k = 0; k < B; ++k) {
-                const int e = e0 + k * kSweepThreads;
-                ok[k] = e < W * n;
-                w[k] = e % W;
-                i[k] = e / W;
-            }
-            stage(w, i, ok);
+        for (int k = 0; k < E; ++k) {
+            const int d = m[k] * step;
+            lo[k] = line[k] + wrap3(pos[k] - d - (positive(r[k]) ? step : 0), period);
+            back[k] = LB + line[k] + wrap3(pos[k] + d - (positive(-r[k]) ? step : 0), period);
+            phi[k] = v[k];
+        }
+        T *const dst = out + q0;
+        const int climit = limit;
+        __syncthreads();   // the previous tile's delta has been read
+#pragma unroll
+        for (int k = 0; k < E; ++k) put(0, k, phi[k]);
+        if (b + (int)gridDim.x < tiles) load(b + gridDim.x);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < E; ++k) {                                     // L_U[Phi]
+            const T a = lds(lo[k]), d = lds(lo[k] + step);
+            L[k] = a + ((positive(r[k]) ? T(1) : T(0)) - r[k]) * (d - a);
+        }
+#pragma unroll
+        for (int k = 0; k < E; ++k) put(LB, k, L[k]);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < E; ++k) {                                     // delta = Phi - L_{-U}[L_U[Phi]]
+            const T a = lds(back[k]), d = lds(back[k] + step);
+            phi[k] -= a + ((positive(-r[k]) ? T(1) : T(0)) + r[k]) * (d - a);
+        }
+#pragma unroll
+        for (int k = 0; k < E; ++k) put(0, k, phi[k]);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < E; ++k) {                                     // departure-cell correction
+            const T a = lds(lo[k]), d = lds(lo[k] + step);
+            const T dj = positive(r[k]) ? d : a;
+            const T du = positive(-r[k]) ? d : a;                             // r = 0: the cell itself
+            const T res = L[k] + dj * T(0.5) + (T(1) + fabs(r[k])) * T(1.0 / 6.0) * (du - dj);
+            if (k * NT < climit) dst[k * hop] = res;
         }
     }
-    __syncthreads();
-    each([&](int w, int i) {                                          // L_U[Phi]
-        T f;
-        bool unused = false;
-        const int b0 = wrapn(i + floor_split<T>(-V[sidx(w, i)], f, unused), n);
-        const int b1 = b0 + 1 == n ? 0 : b0 + 1;
-        const T a = S[sidx(w, b0)], b = S[sidx(w, b1)];
-        Lb[sidx(w, i)] = a + f * (b - a);
-    });
-    __syncthreads();
-    each([&](int w, int i) {                                          // delta = Phi - L_{-U}[L_U[Phi]]
-        T f;
-        bool unused = false;
-        const int b0 = wrapn(i + floor_split<T>(V[sidx(w, i)], f, unused), n);
-        const int b1 = b0 + 1 == n ? 0 : b0 + 1;
-        const T a = Lb[sidx(w, b0)], b = Lb[sidx(w, b1)];
-        S[sidx(w, i)] = S[sidx(w, i)] - (a + f * (b - a));
-    });
-    __syncthreads();
-    each([&](int w, int i) {                                          // departure-cell correction
-        const T c = V[sidx(w, i)], m = trunc(c), r = c - m;
-        const int sg = (r > T(0)) - (r < T(0));
-        const int j = wrapn(i - (int)m, n), ju = wrapn(i - (int)m - sg, n);
-        const T dj = S[sidx(w, j)], du = S[sidx(w, ju)];
-        out[gidx(w, i)] = Lb[sidx(w, i)] + dj * T(0.5) + (T(1) + fabs(r)) * T(1.0 / 6.0) * (du - dj);
-    });
     flag_cfl(g.status, bad);
 }
 
-template <typename T, int AX, int W>
-cudaError_t go_sweep(T *dst, const T *src, const T *vel, const WideGeo &g, cudaStream_t st)
+template <typename T, int AX, int LW, int NT>
+cudaError_t go_sweep(T *dst, const T *src, const T *vel, const WideGeo &g, int rows, unsigned tiles, cudaStream_t st)
 {
-    static int ready[64] = {};
+    // at most NT kSweepCells cells and their repeated elements, in two arrays
+    constexpr size_t cap = 2 * sizeof(T) * (size_t)(NT * kSweepCells + 1 + (AX == 0 ? 256 : 1 << LW));
+    static int ready[64] = {};   // resident CTAs of the GPU
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    const size_t smem = 3 * sizeof(T) * (size_t)W * g.n[AX];
     if (!ready[dev]) {
-        e = cudaFuncSetAttribute(k_wide_sweep<T, AX, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmem);
+        e = cudaFuncSetAttribute(k_wide_sweep<T, AX, LW, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
         if (e != cudaSuccess) return e;
-        ready[dev] = 1;
+        int per_sm = 0, sms = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wide_sweep<T, AX, LW, NT>, NT, cap);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        ready[dev] = sms * (per_sm > 0 ? per_sm : 1);
     }
-    const int64_t nlines = AX == 0 ? (int64_t)g.n[1] * g.n[2] : 0;
-    const int64_t blocks = AX == 0 ? (nlines + W - 1) / W : (int64_t)(g.n[0] / W) * (AX == 1 ? g.n[2] : g.n[1]);
-    k_wide_sweep<T, AX, W><<<(unsigned)blocks, kSweepThreads, smem, st>>>(dst, src, vel, g, nlines);
+    const size_t lines = AX == 0 ? (size_t)rows : (size_t)1 << LW;
+    const size_t smem = 2 * sizeof(T) * (lines * (size_t)(g.n[AX] + 1) + 1);
+    const unsigned grid = std::min(tiles, (unsigned)ready[dev]);
+    k_wide_sweep<T, AX, LW, NT><<<grid, NT, smem, st>>>(dst, src, vel, g, T(g.s[AX]), rows, (int)tiles);
     return cudaGetLastError();
 }
 
-// The fused sweep with the most lines per CTA that fit kSweepSmem (W | nx for
-// lines along y and z); false when not even one line fits.
+// The fused sweep, with 512 threads (2048 cells); lines over 256 cells along y or
+// z take 1024, where 2048 cells would leave column blocks of fewer than 32
+// bytes, and lines of at most 32 cells 256.  False when a line has more than
+// 4096 cells or the blocks do not fit a grid.
 template <typename T, int AX>
 bool sweep_fused(T *dst, const T *src, const T *vel, const WideGeo &g, cudaStream_t st, cudaError_t &e)
 {
-    const size_t line = 3 * sizeof(T) * (size_t)g.n[AX];
-    for (int W = 32; W >= 1; W /= 2) {
-        if (W * line > kSweepSmem || (AX != 0 && g.n[0] % W != 0)) continue;
-        const int64_t blocks = AX == 0 ? ((int64_t)g.n[1] * g.n[2] + W - 1) / W
-                                       : (int64_t)(g.n[0] / W) * (AX == 1 ? g.n[2] : g.n[1]);
+    const int n = g.n[AX];
+    if (n > 1024 * kSweepCells) return false;
+    const int64_t lines = g.ncell / n;
+    if constexpr (AX == 0) {
+        const int nt = n > 512 * kSweepCells ? 1024 : 512;
+        const int rows = (int)std::min<int64_t>(std::min(256, nt * kSweepCells / n), lines);
+        const int64_t blocks = (lines + rows - 1) / rows;
         if (blocks > 0x7fffffff) return false;
-        switch (W) {
-        case 32: e = go_sweep<T, AX, 32>(dst, src, vel, g, st); break;
-        case 16: e = go_sweep<T, AX, 16>(dst, src, vel, g, st); break;
-        case 8: e = go_sweep<T, AX, 8>(dst, src, vel, g, st); break;
-        case 4: e = go_sweep<T, AX, 4>(dst, src, vel, g, st); break;
-        case 2: e = go_sweep<T, AX, 2>(dst, src, vel, g, st); break;
-        default: e = go_sweep<T, AX, 1>(dst, src, vel, g, st); break;
+        e = nt == 1024 ? go_sweep<T, 0, 0, 1024>(dst, src, vel, g, rows, (unsigned)blocks, st)
+                       : go_sweep<T, 0, 0, 512>(dst, src, vel, g, rows, (unsigned)blocks, st);
+    } else {
+        const int lw = n <= 64 ? 5 : n <= 128 ? 4 : n <= 512 ? 3 : n <= 1024 ? 2 : n <= 2048 ? 1 : 0;
+        const int64_t blocks = (((int64_t)g.n[0] + (1 << lw) - 1) >> lw) * (lines / g.n[0]);
+        if (blocks > 0x7fffffff) return false;
+        const unsigned b = (unsigned)blocks;
+        switch (lw) {
+        case 5: e = n <= 32 ? go_sweep<T, AX, 5, 256>(dst, src, vel, g, 0, b, st)
+                            : go_sweep<T, AX, 5, 512>(dst, src, vel, g, 0, b, st); break;
+        case 4: e = go_sweep<T, AX, 4, 512>(dst, src, vel, g, 0, b, st); break;
+        case 3: e = n <= 256 ? go_sweep<T, AX, 3, 512>(dst, src, vel, g, 0, b, st)
+                             : go_sweep<T, AX, 3, 1024>(dst, src, vel, g, 0, b, st); break;
+        case 2: e = go_sweep<T, AX, 2, 1024>(dst, src, vel, g, 0, b, st); break;
+        case 1: e = go_sweep<T, AX, 1, 1024>(dst, src, vel, g, 0, b, st); break;
+        default: e = go_sweep<T, AX, 0, 1024>(dst, src, vel, g, 0, b, st); break;
         }
-        return true;
     }
-    return false;
+    return true;
 }
 
 template <typename T, int NDIM, int AX, int EPI>
