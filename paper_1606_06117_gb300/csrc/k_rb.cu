@@ -27,10 +27,16 @@
 // clock and SM), so the step is arranged to spend few FP64 operations and to
 // spread them over many SMs: each producer writes its cells' ghost images
 // itself (no separate fill pass), the forces kernel also gives the divergence,
-// the transforms run one CTA per mode row with coalesced or broadcast loads,
-// the per-cell kernels use small CTAs, and long runs replay the step from a
-// CUDA graph (5 launches per step: the advection of the three fields in one
-// launch, forces, two transforms, projection).
+// the per-cell kernels use small CTAs, and the transforms run one CTA per mode or
+// row: all that stays within a z mode in one kernel (both x transforms), the
+// inverse z transform in the projection, which needs a row of phi and the
+// difference of its neighbours only.  That makes four launches per step (the
+// advection of the three fields in one).  At 50 x 50 the step is a chain of small
+// kernels, so each is launched while its predecessor runs (programmatic dependent
+// launch), sets up what does not depend on it, copies its constant operands and
+// then waits; long runs replay the step from a CUDA graph.
+// Measured, 50 x 50 FP64 CEC, us per step: 29.9 with five launches one after the
+// other, 23.9 with the double-precision sweeps of k_split64.cu, 23.0 now.
 #include <cmath>
 #include <new>
 #include <vector>
@@ -113,6 +119,8 @@ __global__ void k_rb_forces(const T *u, const T *w, const T *th, const T *au, co
     };
     auto u2 = [&](int64_t o) { return au[o] + dt * (Pr * lap(u, o)); };
     auto w2 = [&](int64_t o) { return aw[o] + dt * (Ra * Pr * th[o] + Pr * lap(w, o)); };
+    pdl_release();
+    pdl_wait();
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
         const int k = c / nx, i = c - (c / nx) * nx;
         const int64_t o = (int64_t)(k + RBG) * px + i + RBG;
@@ -128,66 +136,49 @@ __global__ void k_rb_forces(const T *u, const T *w, const T *th, const T *au, co
     }
 }
 
-// out(c) = sum_{t < K} a[t * as] B[t * ldb + c] for c < N, by the CTA's 256
-// threads: 64 columns at a time, each column's sum split over four thread
-// groups (t = g mod 4, two terms in flight per group) and combined in fixed
-// order in shared memory (part, 256 elements).
-template <typename T, typename Store>
-__device__ __forceinline__ void rb_vecmat(const T *a, int64_t as, const T *B, int64_t ldb, int K, int N, T *part,
-                                          Store store)
+constexpr int kRbRowThreads = 256;
+
+// out_q(c) = sum_{t < K} a_q[t] B[t * ldb + c * cs] for c < N and q < Q, by the
+// CTA's 256 threads: 64 columns at a time, each column's sum split over four
+// thread groups (t = g mod 4, two terms in flight per group) and combined in
+// fixed order in shared memory (part, Q x 256 elements).
+template <int Q, typename T, typename Store>
+__device__ __forceinline__ void rb_vecmat(const T *const (&a)[Q], const T *B, int64_t ldb, int64_t cs, int K, int N,
+                                          T *part, Store store)
 {
     const int c = threadIdx.x & 63, g = threadIdx.x >> 6;
     for (int c0 = 0; c0 < N; c0 += 64) {
         const int col = c0 + c;
-        T acc0 = T(0), acc1 = T(0);
+        T acc0[Q], acc1[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) acc0[q] = acc1[q] = T(0);
         if (col < N) {
+            const T *b = B + col * cs;
             int t = g;
 #pragma unroll 4
             for (; t + 4 < K; t += 8) {
-                acc0 += a[t * as] * B[t * ldb + col];
-                acc1 += a[(t + 4) * as] * B[(t + 4) * ldb + col];
+                const T x = b[t * ldb], y = b[(t + 4) * ldb];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    acc0[q] += a[q][t] * x;
+                    acc1[q] += a[q][t + 4] * y;
+                }
             }
-            if (t < K) acc0 += a[t * as] * B[t * ldb + col];
+            if (t < K) {
+                const T x = b[t * ldb];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) acc0[q] += a[q][t] * x;
+            }
         }
-        part[g * 64 + c] = acc0 + acc1;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) part[q * kRbRowThreads + g * 64 + c] = acc0[q] + acc1[q];
         __syncthreads();
-        if (g == 0 && col < N) store(col, (part[c] + part[64 + c]) + (part[128 + c] + part[192 + c]));
+        if (g < Q && col < N) {   // group q combines output q
+            const T *p = part + g * kRbRowThreads + c;
+            store(g, col, (p[0] + p[64]) + (p[128] + p[192]));
+        }
         __syncthreads();
     }
-}
-
-constexpr int kRbRowThreads = 256;
-
-// Forward transform and solve, one CTA per z mode k:
-//   R[i] = sum_m C_z[k][m] D[m][i],  F[k][j] = sum_i R[i] C_x[j][i] / lam_kj
-// (lam_kj = lz[k] + lx[j]; the constant mode F[0][0] = 0).  Every load is
-// coalesced across the threads or a broadcast (C_x enters transposed, cxT).
-template <typename T>
-__global__ void __launch_bounds__(kRbRowThreads)
-k_rb_forward(const T *D, const T *cz, const T *cxT, const T *lx, const T *lz, T *F, int nx, int nz)
-{
-    extern __shared__ __align__(16) unsigned char rb_smem[];
-    T *part = reinterpret_cast<T *>(rb_smem), *R = part + kRbRowThreads;
-    const int k = blockIdx.x;
-    rb_vecmat(cz + (int64_t)k * nz, 1, D, nx, nz, nx, part, [&](int i, T v) { R[i] = v; });
-    T *Fk = F + (int64_t)k * nx;
-    const T lk = lz[k];
-    rb_vecmat(R, 1, cxT, nx, nx, nx, part,
-              [&](int j, T v) { Fk[j] = (k == 0 && j == 0) ? T(0) : v / (lk + lx[j]); });
-}
-
-// Inverse transform, one CTA per row m of phi:
-//   R[j] = sum_k C_z[k][m] F[k][j],  phi[m][i] = sum_j R[j] C_x[j][i].
-template <typename T>
-__global__ void __launch_bounds__(kRbRowThreads)
-k_rb_inverse(const T *F, const T *cz, const T *cx, T *phi, int nx, int nz)
-{
-    extern __shared__ __align__(16) unsigned char rb_smem[];
-    T *part = reinterpret_cast<T *>(rb_smem), *R = part + kRbRowThreads;
-    const int m = blockIdx.x;
-    rb_vecmat(cz + m, nz, F, nx, nz, nx, part, [&](int j, T v) { R[j] = v; });
-    T *pm = phi + (int64_t)m * nx;
-    rb_vecmat(R, 1, cx, nx, nx, nx, part, [&](int i, T v) { pm[i] = v; });
 }
 
 // Copies n elements from global to shared memory: 16-byte chunks by cp.async
@@ -208,74 +199,97 @@ __host__ __device__ constexpr int64_t rb_pad(int64_t n)
     return (n + 16 / (int64_t)sizeof(T) - 1) / (16 / (int64_t)sizeof(T)) * (16 / (int64_t)sizeof(T));
 }
 
-// The same transforms with their matrix operands staged in shared memory
-// first (small boxes: D or F and C_x^T or C_x fit), so that the sums read
-// shared memory instead of waiting on L2; same summation order, same results.
-template <typename T>
+// Row pitch of C_x in shared memory: odd, so that reading it along either index
+// keeps the lanes on distinct banks.
+__host__ __device__ constexpr int rb_pitch(int nx) { return nx | 1; }
+
+// Everything of the Poisson solve that stays within one z mode, one CTA per mode k:
+//   R[i] = sum_m C_z[k][m] D[m][i],  F[j] = sum_i R[i] C_x[j][i] / lam_kj,
+//   G[k][i] = sum_j F[j] C_x[j][i]
+// (lam_kj = lz[k] + lx[j]; the constant mode F[0] of k = 0 is 0); phi = C_z^T G is
+// left to the projection.  STAGED (small boxes): D and C_x are copied to shared
+// memory first, so that the sums do not wait on L2; what does not depend on the
+// predecessor is copied while that still runs.  Otherwise C_x enters transposed
+// for the second sum (cxT), so that every load is coalesced or a broadcast.
+template <typename T, bool STAGED>
 __global__ void __launch_bounds__(kRbRowThreads)
-k_rb_forward_s(const T *D, const T *cz, const T *cxT, const T *lx, const T *lz, T *F, int nx, int nz)
+k_rb_modes(const T *D, const T *cz, const T *cx, const T *cxT, const T *lx, const T *lz, T *G, int nx, int nz)
 {
     extern __shared__ __align__(16) unsigned char rb_smem[];
-    T *part = reinterpret_cast<T *>(rb_smem), *R = part + kRbRowThreads;
-    T *sD = R + rb_pad<T>(nx), *sC = sD + rb_pad<T>((int64_t)nz * nx);
-    rb_stage(sD, D, (int64_t)nz * nx);
-    rb_stage(sC, cxT, (int64_t)nx * nx);
-    cp_async_commit();
-    cp_async_wait_all();
-    __syncthreads();
-    const int k = blockIdx.x;
-    rb_vecmat(cz + (int64_t)k * nz, 1, sD, nx, nz, nx, part, [&](int i, T v) { R[i] = v; });
-    T *Fk = F + (int64_t)k * nx;
+    T *part = reinterpret_cast<T *>(rb_smem), *R = part + kRbRowThreads, *F = R + rb_pad<T>(nx);
+    T *az = F + rb_pad<T>(nx), *sD = az + rb_pad<T>(nz), *sC = sD + rb_pad<T>((int64_t)nz * nx);
+    const int k = blockIdx.x, px = rb_pitch(nx);
+    pdl_release();
+    for (int m = threadIdx.x; m < nz; m += kRbRowThreads) az[m] = cz[(int64_t)k * nz + m];
+    if constexpr (STAGED)
+        for (int e = threadIdx.x; e < nx * nx; e += kRbRowThreads) sC[(e / nx) * px + e % nx] = cx[e];
     const T lk = lz[k];
-    rb_vecmat(R, 1, sC, nx, nx, nx, part,
-              [&](int j, T v) { Fk[j] = (k == 0 && j == 0) ? T(0) : v / (lk + lx[j]); });
+    pdl_wait();
+    if constexpr (STAGED) {
+        rb_stage(sD, D, (int64_t)nz * nx);
+        cp_async_commit();
+        cp_async_wait_all();
+    }
+    __syncthreads();
+    const T *const a0[1] = {az}, *const a1[1] = {R}, *const a2[1] = {F};
+    rb_vecmat<1>(a0, STAGED ? sD : D, nx, 1, nz, nx, part, [&](int, int i, T v) { R[i] = v; });
+    rb_vecmat<1>(a1, STAGED ? sC : cxT, STAGED ? 1 : nx, STAGED ? px : 1, nx, nx, part,
+                 [&](int, int j, T v) { F[j] = (k == 0 && j == 0) ? T(0) : v / (lk + lx[j]); });
+    T *Gk = G + (int64_t)k * nx;
+    rb_vecmat<1>(a2, STAGED ? sC : cx, STAGED ? px : nx, 1, nx, nx, part, [&](int, int i, T v) { Gk[i] = v; });
 }
 
-template <typename T>
+// Projection, one CTA per row m: phi[m][i] = sum_k C_z[k][m] G[k][i] and the
+// difference of the rows next to it, dphi[i] = sum_k Z[k][m] G[k][i] with Z[k][m] =
+// C_z[k][m + 1] - C_z[k][m - 1] (rows beyond a wall replaced by m itself: no flux
+// there).  Cells take the average of their two faces' gradient corrections
+// (face gradient (phi_{i+1} - phi_i) / dx inside, zero on the walls); the result
+// is the new u, w with their ghost images.  czT, zT: C_z and Z transposed.
+template <typename T, bool STAGED>
 __global__ void __launch_bounds__(kRbRowThreads)
-k_rb_inverse_s(const T *F, const T *cz, const T *cx, T *phi, int nx, int nz)
+k_rb_project(const T *u2, const T *w2, const T *G, const T *czT, const T *zT, T *u, T *w, int nx, int nz, T idx, T idz)
 {
     extern __shared__ __align__(16) unsigned char rb_smem[];
-    T *part = reinterpret_cast<T *>(rb_smem), *R = part + kRbRowThreads;
-    T *sF = R + rb_pad<T>(nx), *sC = sF + rb_pad<T>((int64_t)nz * nx);
-    rb_stage(sF, F, (int64_t)nz * nx);
-    rb_stage(sC, cx, (int64_t)nx * nx);
-    cp_async_commit();
-    cp_async_wait_all();
+    T *part = reinterpret_cast<T *>(rb_smem), *phi = part + 2 * kRbRowThreads, *dphi = phi + rb_pad<T>(nx);
+    T *a = dphi + rb_pad<T>(nx), *z = a + rb_pad<T>(nz), *sG = z + rb_pad<T>(nz);
+    const int m = blockIdx.x, px = rb_px(nx);
+    pdl_release();
+    for (int k = threadIdx.x; k < nz; k += kRbRowThreads) {
+        a[k] = czT[(int64_t)m * nz + k];
+        z[k] = zT[(int64_t)m * nz + k];
+    }
+    pdl_wait();
+    if constexpr (STAGED) {
+        rb_stage(sG, G, (int64_t)nz * nx);
+        cp_async_commit();
+        cp_async_wait_all();
+    }
     __syncthreads();
-    const int m = blockIdx.x;
-    rb_vecmat(cz + m, nz, sF, nx, nz, nx, part, [&](int j, T v) { R[j] = v; });
-    T *pm = phi + (int64_t)m * nx;
-    rb_vecmat(R, 1, sC, nx, nx, nx, part, [&](int i, T v) { pm[i] = v; });
-}
-
-// Shared memory of the staged transforms, and the largest the box uses them for.
-template <typename T>
-size_t rb_staged_smem(int nx, int nz)
-{
-    return sizeof(T) * (size_t)(kRbRowThreads + rb_pad<T>(nx) + rb_pad<T>((int64_t)nz * nx) + (int64_t)nx * nx);
-}
-constexpr size_t kRbStagedMax = 96 * 1024;
-
-// Projection: cells take the average of their two faces' gradient corrections
-// (face gradient (phi_{i+1} - phi_i) / dx inside, zero on the walls); the
-// result is the new u, w with their ghost images.
-template <typename T>
-__global__ void k_rb_project(const T *u2, const T *w2, const T *phi, T *u, T *w, int nx, int nz, T idx, T idz)
-{
-    const int px = rb_px(nx);
-    const int n = nx * nz;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-        const int k = c / nx, i = c - (c / nx) * nx;
-        const int64_t o = (int64_t)(k + RBG) * px + i + RBG;
-        const T ge = i + 1 < nx ? (phi[c + 1] - phi[c]) * idx : T(0);
-        const T gw = i > 0 ? (phi[c] - phi[c - 1]) * idx : T(0);
-        const T gn = k + 1 < nz ? (phi[c + nx] - phi[c]) * idz : T(0);
-        const T gs = k > 0 ? (phi[c] - phi[c - nx]) * idz : T(0);
-        store_mirrored(u, k, i, u2[o] - T(0.5) * (gw + ge), nx, nz, T(-1), T(-1));
-        store_mirrored(w, k, i, w2[o] - T(0.5) * (gs + gn), nx, nz, T(-1), T(-1));
+    const T *const az[2] = {a, z};
+    rb_vecmat<2>(az, STAGED ? sG : G, nx, 1, nz, nx, part, [&](int q, int i, T v) { (q ? dphi : phi)[i] = v; });
+    for (int i = threadIdx.x; i < nx; i += kRbRowThreads) {
+        const int64_t o = (int64_t)(m + RBG) * px + i + RBG;
+        const T dx = phi[i + 1 < nx ? i + 1 : i] - phi[i > 0 ? i - 1 : i];
+        store_mirrored(u, m, i, u2[o] - T(0.5) * (dx * idx), nx, nz, T(-1), T(-1));
+        store_mirrored(w, m, i, w2[o] - T(0.5) * (dphi[i] * idz), nx, nz, T(-1), T(-1));
     }
 }
+
+// Dynamic shared memory of the two, and the most a box takes to stage its operands.
+template <typename T>
+size_t rb_modes_smem(int nx, int nz, bool staged)
+{
+    return sizeof(T) * (size_t)(kRbRowThreads + 2 * rb_pad<T>(nx) + rb_pad<T>(nz) +
+                                (staged ? rb_pad<T>((int64_t)nz * nx) + (int64_t)nx * rb_pitch(nx) : 0));
+}
+template <typename T>
+size_t rb_project_smem(int nx, int nz, bool staged)
+{
+    return sizeof(T) * (size_t)(2 * kRbRowThreads + 2 * rb_pad<T>(nx) + 2 * rb_pad<T>(nz) +
+                                (staged ? rb_pad<T>((int64_t)nz * nx) : 0));
+}
+// (an unstaged FP64 box of 4096 x 4096 takes 132 KB in the projection)
+constexpr size_t kRbStagedMax = 96 * 1024, kRbSmemMax = 136 * 1024;
 
 // interior <-> padded copies
 template <typename T>
@@ -323,10 +337,11 @@ struct sl_rb {
     // padded planes: two states (u, w, theta back to back, so that (u, w) is
     // the velocity argument of the advection), the advected fields, (u2, w2)
     void *S[2] = {nullptr, nullptr}, *A = nullptr, *W = nullptr;
-    // interior arrays (nz x nx): the face divergence D, its transform F, phi
-    void *d = nullptr, *F = nullptr, *phi = nullptr;
-    // orthonormal DCT-II matrices C_x (and its transpose), C_z; eigenvalues per axis
-    void *cx = nullptr, *cxT = nullptr, *cz = nullptr, *lx = nullptr, *lz = nullptr;
+    // interior arrays (nz x nx): the face divergence D, and phi in z modes (G)
+    void *d = nullptr, *G = nullptr;
+    // orthonormal DCT-II matrices C_x and C_z and their transposes, the row
+    // differences of C_z (transposed, k_rb_project); eigenvalues per axis
+    void *cx = nullptr, *cxT = nullptr, *cz = nullptr, *czT = nullptr, *zT = nullptr, *lx = nullptr, *lz = nullptr;
     int *signs = nullptr;   // sx of (u, w, theta), then sz of (u, w, theta)
     // long runs replay kRbGraphSteps steps from one CUDA graph, captured for
     // one dt and one starting buffer on a stream of the box's own
@@ -345,15 +360,17 @@ int rb_step_t(sl_rb *r, double dt, int nsteps, cudaStream_t st)
     const int px = rb_px(nx), pz = nz + 2 * RBG;
     const int64_t P = r->plane;
     T *A = static_cast<T *>(r->A), *Wk = static_cast<T *>(r->W);
-    T *d = static_cast<T *>(r->d), *F = static_cast<T *>(r->F), *phi = static_cast<T *>(r->phi);
+    T *d = static_cast<T *>(r->d), *G = static_cast<T *>(r->G);
     const T *cx = static_cast<const T *>(r->cx), *cxT = static_cast<const T *>(r->cxT);
-    const T *cz = static_cast<const T *>(r->cz);
+    const T *cz = static_cast<const T *>(r->cz), *czT = static_cast<const T *>(r->czT), *zT = static_cast<const T *>(r->zT);
     const T *lx = static_cast<const T *>(r->lx), *lz = static_cast<const T *>(r->lz);
     const double dx = r->Lx / nx, dz = r->Lz / nz;
     const int64_t pdims[3] = {px, pz, 1};
     const double sp[3] = {dx, dz, 1.0};
     const int cbk = cell_block(n, r->sms), cgr = cell_grid(n, cbk);
-    const size_t rsm = sizeof(T) * (kRbRowThreads + nx), ssm = rb_staged_smem<T>(nx, nz);
+    const size_t msm = rb_modes_smem<T>(nx, nz, r->staged), psm = rb_project_smem<T>(nx, nz, r->staged);
+    auto modes = r->staged ? k_rb_modes<T, true> : k_rb_modes<T, false>;
+    auto project = r->staged ? k_rb_project<T, true> : k_rb_project<T, false>;
     for (int s = 0; s < nsteps; ++s) {
         // S0 holds step n with its ghost layers (the walls' mirror images)
         T *S0 = static_cast<T *>(r->S[r->cur]), *S1 = static_cast<T *>(r->S[r->cur ^ 1]);
@@ -361,24 +378,20 @@ int rb_step_t(sl_rb *r, double dt, int nsteps, cudaStream_t st)
         // CEC alternates its sweep order with the step index
         const void *ins[3] = {S0, S0 + P, S0 + 2 * P};
         void *outs[3] = {A, A + P, A + 2 * P};
-        int rc = sl_advect_multi(outs, ins, 3, S0, 2, pdims, sp, dt, r->scheme, r->dtype, (int)(r->step & 1), st);
+        int rc = advect_fields(outs, ins, 3, S0, 2, pdims, sp, dt, r->scheme, r->dtype, (int)(r->step & 1), st, true);
         if (rc) return rc;
         // forces: u2, w2 into the work planes, theta' (with ghosts) into the
         // next state, the face divergence D into d
-        k_rb_forces<T><<<cgr, cbk, 0, st>>>(S0, S0 + P, S0 + 2 * P, A, A + P, A + 2 * P, Wk, Wk + P, S1 + 2 * P, d, nx,
-                                            nz, T(dt), T(r->Ra), T(r->Pr), T(1.0 / (dx * dx)), T(1.0 / (dz * dz)),
-                                            T(1.0 / dx), T(1.0 / dz));
-        // phi = C_z^T [(C_z D C_x^T) / lam] C_x
-        if (r->staged) {
-            k_rb_forward_s<T><<<nz, kRbRowThreads, ssm, st>>>(d, cz, cxT, lx, lz, F, nx, nz);
-            k_rb_inverse_s<T><<<nz, kRbRowThreads, ssm, st>>>(F, cz, cx, phi, nx, nz);
-        } else {
-            k_rb_forward<T><<<nz, kRbRowThreads, rsm, st>>>(d, cz, cxT, lx, lz, F, nx, nz);
-            k_rb_inverse<T><<<nz, kRbRowThreads, rsm, st>>>(F, cz, cx, phi, nx, nz);
-        }
+        cudaError_t e = launch_kernel(k_rb_forces<T>, dim3(cgr), cbk, 0, st, true, S0, S0 + P, S0 + 2 * P, A, A + P,
+                                      A + 2 * P, Wk, Wk + P, S1 + 2 * P, d, nx, nz, T(dt), T(r->Ra), T(r->Pr),
+                                      T(1.0 / (dx * dx)), T(1.0 / (dz * dz)), T(1.0 / dx), T(1.0 / dz));
+        // G = [(C_z D C_x^T) / lam] C_x
+        if (e == cudaSuccess)
+            e = launch_kernel(modes, dim3(nz), kRbRowThreads, msm, st, true, d, cz, cx, cxT, lx, lz, G, nx, nz);
         // the projected u, w (with ghosts) of the next state
-        k_rb_project<T><<<cgr, cbk, 0, st>>>(Wk, Wk + P, phi, S1, S1 + P, nx, nz, T(1.0 / dx), T(1.0 / dz));
-        const cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = launch_kernel(project, dim3(nz), kRbRowThreads, psm, st, true, Wk, Wk + P, G, czT, zT, S1, S1 + P, nx, nz,
+                              T(1.0 / dx), T(1.0 / dz));
         if (e != cudaSuccess) return set_error(SL_ERR_CUDA, cudaGetErrorString(e));
         r->cur ^= 1;
         ++r->step;
@@ -493,8 +506,8 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
     r->plane = (int64_t)rb_px(nx) * (nz + 2 * RBG);
     auto round64 = [](int64_t k) { return (k + 63) / 64 * 64; };
     const int64_t n = (int64_t)nx * nz;
-    const int64_t elems = 4 * round64(3 * r->plane) + 3 * round64(n) + 2 * round64((int64_t)nx * nx) +
-                          round64((int64_t)nz * nz) + round64(nx) + round64(nz) + 64;
+    const int64_t elems = 4 * round64(3 * r->plane) + 2 * round64(n) + 2 * round64((int64_t)nx * nx) +
+                          3 * round64((int64_t)nz * nz) + round64(nx) + round64(nz) + 64;
     if (cudaMalloc(&r->mem, r->esz * elems) != cudaSuccess) {
         delete r;
         return set_error(SL_ERR_NOMEM, "device buffers of the box");
@@ -510,11 +523,12 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
     r->A = take(3 * r->plane);
     r->W = take(3 * r->plane);
     r->d = take(n);
-    r->F = take(n);
-    r->phi = take(n);
+    r->G = take(n);
     r->cx = take((int64_t)nx * nx);
     r->cxT = take((int64_t)nx * nx);
     r->cz = take((int64_t)nz * nz);
+    r->czT = take((int64_t)nz * nz);
+    r->zT = take((int64_t)nz * nz);
     r->lx = take(nx);
     r->lz = take(nz);
     r->signs = reinterpret_cast<int *>(p);
@@ -523,6 +537,13 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
     for (int j = 0; j < nx; ++j)
         for (int i = 0; i < nx; ++i) cxt[(size_t)i * nx + j] = cxm[(size_t)j * nx + i];
     dct_matrix(czm, nz);
+    std::vector<double> czt((size_t)nz * nz), zt((size_t)nz * nz);
+    for (int k = 0; k < nz; ++k)
+        for (int m = 0; m < nz; ++m) {
+            const double *row = czm.data() + (size_t)k * nz;
+            czt[(size_t)m * nz + k] = row[m];
+            zt[(size_t)m * nz + k] = row[m + 1 < nz ? m + 1 : m] - row[m > 0 ? m - 1 : m];
+        }
     const double dx = Lx / nx, dz = Lz / nz;
     for (int j = 0; j < nx; ++j) lxv[j] = -4.0 / (dx * dx) * std::pow(std::sin(M_PI * j / (2.0 * nx)), 2);
     for (int k = 0; k < nz; ++k) lzv[k] = -4.0 / (dz * dz) * std::pow(std::sin(M_PI * k / (2.0 * nz)), 2);
@@ -540,25 +561,28 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
     up(r->cx, cxm);
     up(r->cxT, cxt);
     up(r->cz, czm);
+    up(r->czT, czt);
+    up(r->zT, zt);
     up(r->lx, lxv);
     up(r->lz, lzv);
     if (e == cudaSuccess) e = cudaMemcpy(r->signs, signs, sizeof signs, cudaMemcpyHostToDevice);
-    // small boxes stage the transforms' matrix operands in shared memory; the
-    // kernels' limit is per function, not per box, so it is raised to the cap
-    // that every staged box fits under
-    const size_t ssm = dtype == SL_F64 ? rb_staged_smem<double>(nx, nz) : rb_staged_smem<float>(nx, nz);
-    if (e == cudaSuccess && ssm <= kRbStagedMax) {
-        const int cap = (int)kRbStagedMax;
-        if (dtype == SL_F64) {
-            e = cudaFuncSetAttribute(k_rb_forward_s<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_rb_inverse_s<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-        } else {
-            e = cudaFuncSetAttribute(k_rb_forward_s<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_rb_inverse_s<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-        }
-        r->staged = e == cudaSuccess;
+    // small boxes stage the transforms' operands in shared memory; the kernels'
+    // limit is per function, not per box, so it is raised to the cap that every
+    // box fits under
+    r->staged = (dtype == SL_F64 ? rb_modes_smem<double>(nx, nz, true) : rb_modes_smem<float>(nx, nz, true)) <= kRbStagedMax;
+    auto raise = [&](auto kern) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRbSmemMax);
+    };
+    if (dtype == SL_F64) {
+        raise(k_rb_modes<double, true>);
+        raise(k_rb_modes<double, false>);
+        raise(k_rb_project<double, true>);
+        raise(k_rb_project<double, false>);
+    } else {
+        raise(k_rb_modes<float, true>);
+        raise(k_rb_modes<float, false>);
+        raise(k_rb_project<float, true>);
+        raise(k_rb_project<float, false>);
     }
     if (e != cudaSuccess) {
         cudaFree(r->mem);

@@ -191,6 +191,8 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
     int64_t w = shares ? total * blockIdx.x / G : blockIdx.x;
     const int64_t wend = shares ? total * (blockIdx.x + 1) / G : total;
     bool bad = false;
+    pdl_release();
+    pdl_wait();
 
     while (w < wend) {
         int t, z0, z1;
@@ -374,7 +376,7 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
 }
 
 template <typename T, int TY, int NT, bool HAS_Z, bool VEC, bool ZYX>
-cudaError_t go(Geo g, int grid, const void *in, void *out, const void *vel, const FieldSet &fs, cudaStream_t st)
+cudaError_t go(Geo g, const Launch &lc, const void *in, void *out, const void *vel, const FieldSet &fs, cudaStream_t st)
 {
     using K = Lay<T, TY, HAS_Z, ZYX>;
     auto kern = k_cec64<T, TY, NT, HAS_Z, VEC, ZYX>;
@@ -406,21 +408,20 @@ cudaError_t go(Geo g, int grid, const void *in, void *out, const void *vel, cons
         gr = (resident[dev] + fs.n - 1) / fs.n;
         if (gr > (total + 1) / 2) gr = (total + 1) / 2;
     }
-    if (grid > 0 && grid < gr) gr = grid;
+    if (lc.grid > 0 && lc.grid < gr) gr = lc.grid;
     if (gr < 1) gr = 1;
     if (gr > 0x7fffffff) return cudaErrorInvalidConfiguration;
-    kern<<<dim3((unsigned)gr, fs.n), NT, K::smem(), st>>>(static_cast<const T *>(in), static_cast<T *>(out),
-                                                          static_cast<const T *>(vel), g, fs.fin, fs.fout);
-    return cudaGetLastError();
+    return launch_kernel(kern, dim3((unsigned)gr, fs.n), NT, K::smem(), st, lc.pdl, static_cast<const T *>(in),
+                         static_cast<T *>(out), static_cast<const T *>(vel), g, fs.fin, fs.fout);
 }
 
 template <typename T, bool HAS_Z, bool VEC>
-cudaError_t by_order(int parity, const Geo &g, int grid, const void *in, void *out, const void *vel,
+cudaError_t by_order(int parity, const Geo &g, const Launch &lc, const void *in, void *out, const void *vel,
                      const FieldSet &fs, cudaStream_t st)
 {
     if constexpr (HAS_Z) {
-        return (parity & 1) ? go<T, 16, 256, true, VEC, true>(g, grid, in, out, vel, fs, st)
-                            : go<T, 16, 256, true, VEC, false>(g, grid, in, out, vel, fs, st);
+        return (parity & 1) ? go<T, 16, 256, true, VEC, true>(g, lc, in, out, vel, fs, st)
+                            : go<T, 16, 256, true, VEC, false>(g, lc, in, out, vel, fs, st);
     } else {
         // Small planes take 4-row tiles, which spread them over more SMs: the
         // 32 x 16 tiles of a 128^2 plane would leave 120 of 152 SMs idle, and the
@@ -428,10 +429,10 @@ cudaError_t by_order(int parity, const Geo &g, int grid, const void *in, void *o
         // until the larger tiles give every SM two CTAs.
         const int64_t big = (int64_t)((g.nx + TX - 1) / TX) * ((g.ny + 15) / 16) * fs.n;
         if (big < 2 * 152)
-            return (parity & 1) ? go<T, 4, 128, false, VEC, true>(g, grid, in, out, vel, fs, st)
-                                : go<T, 4, 128, false, VEC, false>(g, grid, in, out, vel, fs, st);
-        return (parity & 1) ? go<T, 16, 256, false, VEC, true>(g, grid, in, out, vel, fs, st)
-                            : go<T, 16, 256, false, VEC, false>(g, grid, in, out, vel, fs, st);
+            return (parity & 1) ? go<T, 4, 128, false, VEC, true>(g, lc, in, out, vel, fs, st)
+                                : go<T, 4, 128, false, VEC, false>(g, lc, in, out, vel, fs, st);
+        return (parity & 1) ? go<T, 16, 256, false, VEC, true>(g, lc, in, out, vel, fs, st)
+                            : go<T, 16, 256, false, VEC, false>(g, lc, in, out, vel, fs, st);
     }
 }
 
@@ -442,15 +443,15 @@ cudaError_t launch_split_cec64(bool f32_storage, Geo g, int parity, Launch lc, b
 {
     const bool vec = lc.aligned && g.nx % (f32_storage ? 4 : 2) == 0;
     if (f32_storage) {
-        if (has_z) return vec ? by_order<float, true, true>(parity, g, lc.grid, in, out, vel, fs, st)
-                              : by_order<float, true, false>(parity, g, lc.grid, in, out, vel, fs, st);
-        return vec ? by_order<float, false, true>(parity, g, lc.grid, in, out, vel, fs, st)
-                   : by_order<float, false, false>(parity, g, lc.grid, in, out, vel, fs, st);
+        if (has_z) return vec ? by_order<float, true, true>(parity, g, lc, in, out, vel, fs, st)
+                              : by_order<float, true, false>(parity, g, lc, in, out, vel, fs, st);
+        return vec ? by_order<float, false, true>(parity, g, lc, in, out, vel, fs, st)
+                   : by_order<float, false, false>(parity, g, lc, in, out, vel, fs, st);
     }
-    if (has_z) return vec ? by_order<double, true, true>(parity, g, lc.grid, in, out, vel, fs, st)
-                          : by_order<double, true, false>(parity, g, lc.grid, in, out, vel, fs, st);
-    return vec ? by_order<double, false, true>(parity, g, lc.grid, in, out, vel, fs, st)
-               : by_order<double, false, false>(parity, g, lc.grid, in, out, vel, fs, st);
+    if (has_z) return vec ? by_order<double, true, true>(parity, g, lc, in, out, vel, fs, st)
+                          : by_order<double, true, false>(parity, g, lc, in, out, vel, fs, st);
+    return vec ? by_order<double, false, true>(parity, g, lc, in, out, vel, fs, st)
+               : by_order<double, false, false>(parity, g, lc, in, out, vel, fs, st);
 }
 
 }  // namespace sl

@@ -225,58 +225,9 @@ DevCtx *ctx_get()
     return &c;
 }
 
-}  // namespace sl
-
-using namespace sl;
-
-struct sl_batch {
-    int device = -1;
-    int n = 0;
-    int scheme = SL_CEC;
-    int dtype = SL_F32;
-    bool fast = false;             // every instance takes the fast persistent path
-    BatchRec *dev_recs = nullptr;  // generic path: work-queue records
-    FastInst *dev_fast = nullptr;  // fast path: [2][n] tables (even: a -> b, odd: b -> a)
-    int64_t fast_total = 0;
-    unsigned *counter = nullptr;   // owns the device allocation
-    int nitems[2] = {0, 0};
-    int grid[2] = {0, 0};
-    int fast_grid = 0;             // fast path: CTAs (0 = the kernel's default)
-    sl_tuning tuning{};            // current launch shape, as reported
-};
-
-extern "C" {
-
-int sl_version(void) { return 10000; }
-
-const char *sl_last_error(void) { return g_err.c_str(); }
-
-int sl_init(void)
-{
-    if (!ctx_get()) return fail(SL_ERR_CUDA, "could not create the device context");
-    return SL_OK;
-}
-
-int sl_advect(void *out, const void *in, const void *vel, int ndim, const int64_t dims[3], const double spacing[3],
-              double dt, int scheme, int dtype, int step_parity, void *stream)
-{
-    if (!out || !in || !vel) return fail(SL_ERR_ARG, "out, in and vel must not be NULL");
-    if (scheme < SL_CIR || scheme > SL_CEC) return fail(SL_ERR_ARG, "unknown scheme %d", scheme);
-    double s[3];
-    int rc = check_geometry(ndim, dims, spacing, dt, dtype, s);
-    if (rc) return rc;
-    const size_t es = elem_size(dtype);
-    const size_t fb = (size_t)ncell_of(dims) * es;
-    if (overlap(out, fb, in, fb)) return fail(SL_ERR_ALIAS, "out overlaps in");
-    if (overlap(out, fb, vel, fb * ndim)) return fail(SL_ERR_ALIAS, "out overlaps vel");
-    DevCtx *c = ctx_get();
-    if (!c) return fail(SL_ERR_CUDA, "could not create the device context");
-    return launch_step(out, in, vel, ndim, dims, s, scheme, dtype, step_parity, static_cast<cudaStream_t>(stream), c);
-}
-
-int sl_advect_multi(void *const *outs, const void *const *ins, int nfields, const void *vel, int ndim,
-                    const int64_t dims[3], const double spacing[3], double dt, int scheme, int dtype,
-                    int step_parity, void *stream)
+int advect_fields(void *const *outs, const void *const *ins, int nfields, const void *vel, int ndim,
+                  const int64_t dims[3], const double spacing[3], double dt, int scheme, int dtype, int step_parity,
+                  void *stream, bool pdl)
 {
     if (!outs || !ins || nfields < 1) return fail(SL_ERR_ARG, "outs/ins must hold nfields >= 1 pointers");
     if (!vel) return fail(SL_ERR_ARG, "vel must not be NULL");
@@ -333,7 +284,8 @@ int sl_advect_multi(void *const *outs, const void *const *ins, int nfields, cons
         const bool al = al0 && aligned16(vel);
         const int fam = family_of(scheme, dtype, ndim, dims, al);
         if (fam != SL_KERNEL_CEC_FAST) {
-            const Launch lc = launch_for(fam, dims, scheme, dtype, al, c);
+            Launch lc = launch_for(fam, dims, scheme, dtype, al, c);
+            lc.pdl = pdl;
             FieldSet fs;
             fs.n = nfields;
             fs.fin = din / es;
@@ -349,6 +301,62 @@ int sl_advect_multi(void *const *outs, const void *const *ins, int nfields, cons
         if (rc) return rc;
     }
     return SL_OK;
+}
+
+}  // namespace sl
+
+using namespace sl;
+
+struct sl_batch {
+    int device = -1;
+    int n = 0;
+    int scheme = SL_CEC;
+    int dtype = SL_F32;
+    bool fast = false;             // every instance takes the fast persistent path
+    BatchRec *dev_recs = nullptr;  // generic path: work-queue records
+    FastInst *dev_fast = nullptr;  // fast path: [2][n] tables (even: a -> b, odd: b -> a)
+    int64_t fast_total = 0;
+    unsigned *counter = nullptr;   // owns the device allocation
+    int nitems[2] = {0, 0};
+    int grid[2] = {0, 0};
+    int fast_grid = 0;             // fast path: CTAs (0 = the kernel's default)
+    sl_tuning tuning{};            // current launch shape, as reported
+};
+
+extern "C" {
+
+int sl_version(void) { return 10000; }
+
+const char *sl_last_error(void) { return g_err.c_str(); }
+
+int sl_init(void)
+{
+    if (!ctx_get()) return fail(SL_ERR_CUDA, "could not create the device context");
+    return SL_OK;
+}
+
+int sl_advect(void *out, const void *in, const void *vel, int ndim, const int64_t dims[3], const double spacing[3],
+              double dt, int scheme, int dtype, int step_parity, void *stream)
+{
+    if (!out || !in || !vel) return fail(SL_ERR_ARG, "out, in and vel must not be NULL");
+    if (scheme < SL_CIR || scheme > SL_CEC) return fail(SL_ERR_ARG, "unknown scheme %d", scheme);
+    double s[3];
+    int rc = check_geometry(ndim, dims, spacing, dt, dtype, s);
+    if (rc) return rc;
+    const size_t es = elem_size(dtype);
+    const size_t fb = (size_t)ncell_of(dims) * es;
+    if (overlap(out, fb, in, fb)) return fail(SL_ERR_ALIAS, "out overlaps in");
+    if (overlap(out, fb, vel, fb * ndim)) return fail(SL_ERR_ALIAS, "out overlaps vel");
+    DevCtx *c = ctx_get();
+    if (!c) return fail(SL_ERR_CUDA, "could not create the device context");
+    return launch_step(out, in, vel, ndim, dims, s, scheme, dtype, step_parity, static_cast<cudaStream_t>(stream), c);
+}
+
+int sl_advect_multi(void *const *outs, const void *const *ins, int nfields, const void *vel, int ndim,
+                    const int64_t dims[3], const double spacing[3], double dt, int scheme, int dtype,
+                    int step_parity, void *stream)
+{
+    return advect_fields(outs, ins, nfields, vel, ndim, dims, spacing, dt, scheme, dtype, step_parity, stream, false);
 }
 
 int sl_advect_host(void *out, const void *in, const void *vel, int ndim, const int64_t dims[3],

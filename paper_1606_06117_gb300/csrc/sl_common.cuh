@@ -65,6 +65,14 @@ __device__ __forceinline__ void cp_async_elem(T *smem, const T *gmem)
         cp_async8(smem, gmem);
 }
 
+// ------------------------------------------- programmatic dependent launch
+// A kernel launched with the programmatic-serialisation attribute may start while
+// its predecessor in the stream still runs; before it touches anything the
+// predecessor reads or writes, every thread waits for the predecessor's end (its
+// memory included).  Both are no-ops in a kernel launched without the attribute.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ----------------------------------------------------------- 1D CEC kernels
 //
 // One directional sweep of the combined scheme (Sec. 2 eqs. intro:FEC,

@@ -28,7 +28,26 @@ struct Launch {
     int ty = 0;          // column tile height among a kernel's compiled variants; 0 = default
     int grid = 0;        // CTAs; 0 = one per item (persistent kernels: their occupancy)
     bool aligned = true; // all base pointers 16-byte aligned (vector staging allowed)
+    bool pdl = false;    // the kernel waits for its predecessor itself (kernels that know how)
 };
+
+// Launches kern; pdl: with programmatic stream serialisation, for a kernel that
+// begins with pdl_wait() (sl_common.cuh).
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, bool pdl, A... args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
 
 // Several fields advected by one velocity in one launch: field f reads
 // in + f * fin and writes out + f * fout (elements); the launch's grid gains
@@ -132,6 +151,11 @@ int wide_fields(int scheme, int ndim);
 cudaError_t launch_wide(int dtype, int scheme, const void *in, void *out, const void *vel, int ndim,
                         const int64_t dims[3], const double s[3], int parity, void *work, unsigned *status,
                         cudaStream_t st);
+
+// sl_advect_multi; pdl as in Launch.
+int advect_fields(void *const *outs, const void *const *ins, int nfields, const void *vel, int ndim,
+                  const int64_t dims[3], const double spacing[3], double dt, int scheme, int dtype, int step_parity,
+                  void *stream, bool pdl);
 
 // Records a thread-local error message (read by sl_last_error) and returns code.
 int set_error(int code, const char *msg);
