@@ -1,7 +1,13 @@
-// k_cec_fast.cu -- the fused split third-order step (SL_CEC, FP32) for grids
-// of whole 32 x 32 column tiles (nx, ny multiples of 32, nx >= 64, nz >= 8,
-// 16-byte aligned buffers): one persistent launch per step, one HBM read of
-// Phi and u and one write of the result per cell.
+// k_cec_fast.cu -- the fused split third-order step (SL_CEC, FP32): one
+// persistent launch per step, one HBM read of Phi and u and one write of the
+// result per cell.  Grids of whole 32 x 32 column tiles (nx, ny multiples of 32,
+// nx >= 64, nz >= 8, 16-byte aligned buffers) are staged by the tensor-memory
+// accelerator; all other 3D grids of 8 planes or more by per-thread copies from a
+// table of wrapped offsets (CH below), with the same sweeps and the same bits.
+// Measured (us per step, x,y,z / z,y,x; the generic kernel of k_split.cu before):
+// 187 x 150 x 131 55 / 79 -> 49 / 58, 188 x 150 x 131 46 / 70 -> 40 / 44,
+// 300^3 234 / 359 -> 192 / 235, 301 x 300 x 300 280 / 382 -> 226 / 333,
+// 65 x 40 x 30 31 / 29 -> 17 / 17.
 //
 // Mathematics (Sec. 2 eqs. intro:FEC, intro:BEC, intro:CEC, intro:CECcoef; one
 // 1D sweep per axis as in Sec. 2 last paragraph and Sec. 5 eqs. split:1-2).
@@ -46,6 +52,7 @@
 // Only the window push is compiled once per window parity; the rest of the
 // plane loop exists once (instruction-cache pressure measured on z,y,x).
 #include <cuda.h>
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -438,9 +445,9 @@ __device__ __forceinline__ int wrapz(int p, int nz) { return ((p % nz) + nz) % n
 constexpr unsigned kPolls = 1u << 20;   // bound of every mbarrier wait
 constexpr int PW = 44;                  // staged row stride (floats)
 
-__device__ __forceinline__ void bar_init(uint64_t *b)
+__device__ __forceinline__ void bar_init(uint64_t *b, unsigned arrivals)
 {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(b)) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(b)), "r"(arrivals) : "memory");
 }
 
 // the one arrival of a slot's phase, announcing the bytes its copies deliver
@@ -489,6 +496,11 @@ struct FastMaps {
     CUtensorMap fx[kFastFields - 1][NFMAPS];       // fields 1 .. nf-1
 };
 static_assert(sizeof(FastMaps) == kFastMapsBytes, "tensor map block size");
+struct NoMaps {
+    int unused;
+};
+template <int CH>
+using MapsOf = std::conditional_t<CH == 0, FastMaps, NoMaps>;   // copies need no maps
 
 // Row bands of one staged array of rows [-8, 32 + nb) (nb = 2 or 3): wide
 // boxes at x0 - 4 into dst, and at the seam the 4-wide side boxes at xs into
@@ -507,6 +519,40 @@ __device__ __forceinline__ void stage_rows(float *dst, float *side, const CUtens
         tma3(side, &m[b.s8], xs, yt, z, bar);
         tma3(side + 32, &m[b.s32], xs, y0, z, bar);
         tma3(side + 160, &m[b.sb], xs, yb, z, bar);
+    }
+}
+
+// Staging of grids of any size and alignment (CH = 4 floats per copy where rows
+// are whole 16-byte chunks, else 1): every thread copies its share of a plane with
+// cp.async, from a table of in-plane offsets in shared memory (rows [-3, TY+3) of
+// the tile, columns from -4 on, periodic wrap included) that is built once per
+// column tile, and the slot's mbarrier counts the threads' completions.  The
+// slots hold the same rows and columns as with the tensor-memory accelerator,
+// except that the wrapped columns are in place, so that the sweeps need no side
+// buffers; ragged tiles work on wrapped cells and do not store them.
+template <int CH>
+__device__ __forceinline__ void copy_chunk(float *dst, const float *src)
+{
+    if constexpr (CH == 4)
+        cp_async16(dst, src);
+    else
+        cp_async4(dst, src);
+}
+
+// the arrival of this thread's copies so far on a slot's mbarrier
+__device__ __forceinline__ void bar_arrive_copies(uint64_t *b)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_u32(b)) : "memory");
+}
+
+// offsets of LW / CH chunks in each of the 38 rows
+template <int CH, int LW>
+__device__ __forceinline__ void build_table(int *tab, int tid, int x0, int y0, int nx, int ny)
+{
+    constexpr int CPR = LW / CH;
+    for (int i = tid; i < 38 * CPR; i += NT) {
+        const int r = i / CPR, c = i - (i / CPR) * CPR;
+        tab[i] = wrapi(y0 - 3 + r, ny) * nx + wrapi(x0 - 4 + c * CH, nx);
     }
 }
 
@@ -582,8 +628,9 @@ static_assert(43 * PW <= 1920 && 43 * 4 <= 192 && SLOT % 32 == 0, "slot layout")
 constexpr int XW = 36;                                // x-swept row stride (bank-conflict-free stores)
 constexpr int SZ_X = (TY + 6) * XW;                   // one x-swept plane, rows [-3, TY+3)
 constexpr unsigned BYTES = 4u * (2 * 43 * PW + (TY + 4) * TX + TY * TX), BYTES_SEAM = 4u * 2 * 43 * 4;
-template <int NS>
-constexpr size_t smem() { return sizeof(float) * (NS * SLOT + 2 * SZ_X) + 128; }
+constexpr int tab_size(int ch) { return ch ? 38 * PW / ch : 0; }   // copied rows: whole shared rows
+template <int NS, int CH>
+constexpr size_t smem() { return sizeof(float) * (NS * SLOT + 2 * SZ_X + tab_size(CH)) + 128; }
 }  // namespace xyz
 
 // Stages the bundle of plane pz (reduced modulo nz) for the x,y,z order into
@@ -607,6 +654,38 @@ __device__ __forceinline__ void xyz_issue(float *sb, uint64_t *b, const CUtensor
     tma3(sb + O_UZ, &m[M_V32_32], x0, y0, 2 * nz + pz1, b);
 }
 
+// The same bundle by copies of CH floats (all threads): Phi and u_x rows
+// [-3, TY+3) in whole shared rows, u_y rows [-2, TY+2) and u_z rows [0, TY) of the
+// tile's columns.  in, vel: the planes' bases; at, at1: plane offsets of pz, pz - 1.
+template <int CH>
+__device__ __forceinline__ void xyz_copy(float *sb, uint64_t *b, const int *tab, int tid, const float *in,
+                                         const float *vel, int64_t ncell, int64_t at, int64_t at1)
+{
+    using namespace xyz;
+    constexpr int CPR = PW / CH, N = 38 * CPR, C2 = TX / CH;
+    const float *ph = in + at, *ux = vel + at, *uy = vel + ncell + at, *uz = vel + 2 * ncell + at1;
+#pragma unroll
+    for (int k = 0; k < (N + NT - 1) / NT; ++k) {
+        const int i = tid + k * NT;
+        if (i < N) {
+            const int o = tab[i];
+            copy_chunk<CH>(sb + O_PHI + 5 * PW + CH * i, ph + o);
+            copy_chunk<CH>(sb + O_UX + 5 * PW + CH * i, ux + o);
+        }
+    }
+    // chunk i of a row block of the tile's columns: row i / C2, chunk i mod C2
+    const int t0 = (tid / C2) * CPR + tid % C2 + 4 / CH;
+#pragma unroll
+    for (int k = 0; k < ((TY + 4) * C2 + NT - 1) / NT; ++k) {
+        const int i = tid + k * NT;
+        if (i < (TY + 4) * C2) copy_chunk<CH>(sb + O_UY + CH * i, uy + tab[t0 + (k * (NT / C2) + 1) * CPR]);
+    }
+#pragma unroll
+    for (int k = 0; k < TY * C2 / NT; ++k)
+        copy_chunk<CH>(sb + O_UZ + CH * (tid + k * NT), uz + tab[t0 + (k * (NT / C2) + 3) * CPR]);
+    bar_arrive_copies(b);
+}
+
 #ifndef SL_XYZ_MINB
 #define SL_XYZ_MINB 2      // CTAs per SM the x,y,z kernel is compiled for
 #endif
@@ -624,14 +703,15 @@ __device__ __forceinline__ float *smem_base()
     return base + (((128u - (smem_u32(base) & 127u)) & 127u) >> 2);
 }
 
-template <bool BATCH, int NS>
+template <bool BATCH, int NS, int CH>
 __global__ void __launch_bounds__(NT, SL_XYZ_MINB)
-k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ FastMaps one_maps,
+k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ MapsOf<CH> one_maps,
                const FastInst *__restrict__ table, int ninst, int64_t total, unsigned *status)
 {
     using namespace xyz;
     float *const buf = smem_base();
     float *const sX = buf + NS * SLOT;                // two x-swept planes
+    int *const offs = reinterpret_cast<int *>(sX + 2 * SZ_X);   // CH: the tile's copy offsets
 
     const int tid = threadIdx.x;
     const FastInst *tab = BATCH ? table : &one;
@@ -655,7 +735,7 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
     constexpr int ISSUER = NT - 1;                    // idle in the x phase
     __shared__ uint64_t bars[NS];
     if (tid == 0) {
-        for (int k = 0; k < NS; ++k) bar_init(&bars[k]);
+        for (int k = 0; k < NS; ++k) bar_init(&bars[k], CH ? NT : 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     __syncthreads();
@@ -670,25 +750,36 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
 
     while (next_seg(tab, ninst, w, wend, hint, (double)total / (double)G, sg)) {
         const FastInst &I = tab[sg.inst];
-        const CUtensorMap *maps = BATCH ? static_cast<const FastMaps *>(I.maps)->m : one_maps.m;
-        const CUtensorMap *fmaps = fld == 0 ? maps : one_maps.fx[fld - 1];
+        const CUtensorMap *maps = nullptr, *fmaps = nullptr;
+        if constexpr (CH == 0) {
+            maps = BATCH ? static_cast<const FastMaps *>(I.maps)->m : one_maps.m;
+            fmaps = fld == 0 ? maps : one_maps.fx[fld - 1];
+        }
         const int x0 = sg.tx * TX, y0 = sg.ty * TY, nz = I.nz;
         const int64_t plane_n = I.plane;
         const float msx = -I.sx, msy = -I.sy, msz = -I.sz;
         const int pfirst = sg.z0 - 3, plast = sg.z1 + 2;
-        const bool sl = x0 == 0, sr = x0 + TX == I.nx, seam = sl || sr;
+        const bool sl = CH == 0 && x0 == 0, sr = CH == 0 && x0 + TX == I.nx, seam = sl || sr;
         Blocks bp, bu;
         bp.set(O_PHI + (xrow + 5) * PW, O_SP + 4 * (xrow + 5), xr, sl, sr);
         bu.set(O_UX + (xrow + 5) * PW, O_SX + 4 * (xrow + 5), xr, sl, sr);
         float *const obase = (BATCH ? I.out : I.fout[fld]) + (int64_t)(y0 + yr) * I.nx + x0 + 2 * cp;
         const int onx = I.nx;
         auto issue = [&](int pz, int s) {
-            if (tid == ISSUER && !tmo) {
+            if constexpr (CH) {
+                if (!tmo)
+                    xyz_copy<CH>(buf + s * SLOT, &bars[s], offs, tid, I.fin[fld], I.vel, I.ncell, pz * plane_n,
+                                 (pz == 0 ? nz - 1 : pz - 1) * plane_n);
+            } else if (tid == ISSUER && !tmo) {
                 xyz_issue(buf + s * SLOT, &bars[s], fmaps, maps, x0, y0, I.nx, I.ny, nz, pz, seam);
                 armed |= 1u << s;
             }
         };
 
+        if constexpr (CH) {
+            build_table<CH, PW>(offs, tid, x0, y0, I.nx, I.ny);
+            __syncthreads();
+        }
         ZWin<L2> win[2];
         win[0].init();
         win[1].init();
@@ -783,8 +874,18 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
             if (p - 3 >= sg.z0) {
                 const int kw = zp >= 3 ? zp - 3 : zp - 3 + nz;
                 float *dst = obase + (int64_t)kw * plane_n;
-                *reinterpret_cast<float2 *>(dst) = res[0];
-                *reinterpret_cast<float2 *>(dst + onx) = res[1];
+                if constexpr (CH == 1) {
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+                        if (y0 + yr + i < I.ny) {
+                            if (x0 + 2 * cp < onx) dst[i * onx] = res[i].x;
+                            if (x0 + 2 * cp + 1 < onx) dst[i * onx + 1] = res[i].y;
+                        }
+                } else {
+                    const bool in_x = CH == 0 || x0 + 2 * cp < onx;
+                    if (in_x && (CH == 0 || y0 + yr < I.ny)) *reinterpret_cast<float2 *>(dst) = res[0];
+                    if (in_x && (CH == 0 || y0 + yr + 1 < I.ny)) *reinterpret_cast<float2 *>(dst + onx) = res[1];
+                }
             }
         };
 
@@ -794,7 +895,10 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
         }
         __syncthreads();   // shared buffers are reused by the next segment
     }
-    if (tid == ISSUER && armed) drain<NS>(bars, armed, par);
+    if constexpr (CH)
+        cp_async_wait_all();
+    else if (tid == ISSUER && armed)
+        drain<NS>(bars, armed, par);
     if (tmo) atomicOr(status, 2u);
     flag_cfl(status, bad);
 }
@@ -818,8 +922,9 @@ static_assert(39 * ZS <= O_SP && O_SP + 192 <= DZ && O_SZ + 192 <= O_UY && O_UY 
 constexpr int SZ_Z = (TY + 6) * ZS;                   // one z-swept plane, rows [-3, TY+3)
 constexpr int SZ_Y = TY * ZS;                         // y-swept rows [0, TY)
 constexpr unsigned BYTES = 4u * (39 + 39 + 38 + 32) * ZS, BYTES_SEAM = 4u * 4 * (43 + 43 + 42 + 32);
-template <int NS>
-constexpr size_t smem() { return sizeof(float) * (NS * SLOT + 2 * SZ_Z + SZ_Y) + 128; }
+constexpr int tab_size(int ch) { return ch ? 38 * ZS / ch : 0; }
+template <int NS, int CH>
+constexpr size_t smem() { return sizeof(float) * (NS * SLOT + 2 * SZ_Z + SZ_Y + tab_size(CH)) + 128; }
 }  // namespace zyx
 
 // Row zr in [0, 38) and pair column zc in [0, 20) of z-window pair q: the
@@ -877,6 +982,30 @@ __device__ __forceinline__ void zyx_issue(float *sb, uint64_t *b, const CUtensor
     if (seam) tma3(sb + O_SX + 32, &m[M_V4_32], xs, y0, pz3, b);
 }
 
+// The same bundle by copies of CH floats (all threads): Phi and u_z rows
+// [-3, TY+3), u_y rows [-2, TY+2), u_x rows [0, TY), each of whole shared rows.
+// at, at1, at3: plane offsets of pz, pz - 1, pz - 3.
+template <int CH>
+__device__ __forceinline__ void zyx_copy(float *sb, uint64_t *b, const int *tab, int tid, const float *in,
+                                         const float *vel, int64_t ncell, int64_t at, int64_t at1, int64_t at3)
+{
+    using namespace zyx;
+    constexpr int CPR = ZS / CH;
+    auto rows = [&](auto nr, int r0, float *dst, const float *src) {   // rows [r0, r0 + nr), counted from -3
+        constexpr int N = decltype(nr)::value * CPR;
+#pragma unroll
+        for (int k = 0; k < (N + NT - 1) / NT; ++k) {
+            const int i = tid + k * NT;
+            if (i < N) copy_chunk<CH>(dst + CH * i, src + tab[r0 * CPR + i]);
+        }
+    };
+    rows(std::integral_constant<int, 38>{}, 0, sb + O_PHI + ZS, in + at);
+    rows(std::integral_constant<int, 38>{}, 0, sb + O_UZ + ZS, vel + 2 * ncell + at1);
+    rows(std::integral_constant<int, 36>{}, 1, sb + O_UY + 2 * ZS, vel + ncell + at3);
+    rows(std::integral_constant<int, 32>{}, 3, sb + O_UX, vel + at3);
+    bar_arrive_copies(b);
+}
+
 // The 3 blocks [xr - 4, xr + 8) of a row for an x-run of 4 (offsets from the
 // array base; the first / last block from the side buffer at the seam).
 struct Blocks3 {
@@ -921,15 +1050,16 @@ __device__ __forceinline__ void x_run4(const float *pbase, const Blocks3 &pb, co
     run_cls<L1, R>(cls, p, m, o);
 }
 
-template <bool BATCH, int NS>
+template <bool BATCH, int NS, int CH>
 __global__ void __launch_bounds__(NT, SL_ZYX_MINB)
-k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ FastMaps one_maps,
+k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ MapsOf<CH> one_maps,
                const FastInst *__restrict__ table, int ninst, int64_t total, unsigned *status)
 {
     using namespace zyx;
     float *const buf = smem_base();
     float *const sZ = buf + NS * SLOT;                // two z-swept planes
     float *const sY = sZ + 2 * SZ_Z;                  // y-swept plane (each warp its own 4 rows)
+    int *const offs = reinterpret_cast<int *>(sY + SZ_Y);   // CH: the tile's copy offsets
 
     const int tid = threadIdx.x, lane = tid & 31, wq = tid >> 5;
     const FastInst *tab = BATCH ? table : &one;
@@ -944,7 +1074,7 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
     constexpr int ISSUER = NT - 1;                    // idle in the y phase
     __shared__ uint64_t bars[NS];
     if (tid == 0) {
-        for (int k = 0; k < NS; ++k) bar_init(&bars[k]);
+        for (int k = 0; k < NS; ++k) bar_init(&bars[k], CH ? NT : 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     __syncthreads();
@@ -971,16 +1101,23 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
 
     while (next_seg(tab, ninst, w, wend, hint, (double)total / (double)G, sg)) {
         const FastInst &I = tab[sg.inst];
-        const CUtensorMap *maps = BATCH ? static_cast<const FastMaps *>(I.maps)->m : one_maps.m;
-        const CUtensorMap *fmaps = fld == 0 ? maps : one_maps.fx[fld - 1];
+        const CUtensorMap *maps = nullptr, *fmaps = nullptr;
+        if constexpr (CH == 0) {
+            maps = BATCH ? static_cast<const FastMaps *>(I.maps)->m : one_maps.m;
+            fmaps = fld == 0 ? maps : one_maps.fx[fld - 1];
+        }
         const int x0 = sg.tx * TX, y0 = sg.ty * TY, nz = I.nz;
         const int64_t plane_n = I.plane;
         const float msx = -I.sx, msy = -I.sy, msz = -I.sz;
         const int pfirst = sg.z0 - 3, plast = sg.z1 + 2;
-        const bool sl = x0 == 0, sr = x0 + TX == I.nx, seam = sl || sr;
+        const bool sl = CH == 0 && x0 == 0, sr = CH == 0 && x0 + TX == I.nx, seam = sl || sr;
         const int edge = (sl ? 1 : 0) | (sr ? 2 : 0);
         auto issue = [&](int pz, int s) {
-            if (tid == ISSUER && !tmo) {
+            if constexpr (CH) {
+                if (!tmo)
+                    zyx_copy<CH>(buf + s * SLOT, &bars[s], offs, tid, I.fin[fld], I.vel, I.ncell, pz * plane_n,
+                                 (pz == 0 ? nz - 1 : pz - 1) * plane_n, (pz >= 3 ? pz - 3 : pz - 3 + nz) * plane_n);
+            } else if (tid == ISSUER && !tmo) {
                 zyx_issue(buf + s * SLOT, &bars[s], fmaps, maps, x0, y0, I.nx, I.ny, nz, pz, seam);
                 armed |= 1u << s;
             }
@@ -1004,6 +1141,10 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
         bu.set(O_UX + xrow * ZS, O_SX + 32 + 4 * xrow, xr, sl, sr);
         float *const obase = (BATCH ? I.out : I.fout[fld]) + (int64_t)(y0 + xrow) * I.nx + x0 + xr;
 
+        if constexpr (CH) {
+            build_table<CH, ZS>(offs, tid, x0, y0, I.nx, I.ny);
+            __syncthreads();
+        }
         ZWin<L2> win[NZW];
 #pragma unroll
         for (int k = 0; k < NZW; ++k) win[k].init();
@@ -1118,7 +1259,15 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
             bp.b2 = bp.mid + 4;
             x_run4(sY, bp, sb, bu, msx, o, bad);
             const int kw = zp >= 3 ? zp - 3 : zp - 3 + nz;
-            *reinterpret_cast<float4 *>(obase + (int64_t)kw * plane_n) = make_float4(o[0], o[1], o[2], o[3]);
+            float *dst = obase + (int64_t)kw * plane_n;
+            if constexpr (CH == 1) {
+                if (y0 + xrow < I.ny)
+#pragma unroll
+                    for (int i = 0; i < RX; ++i)
+                        if (x0 + xr + i < I.nx) dst[i] = o[i];
+            } else if (CH == 0 || (x0 + xr < I.nx && y0 + xrow < I.ny)) {
+                *reinterpret_cast<float4 *>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+            }
         };
 
         for (int p = pfirst; p <= plast; ++p) {
@@ -1127,7 +1276,10 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
         }
         __syncthreads();
     }
-    if (tid == ISSUER && armed) drain<NS>(bars, armed, par);
+    if constexpr (CH)
+        cp_async_wait_all();
+    else if (tid == ISSUER && armed)
+        drain<NS>(bars, armed, par);
     if (tmo) atomicOr(status, 2u);
     flag_cfl(status, bad);
 }
@@ -1140,17 +1292,26 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Fas
 #endif
 
 // Shared-memory opt-in and persistent grid size of one kernel, once per device.
-template <bool ZYX, bool BATCH>
-cudaError_t prepare(int &grid)
+template <bool ZYX, bool BATCH, int CH>
+constexpr auto kernel_of()
 {
-    static int cached[64] = {};
+    if constexpr (ZYX)
+        return k_cec_zyx_fast<BATCH, SL_ZYX_SLOTS, CH>;
+    else
+        return k_cec_xyz_fast<BATCH, SL_XYZ_SLOTS, CH>;
+}
+
+template <bool ZYX, bool BATCH, int CH>
+cudaError_t prepare(int &grid, int &nsm)
+{
+    static int cached[64] = {}, count[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (cached[dev] == 0) {
-        auto kern = ZYX ? k_cec_zyx_fast<BATCH, SL_ZYX_SLOTS> : k_cec_xyz_fast<BATCH, SL_XYZ_SLOTS>;
-        const size_t smem = ZYX ? zyx::smem<SL_ZYX_SLOTS>() : xyz::smem<SL_XYZ_SLOTS>();
+        auto kern = kernel_of<ZYX, BATCH, CH>();
+        const size_t smem = ZYX ? zyx::smem<SL_ZYX_SLOTS, CH>() : xyz::smem<SL_XYZ_SLOTS, CH>();
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         int per_sm = 0, sms = 0;
@@ -1158,30 +1319,31 @@ cudaError_t prepare(int &grid)
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
+        count[dev] = sms;
         cached[dev] = sms * (per_sm > 0 ? per_sm : 1);
     }
     grid = cached[dev];
+    nsm = count[dev];
     return cudaSuccess;
 }
 
-template <bool ZYX, bool BATCH>
-cudaError_t go_fast(const FastInst &one, const FastMaps &maps, const FastInst *tab, int ninst, int64_t total,
+template <bool ZYX, bool BATCH, int CH>
+cudaError_t go_fast(const FastInst &one, const MapsOf<CH> &maps, const FastInst *tab, int ninst, int64_t total,
                     unsigned *status, int grid_req, cudaStream_t st)
 {
-    int grid = 0;
-    cudaError_t e = prepare<ZYX, BATCH>(grid);
+    int grid = 0, sms = 1;
+    cudaError_t e = prepare<ZYX, BATCH, CH>(grid, sms);
     if (e != cudaSuccess) return e;
-    if (grid_req > 0) grid = grid_req;
     const int nf = tab ? 1 : one.nf;
+    if (grid_req > 0)
+        grid = grid_req;
+    else if (!tab)   // a plane of one CTA per SM takes 0.7 of a plane of two (300^3)
+        grid = (int)plan_ctas(one.ntiles, one.nzr, kFastHaloBelow, 0.7, grid / sms, sms, nf) * nf;
     if (grid > total) grid = (int)total;
     grid = grid >= nf ? grid / nf * nf : nf;   // whole groups of nf CTAs
     if (grid > total * nf) grid = (int)(total * nf);
-    if (ZYX)
-        k_cec_zyx_fast<BATCH, SL_ZYX_SLOTS>
-            <<<grid, NT, zyx::smem<SL_ZYX_SLOTS>(), st>>>(one, maps, tab, ninst, total, status);
-    else
-        k_cec_xyz_fast<BATCH, SL_XYZ_SLOTS>
-            <<<grid, NT, xyz::smem<SL_XYZ_SLOTS>(), st>>>(one, maps, tab, ninst, total, status);
+    const size_t smem = ZYX ? zyx::smem<SL_ZYX_SLOTS, CH>() : xyz::smem<SL_XYZ_SLOTS, CH>();
+    kernel_of<ZYX, BATCH, CH>()<<<grid, NT, smem, st>>>(one, maps, tab, ninst, total, status);
     return cudaGetLastError();
 }
 
@@ -1295,6 +1457,42 @@ bool fast_eligible(const int64_t dims[3], int ndim, int dtype, bool aligned)
            dims[1] >= 32 && dims[2] >= 8;
 }
 
+bool any_eligible(const int64_t dims[3], int ndim, int dtype)
+{
+    // planes reduced modulo nz by at most one period (nz >= 8)
+    return dtype == 0 && ndim == 3 && dims[2] >= 8;
+}
+
+cudaError_t launch_cec_any(const void *in, void *out, const void *vel, const int64_t dims[3], const double s[3],
+                           int parity, Launch lc, unsigned *status, const FieldSet &fs, cudaStream_t st)
+{
+    FastInst one;
+    fast_fill(one, in, out, vel, dims, s, 0);
+    one.tiles_x = (one.nx + TX - 1) / TX;
+    one.ntiles = one.tiles_x * ((one.ny + TY - 1) / TY);
+    const int64_t total = (int64_t)one.ntiles * one.nz;
+    const bool vec = lc.aligned && one.nx % 4 == 0;
+    const NoMaps none{};
+    for (int f0 = 0; f0 < fs.n; f0 += kFastFields) {
+        one.nf = fs.n - f0 < kFastFields ? fs.n - f0 : kFastFields;
+        for (int i = 0; i < one.nf; ++i) {
+            one.fin[i] = static_cast<const float *>(in) + (f0 + i) * fs.fin;
+            one.fout[i] = static_cast<float *>(out) + (f0 + i) * fs.fout;
+        }
+        int64_t grid = lc.tz > 0 ? (total + lc.tz - 1) / lc.tz * one.nf : 0;   // shares of lc.tz planes
+        if (grid > 0x7fffffff) grid = 0x7fffffff;
+        cudaError_t e;
+        if (parity & 1)
+            e = vec ? go_fast<true, false, 4>(one, none, nullptr, 1, total, status, (int)grid, st)
+                    : go_fast<true, false, 1>(one, none, nullptr, 1, total, status, (int)grid, st);
+        else
+            e = vec ? go_fast<false, false, 4>(one, none, nullptr, 1, total, status, (int)grid, st)
+                    : go_fast<false, false, 1>(one, none, nullptr, 1, total, status, (int)grid, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 void fast_fill(FastInst &f, const void *in, void *out, const void *vel, const int64_t dims[3], const double s[3],
                int64_t w0)
 {
@@ -1328,19 +1526,19 @@ cudaError_t launch_cec_fast(const FastInst &one, const FastInst *dev_table, int 
     const bool zyx_order = parity & 1;
     static FastMaps unused;   // batched launches read each instance's maps from the table
     if (dev_table)
-        return zyx_order ? go_fast<true, true>(one, unused, dev_table, ninst, total, status, grid_req, st)
-                         : go_fast<false, true>(one, unused, dev_table, ninst, total, status, grid_req, st);
+        return zyx_order ? go_fast<true, true, 0>(one, unused, dev_table, ninst, total, status, grid_req, st)
+                         : go_fast<false, true, 0>(one, unused, dev_table, ninst, total, status, grid_req, st);
     FastMaps maps;
     cudaError_t e = cached_maps(maps, one);
     if (e != cudaSuccess) return e;
-    return zyx_order ? go_fast<true, false>(one, maps, nullptr, 1, total, status, grid_req, st)
-                     : go_fast<false, false>(one, maps, nullptr, 1, total, status, grid_req, st);
+    return zyx_order ? go_fast<true, false, 0>(one, maps, nullptr, 1, total, status, grid_req, st)
+                     : go_fast<false, false, 0>(one, maps, nullptr, 1, total, status, grid_req, st);
 }
 
 int fast_grid(int parity)
 {
-    int g = 0;
-    if (((parity & 1) ? prepare<true, false>(g) : prepare<false, false>(g)) != cudaSuccess) return 0;
+    int g = 0, sms = 0;
+    if (((parity & 1) ? prepare<true, false, 0>(g, sms) : prepare<false, false, 0>(g, sms)) != cudaSuccess) return 0;
     return g;
 }
 

@@ -1,4 +1,6 @@
-// k_split.cu -- fused directionally split third-order step (SL_CEC).
+// k_split.cu -- fused directionally split third-order step (SL_CEC) in FP32 on
+// planes and on 3D grids of fewer than 8 planes, and the generic batched step
+// (k_cec_fast.cu and k_split64.cu serve the rest).
 //
 // One kernel performs the three 1D CEC sweeps of a time step (Sec. 2 last
 // paragraph, Sec. 5 eqs. split:1-2; per-axis coefficients of eq.
@@ -17,6 +19,8 @@
 // Loads are 16-byte cp.async copies of whole aligned rows (x staged over
 // [-4, TX+4)), double-buffered one plane ahead; periodic wrap-around is folded
 // into per-thread source offsets computed once per work item.
+#include <cmath>
+
 #include "sl_internal.h"
 
 namespace sl {
@@ -72,7 +76,7 @@ __device__ __forceinline__ void sts_vec(T *dst, const T (&src)[N])
 // row arithmetic).  The periodic wrap is in per-thread source offsets, computed
 // once per work item; wrapping every element of every plane again took most of
 // the time on grids whose rows are no multiple of 16 bytes (187 x 150 x 131,
-// x,y,z / z,y,x: 123 / 173 us before, 55 / 79 now; 46 / 69 us with rows of 188).
+// x,y,z / z,y,x: 123 / 173 us before, 55 / 79 after, when this kernel served it).
 template <typename T, int NT, int NR, int NC, int LD, bool VEC>
 struct Stager {
     static constexpr int V = VEC ? 16 / sizeof(T) : 1;
@@ -515,10 +519,32 @@ int default_tz(int dtype, int ndim, const int64_t dims[3])
     return tz < 1 ? 1 : tz;
 }
 
+int64_t plan_ctas(int64_t tiles, int64_t nz, int warm, double alone, int per_sm, int sms, int fields)
+{
+    auto plane = [&](int64_t ctas) {
+        const int64_t k = (ctas * fields + sms - 1) / sms;   // CTAs of the busiest SM
+        return k <= 1 ? alone : 0.5 * (double)k;
+    };
+    const int64_t total = tiles * nz, all = (int64_t)per_sm * sms / fields;
+    int64_t best = all < 1 ? 1 : (all < total ? all : total);
+    const double share = (double)total / (double)best;
+    double cost = (share + warm * (2.0 + floor(share / (double)nz))) * plane(best);
+    for (int64_t c = 1; c <= nz && tiles * c <= all; ++c) {
+        const double t = (double)((nz + c - 1) / c + warm) * plane(tiles * c);
+        if (t < cost) {
+            cost = t;
+            best = tiles * c;
+        }
+    }
+    return best;
+}
+
 cudaError_t launch_split_cec(int dtype, const void *in, void *out, const void *vel, int ndim,
                              const int64_t dims[3], const double s[3], int parity, Launch lc,
                              unsigned *status, cudaStream_t st, FieldSet fs)
 {
+    if (any_eligible(dims, ndim, dtype))
+        return launch_cec_any(in, out, vel, dims, s, parity, lc, status, fs, st);
     constexpr int TX = 32;
     Geo g;
     g.nx = (int)dims[0];

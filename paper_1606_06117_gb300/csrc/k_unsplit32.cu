@@ -23,10 +23,9 @@
 // (BEC, 256^3: 265 and 245 us), at 50 % issue activity and 44 % of the
 // shared-memory pipe, each plane's three stages separated by barriers.
 // Measured (CUDA events, us per step, k_unsplit.cu -> here):
-//   rows of no 16-byte multiple, 187 x 150 x 131: CIR 88 -> 27, FEC 132 -> 41,
-//   BEC 188 -> 62; 65 x 40 x 30: CIR 39.9 -> 4.8, BEC 33.7 -> 10.6;
-//   whole chunks: 64^3 FEC 20.8 -> 8.7, BEC 19.9 -> 12.6; 160^3 FEC 48.7 -> 45.1;
-//   188 x 150 x 131 BEC 74 -> 62; but 256^3 FEC 154 -> 182, 384^3 BEC 751 -> 808,
+//   rows of no 16-byte multiple, 187 x 150 x 131: CIR 88 -> 24, FEC 132 -> 41,
+//   BEC 188 -> 56; 65 x 40 x 30: CIR 39.9 -> 4.8, BEC 33.7 -> 10.6;
+//   whole chunks: 64^3 FEC 20.8 -> 8.7, BEC 19.9 -> 12.6; 128^3 FEC 29 -> 26, BEC 49 -> 38; but 256^3 FEC 154 -> 182, 384^3 BEC 751 -> 808,
 //   so large grids of whole chunks keep k_unsplit.cu (unsplit32_serves).
 #include <type_traits>
 
@@ -333,15 +332,9 @@ cudaError_t go(Geo g, int grid, const float *in, float *out, const float *vel, c
     g.tiles_y = (g.ny + TY - 1) / TY;
     const int64_t total = (int64_t)g.tiles_x * g.tiles_y * (g.tz > 0 ? g.chunks : g.nz);
     int64_t gr = total;
-    if (g.tz == 0) {
-        // as many CTAs as the GPU holds, or one per SM while their shares would be
-        // under 5 NST planes (each begins with 2 NST planes of warm-up: 96^3 FEC 17.1
-        // us with one per SM, 19.4 with two; 128^3 28.2 and 27.4), and two planes or
-        // more each
-        gr = (resident[dev] + fs.n - 1) / fs.n;
-        if (total < 5 * NST * gr) gr = (sms[dev] + fs.n - 1) / fs.n;
-        if (gr > (total + 1) / 2) gr = (total + 1) / 2;
-    }
+    // a plane of one CTA per SM takes 0.58 of a plane of two (BEC, 256^3)
+    if (g.tz == 0)
+        gr = plan_ctas((int64_t)g.tiles_x * g.tiles_y, g.nz, 2 * NST, 0.58, resident[dev] / sms[dev], sms[dev], fs.n);
     if (grid > 0 && grid < total) gr = grid;
     if (gr < 1) gr = 1;
     if (gr > 0x7fffffff) return cudaErrorInvalidConfiguration;
@@ -357,10 +350,10 @@ bool unsplit32_serves(int scheme, int ndim, const int64_t dims[3], bool vec)
     if (ndim != 3) return false;
     if (!vec) return true;
     // planes per share of two CTAs per SM: FEC crosses over between 26 (160^3: 45.1
-    // against 48.7 us) and 45 (192^3: 83 against 74), BEC between 45 (115 against
-    // 119) and 108 (256^3: 245 against 238)
+    // against 48.7 us) and 45 (192^3: 83 against 74), BEC between 45 (192^3: 115
+    // against 119) and some 50 (8 M cells: 121 against 118)
     const int64_t pairs = ((dims[0] + TX - 1) / TX) * ((dims[1] + TY - 1) / TY) * dims[2];
-    return pairs < (scheme == 2 ? 64 : 32) * 2 * 152;
+    return pairs < (scheme == 2 ? 46 : 28) * 2 * 152;
 }
 
 cudaError_t launch_unsplit32(int scheme, Geo g, int grid, const void *in, void *out, const void *vel,

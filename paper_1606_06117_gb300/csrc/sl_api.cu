@@ -821,6 +821,10 @@ int sl_autotune_scheme(void *out, const void *in, const void *vel, int ndim, con
         for (int k = 1; k <= std::min(occ, 2); ++k) cands.push_back({0, 0, k});
     } else if (fam == SL_KERNEL_CEC_SPLIT) {
         if (dtype != SL_F32 && ndim == 3) cands.push_back({0, 0, 0});   // equal shares
+        if (any_eligible(dims, ndim, dtype)) {                          // the default shares, as planes
+            const int64_t pairs = (dims[0] + 31) / 32 * ((dims[1] + 31) / 32) * dims[2], ctas = 2 * c->num_sms;
+            cands.push_back({0, (int)std::max<int64_t>(1, (pairs + ctas - 1) / ctas), 0});
+        }
         for (int tz : tzs) cands.push_back({0, tz, 0});
     } else if (fam == SL_KERNEL_CIR_GROUPS) {
         for (int ty : {16, 32})

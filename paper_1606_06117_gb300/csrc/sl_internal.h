@@ -105,6 +105,18 @@ cudaError_t launch_batched_cec(const BatchRec *dev_recs, int ninst, int nitems, 
 
 int default_tz(int dtype, int ndim, const int64_t dims[3]);
 
+// CTAs per field for a kernel whose CTAs take equal shares of the (column tile,
+// plane) pairs of `tiles` tiles of nz planes and begin every run of planes with
+// `warm` planes of warm-up.  A share that starts inside a tile and ends in the
+// next warms up twice; tiles * c CTAs cut every tile into c runs of at most
+// ceil(nz / c) planes that never do.  The cost of a choice is the planes its
+// busiest CTA works on, warm-ups included, times what a plane takes with that many
+// CTAs on an SM (two: 1, one: `alone`, k > 2: k / 2).
+// Measured, CEC x,y,z / z,y,x us per step, equal shares of all resident CTAs and
+// this: 187 x 150 x 131 59 / 68 and 49 / 58, 96^3 25 / 28 and 17.5 / 23, 192^3
+// 58 / 72 and 51 / 68, 24 x 400 x 60 30 / 30 and 20 / 21.
+int64_t plan_ctas(int64_t tiles, int64_t nz, int warm, double alone, int per_sm, int sms, int fields);
+
 // Fast FP32 CEC path (k_cec_fast.cu): one periodic grid of whole 32 x 32 column
 // tiles; w0 numbers its first (column tile, plane) pair in a batch.  A launch
 // writes the output planes [zb, zb + nzr) (fast_fill: all nz planes) and reads
@@ -141,6 +153,11 @@ void fast_fill(FastInst &f, const void *in, void *out, const void *vel, const in
 cudaError_t launch_cec_fast(const FastInst &one, const FastInst *dev_table, int ninst, int64_t total, int parity,
                             unsigned *status, int grid_req, cudaStream_t st);
 int fast_grid(int parity);
+// The same kernels on FP32 3D grids of any x and y size and alignment (nz >= 8);
+// lc.tz > 0: CTAs take shares of that many planes.
+bool any_eligible(const int64_t dims[3], int ndim, int dtype);
+cudaError_t launch_cec_any(const void *in, void *out, const void *vel, const int64_t dims[3], const double s[3],
+                           int parity, Launch lc, unsigned *status, const FieldSet &fs, cudaStream_t st);
 
 // Steps at any Courant number (k_wide.cu): non-local interpolation, unfused
 // kernels, intermediate fields in a caller-owned workspace of wide_fields()
