@@ -135,6 +135,24 @@ struct RowChunks {
     }
 };
 
+// The cells of a stage that this thread owns on every plane: those of the tile
+// widened by h cells with flat index tid + k NT, as offsets in the shared planes
+// (-1: none).
+template <int NT, int TX, int TY, int h, int H, int PW>
+struct Cells {
+    static constexpr int RW = TX + 2 * h, RH = TY + 2 * h, N = RW * RH, K = (N + NT - 1) / NT;
+    int o[K];
+
+    __device__ __forceinline__ void setup(int tid)
+    {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int r = tid + k * NT, yy = r / RW, xx = r - yy * RW;
+            o[k] = r < N ? (yy - h + H) * PW + (xx - h + 4) : -1;
+        }
+    }
+};
+
 template <typename T, typename D, int NST, int TX, int TY, bool HAS_Z, bool VEC>
 __global__ void __launch_bounds__(256)
 k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel, Geo g, int64_t fin, int64_t fout)
@@ -153,6 +171,12 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
     const int tid = threadIdx.x;
     const D sxd = D(g.sx), syd = D(g.sy), szd = D(g.sz);
     bool bad = false;
+    Cells<NT, TX, TY, NST - 1, H, PW> c1;
+    Cells<NT, TX, TY, NST >= 2 ? NST - 2 : 0, H, PW> c2;
+    Cells<NT, TX, TY, 0, H, PW> c3;
+    c1.setup(tid);
+    if constexpr (NST >= 2) c2.setup(tid);
+    if constexpr (NST >= 3) c3.setup(tid);
     // Work split.  BEC (three stages; its shared memory allows two CTAs per SM):
     // persistent CTAs; the (column tile, plane) pairs are numbered tile by tile
     // and every CTA takes one contiguous, equal share, walking z inside each
@@ -225,6 +249,14 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
         auto sl_l = [&](int q) { return sL + (K::NL > 1 ? ((q + 1 - pfirst) % 3) : 0) * SLL - K::SHL * PW; };
         auto sl_p = [&](int q) { return sP + (K::NP > 1 ? ((q + 1 - pfirst) % 3) : 0) * SLP - K::SHP * PW; };
 
+        // the results: rows tid / TX + k NT / TX of the tile, column tid mod TX
+        const int gx = x0 + tid % TX, gy = y0 + tid / TX;
+        T *const gout = out + (int64_t)gy * g.nx + gx;
+        auto store = [&](int k, int q, T v) {
+            if (gx < g.nx && gy + k * (NT / TX) < g.ny && (TX * TY % NT == 0 || tid + k * NT < TX * TY))
+                gout[(int64_t)(q >= g.nz ? q - g.nz : q) * g.plane + k * (NT / TX) * (int64_t)g.nx] = v;
+        };
+
         issue(pfirst);
         for (int p = pfirst; p <= plast; ++p) {
             cp_async_wait_all();
@@ -234,19 +266,14 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
             // ------------------------------------------------ stage 1: L_U[Phi]
             if (!HAS_Z || p >= z0 - NST + 2) {
                 const int q = HAS_Z ? p - 1 : 0;
-                constexpr int h = NST - 1;
-                constexpr int RW = TX + 2 * h, RH = TY + 2 * h;
                 const T *phi0 = sl_phi(q);
                 const T *cP = sl_c(q);
                 const T *phim = HAS_Z ? sl_phi(q - 1) : phi0, *php = HAS_Z ? sl_phi(q + 1) : phi0;
                 D *const lq = sl_l(q);
-                int yy = tid / RW, xx = tid - (tid / RW) * RW;
-                for (int r = tid; r < RW * RH; r += NT, xx += NT % RW, yy += NT / RW) {
-                    if (xx >= RW) {
-                        xx -= RW;
-                        ++yy;
-                    }
-                    const int o = (yy - h + H) * PW + (xx - h + 4);
+#pragma unroll
+                for (int k = 0; k < c1.K; ++k) {
+                    const int o = c1.o[k];
+                    if (c1.N % NT != 0 && o < 0) continue;
                     const D cx = D(cP[o]) * sxd, cy = D(cP[SC + o]) * syd;
                     const D cz = HAS_Z ? D(cP[2 * SC + o]) * szd : D(0);
                     const int ox = by_sign(cx, -1, 1, 0), oy = by_sign(cy, -PW, PW, 0);
@@ -255,8 +282,7 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                                                 D(1) - fabs(cz));
                     if constexpr (NST == 1) {
                         bad |= fabs(cx) > D(1) || fabs(cy) > D(1) || fabs(cz) > D(1);
-                        const int gx = x0 + xx, gy = y0 + yy;
-                        if (gx < g.nx && gy < g.ny) out[(int64_t)(q >= g.nz ? q - g.nz : q) * g.plane + (int64_t)gy * g.nx + gx] = T(v);
+                        store(k, q, T(v));
                     } else {
                         lq[o] = v;
                     }
@@ -267,20 +293,15 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                 // -------------------------------- stage 2: Phi_bar and the correction
                 if (!HAS_Z || p >= z0 - NST + 4) {
                     const int q = HAS_Z ? p - 2 : 0;
-                    constexpr int h = NST - 2;
-                    constexpr int RW = TX + 2 * h, RH = TY + 2 * h;
                     const T *phiq = sl_phi(q);
                     const T *cP = sl_c(q);
                     const D *l0 = sl_l(q);
                     const D *lp = HAS_Z ? sl_l(q + 1) : l0, *lm = HAS_Z ? sl_l(q - 1) : l0;
                     T *const pq = sl_p(q);
-                    int yy = tid / RW, xx = tid - (tid / RW) * RW;
-                    for (int r = tid; r < RW * RH; r += NT, xx += NT % RW, yy += NT / RW) {
-                        if (xx >= RW) {
-                            xx -= RW;
-                            ++yy;
-                        }
-                        const int o = (yy - h + H) * PW + (xx - h + 4);
+#pragma unroll
+                    for (int k = 0; k < c2.K; ++k) {
+                        const int o = c2.o[k];
+                        if (c2.N % NT != 0 && o < 0) continue;
                         const D cx = D(cP[o]) * sxd, cy = D(cP[SC + o]) * syd;
                         const D cz = HAS_Z ? D(cP[2 * SC + o]) * szd : D(0);
                         // reversed flow: departure x + u dt, corners toward +s
@@ -291,9 +312,7 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                         const D delta = D(phiq[o]) - bar;
                         if constexpr (NST == 2) {
                             bad |= fabs(cx) > D(1) || fabs(cy) > D(1) || fabs(cz) > D(1);
-                            const int gx = x0 + xx, gy = y0 + yy;
-                            if (gx < g.nx && gy < g.ny)
-                                out[(int64_t)(q >= g.nz ? q - g.nz : q) * g.plane + (int64_t)gy * g.nx + gx] = T(l0[o] + delta * D(0.5));
+                            store(k, q, T(l0[o] + delta * D(0.5)));
                         } else {
                             pq[o] = T(D(phiq[o]) + delta * D(0.5));
                         }
@@ -308,9 +327,10 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                     const T *cP = sl_c(q);
                     const T *p0 = sl_p(q);
                     const T *pm = HAS_Z ? sl_p(q - 1) : p0, *pp = HAS_Z ? sl_p(q + 1) : p0;
-                    for (int r = tid; r < TX * TY; r += NT) {
-                        const int yy = r / TX, xx = r - (r / TX) * TX;
-                        const int o = (yy + H) * PW + (xx + 4);
+#pragma unroll
+                    for (int k = 0; k < c3.K; ++k) {
+                        const int o = c3.o[k];
+                        if (c3.N % NT != 0 && o < 0) continue;
                         const T cx = T(D(cP[o]) * sxd), cy = T(D(cP[SC + o]) * syd);
                         const T cz = HAS_Z ? T(D(cP[2 * SC + o]) * szd) : T(0);
                         bad |= fabs(cx) > T(1) || fabs(cy) > T(1) || fabs(cz) > T(1);
@@ -318,8 +338,7 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                         const T *p1 = HAS_Z ? by_sign<T, const T *>(cz, pm, pp, p0) : p0;
                         const T v = mlerp<T, HAS_Z>(p0, p1, o, ox, oy, T(1) - fabs(cx), T(1) - fabs(cy),
                                                     T(1) - fabs(cz));
-                        const int gx = x0 + xx, gy = y0 + yy;
-                        if (gx < g.nx && gy < g.ny) out[(int64_t)(q >= g.nz ? q - g.nz : q) * g.plane + (int64_t)gy * g.nx + gx] = v;
+                        store(k, q, v);
                     }
                 }
             }
