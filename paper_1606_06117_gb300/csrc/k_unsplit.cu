@@ -13,6 +13,16 @@
 // behind the newest loaded plane, and each stage keeps the three planes its
 // successor reads in a shared-memory ring.  One HBM read of Phi and u and one
 // write of the result per cell.
+//
+// What bounds it: instruction issue (BEC, 256^3: 69 % of the slots), then the
+// shared-memory pipe (53 %).  A cell's evaluation gathers eight corners at offsets
+// of its own, so what can be saved is everything around the gathers: the cells of
+// a thread are fixed per stage before the plane loop, a warp's tile cells are one
+// row (a row-by-row numbering of the widened tile straddled two rows of another
+// pitch in nearly every warp, two wavefronts per load), ring slots step with the
+// plane.  Measured (us per step, in that order): FEC 256^3 153 -> 142 -> 133.5 ->
+// 133.5, BEC 512^3 1735 -> 1651 -> 1570 -> 1530; items of 64 planes at most, FEC
+// 512^3 987 -> 925.
 #include "sl_internal.h"
 
 namespace sl {
@@ -135,20 +145,46 @@ struct RowChunks {
     }
 };
 
-// The cells of a stage that this thread owns on every plane: those of the tile
-// widened by h cells with flat index tid + k NT, as offsets in the shared planes
-// (-1: none).
+// The cells of a stage that this thread owns on every plane, as offsets in the
+// shared planes (-1: none): those of the tile first, whole rows of 32 to a warp,
+// then the rings that widen the tile by 1 .. h cells, each as its top row, bottom
+// row and sides.  (Numbering the widened tile row by row makes nearly every warp
+// straddle two rows, whose staged pitch differs from the widened width: two
+// wavefronts per shared load.)
 template <int NT, int TX, int TY, int h, int H, int PW>
 struct Cells {
-    static constexpr int RW = TX + 2 * h, RH = TY + 2 * h, N = RW * RH, K = (N + NT - 1) / NT;
+    static constexpr int KI = (TX * TY + NT - 1) / NT;
+    static constexpr int NR = (TX + 2 * h) * (TY + 2 * h) - TX * TY, K = KI + (NR + NT - 1) / NT;
     int o[K];
 
     __device__ __forceinline__ void setup(int tid)
     {
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int r = tid + k * NT, yy = r / RW, xx = r - yy * RW;
-            o[k] = r < N ? (yy - h + H) * PW + (xx - h + 4) : -1;
+        for (int k = 0; k < KI; ++k) {
+            const int r = tid + k * NT;
+            o[k] = r < TX * TY ? (r / TX + H) * PW + r % TX + 4 : -1;
+        }
+#pragma unroll
+        for (int k = KI; k < K; ++k) {
+            int i = tid + (k - KI) * NT, w = 1;
+            o[k] = -1;
+            if (i < NR) {
+                while (w < h && i >= 2 * (TX + TY + 4 * w - 2)) {   // cells of ring w
+                    i -= 2 * (TX + TY + 4 * w - 2);
+                    ++w;
+                }
+                const int W = TX + 2 * w;
+                int x, y;
+                if (i < 2 * W) {
+                    x = i < W ? i - w : i - W - w;
+                    y = i < W ? -w : TY + w - 1;
+                } else {
+                    i -= 2 * W;
+                    x = (i & 1) ? TX + w - 1 : -w;
+                    y = 1 - w + (i >> 1);
+                }
+                o[k] = (y + H) * PW + x + 4;
+            }
         }
     }
 };
@@ -224,11 +260,11 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
             chC.setup(tid, x0, y0, -(H - 1), H, g.nx, g.ny);
         }
 
-        auto issue = [&](int p) {
-            const int b = p - pfirst;
+        auto issue = [&](int p, int cslot) {
+            const unsigned b = p - pfirst;
             const int64_t base = (int64_t)wrapi(p, g.nz) * g.plane;
             const int64_t bc = HAS_Z ? (int64_t)wrapi(p - 1, g.nz) * g.plane : base;
-            T *cdst = sC + (b % K::NCS) * K::NC * SC - K::SHC * PW;
+            T *cdst = sC + cslot * K::NC * SC - K::SHC * PW;
             if (once) {
                 chPhi.issue(sPhi + (b % K::NPHI) * SLOT, in + base);
 #pragma unroll
@@ -243,11 +279,15 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
             }
             cp_async_commit();
         };
-        // ring slots of plane q
-        auto sl_phi = [&](int q) { return sPhi + ((q - pfirst) % K::NPHI) * SLOT; };
-        auto sl_c = [&](int q) { return sC + ((q + 1 - pfirst) % K::NCS) * K::NC * SC - K::SHC * PW; };
-        auto sl_l = [&](int q) { return sL + (K::NL > 1 ? ((q + 1 - pfirst) % 3) : 0) * SLL - K::SHL * PW; };
-        auto sl_p = [&](int q) { return sP + (K::NP > 1 ? ((q + 1 - pfirst) % 3) : 0) * SLP - K::SHP * PW; };
+        // Ring slots of plane p - back, from this iteration's places i3 = b mod 3 and
+        // ic = b mod NCS, b = p - pfirst (the places step with p: a signed remainder
+        // per slot, plane and thread was a fifth of the kernel's instructions).
+        int i3 = 0, ic = 0;
+        auto behind = [](int i, int back, int n) { return i >= back ? i - back : i - back + n; };
+        auto sl_phi = [&](int b, int back) { return sPhi + (HAS_Z ? (unsigned)(b - back) % K::NPHI : 0) * SLOT; };
+        auto sl_c = [&](int back) { return sC + (HAS_Z ? behind(ic, back - 1, K::NCS) : 0) * K::NC * SC - K::SHC * PW; };
+        auto sl_l = [&](int back) { return sL + (K::NL > 1 ? behind(i3, back - 1, 3) : 0) * SLL - K::SHL * PW; };
+        auto sl_p = [&](int back) { return sP + (K::NP > 1 ? behind(i3, back - 2, 3) : 0) * SLP - K::SHP * PW; };
 
         // the results: rows tid / TX + k NT / TX of the tile, column tid mod TX
         const int gx = x0 + tid % TX, gy = y0 + tid / TX;
@@ -257,23 +297,24 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                 gout[(int64_t)(q >= g.nz ? q - g.nz : q) * g.plane + k * (NT / TX) * (int64_t)g.nx] = v;
         };
 
-        issue(pfirst);
+        issue(pfirst, 0);
         for (int p = pfirst; p <= plast; ++p) {
             cp_async_wait_all();
             __syncthreads();
-            if (p < plast) issue(p + 1);
+            const int b = p - pfirst;
+            if (p < plast) issue(p + 1, ic + 1 == K::NCS ? 0 : ic + 1);
 
             // ------------------------------------------------ stage 1: L_U[Phi]
             if (!HAS_Z || p >= z0 - NST + 2) {
                 const int q = HAS_Z ? p - 1 : 0;
-                const T *phi0 = sl_phi(q);
-                const T *cP = sl_c(q);
-                const T *phim = HAS_Z ? sl_phi(q - 1) : phi0, *php = HAS_Z ? sl_phi(q + 1) : phi0;
-                D *const lq = sl_l(q);
+                const T *phi0 = sl_phi(b, 1);
+                const T *cP = sl_c(1);
+                const T *phim = HAS_Z ? sl_phi(b, 2) : phi0, *php = HAS_Z ? sl_phi(b, 0) : phi0;
+                D *const lq = sl_l(1);
 #pragma unroll
                 for (int k = 0; k < c1.K; ++k) {
                     const int o = c1.o[k];
-                    if (c1.N % NT != 0 && o < 0) continue;
+                    if ((k >= c1.KI || TX * TY % NT != 0) && o < 0) continue;
                     const D cx = D(cP[o]) * sxd, cy = D(cP[SC + o]) * syd;
                     const D cz = HAS_Z ? D(cP[2 * SC + o]) * szd : D(0);
                     const int ox = by_sign(cx, -1, 1, 0), oy = by_sign(cy, -PW, PW, 0);
@@ -293,15 +334,15 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                 // -------------------------------- stage 2: Phi_bar and the correction
                 if (!HAS_Z || p >= z0 - NST + 4) {
                     const int q = HAS_Z ? p - 2 : 0;
-                    const T *phiq = sl_phi(q);
-                    const T *cP = sl_c(q);
-                    const D *l0 = sl_l(q);
-                    const D *lp = HAS_Z ? sl_l(q + 1) : l0, *lm = HAS_Z ? sl_l(q - 1) : l0;
-                    T *const pq = sl_p(q);
+                    const T *phiq = sl_phi(b, 2);
+                    const T *cP = sl_c(2);
+                    const D *l0 = sl_l(2);
+                    const D *lp = HAS_Z ? sl_l(1) : l0, *lm = HAS_Z ? sl_l(3) : l0;
+                    T *const pq = sl_p(2);
 #pragma unroll
                     for (int k = 0; k < c2.K; ++k) {
                         const int o = c2.o[k];
-                        if (c2.N % NT != 0 && o < 0) continue;
+                        if ((k >= c2.KI || TX * TY % NT != 0) && o < 0) continue;
                         const D cx = D(cP[o]) * sxd, cy = D(cP[SC + o]) * syd;
                         const D cz = HAS_Z ? D(cP[2 * SC + o]) * szd : D(0);
                         // reversed flow: departure x + u dt, corners toward +s
@@ -324,13 +365,13 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                 // -------------------------------------------- stage 3: L_U[Psi]
                 if (!HAS_Z || p >= z0 + 3) {
                     const int q = HAS_Z ? p - 3 : 0;
-                    const T *cP = sl_c(q);
-                    const T *p0 = sl_p(q);
-                    const T *pm = HAS_Z ? sl_p(q - 1) : p0, *pp = HAS_Z ? sl_p(q + 1) : p0;
+                    const T *cP = sl_c(3);
+                    const T *p0 = sl_p(3);
+                    const T *pm = HAS_Z ? sl_p(4) : p0, *pp = HAS_Z ? sl_p(2) : p0;
 #pragma unroll
                     for (int k = 0; k < c3.K; ++k) {
                         const int o = c3.o[k];
-                        if (c3.N % NT != 0 && o < 0) continue;
+                        if (TX * TY % NT != 0 && o < 0) continue;
                         const T cx = T(D(cP[o]) * sxd), cy = T(D(cP[SC + o]) * syd);
                         const T cz = HAS_Z ? T(D(cP[2 * SC + o]) * szd) : T(0);
                         bad |= fabs(cx) > T(1) || fabs(cy) > T(1) || fabs(cz) > T(1);
@@ -342,6 +383,8 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                     }
                 }
             }
+            i3 = i3 == 2 ? 0 : i3 + 1;
+            ic = ic + 1 == K::NCS ? 0 : ic + 1;
         }
         __syncthreads();
     }
@@ -354,7 +397,7 @@ cudaError_t go(Geo g, int grid, const void *in, void *out, const void *vel, cons
     using K = Cfg<T, D, NST, TX, TY, HAS_Z>;
     auto kern = k_unsplit<T, D, NST, TX, TY, HAS_Z, VEC>;
     // shared-memory opt-in and resident CTAs per SM, once per device
-    static int per_dev[64] = {};
+    static int per_dev[64] = {}, sm_count[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -367,12 +410,16 @@ cudaError_t go(Geo g, int grid, const void *in, void *out, const void *vel, cons
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, K::NT, K::smem());
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
+        sm_count[dev] = sms;
         per_dev[dev] = sms * (per_sm > 0 ? per_sm : 1);
     }
     g.tiles_y = (g.ny + TY - 1) / TY;
     const bool persist = NST == 3 && HAS_Z;
     const int64_t total = (int64_t)g.tiles_x * g.tiles_y * (persist ? g.nz : g.chunks);
-    int gr = grid > 0 ? grid : (persist ? per_dev[dev] : (int)total);
+    int gr = grid > 0 ? grid : (int)total;
+    if (persist && grid <= 0)   // a plane of one CTA per SM takes 0.7 of a plane of two (256^3)
+        gr = (int)plan_ctas((int64_t)g.tiles_x * g.tiles_y, g.nz, 2 * NST, 0.7, per_dev[dev] / sm_count[dev],
+                            sm_count[dev], fs.n);
     if (gr > total) gr = (int)total;
     kern<<<dim3(gr, fs.n), K::NT, K::smem(), st>>>(static_cast<const T *>(in), static_cast<T *>(out),
                                                    static_cast<const T *>(vel), g, fs.fin, fs.fout);
@@ -428,6 +475,9 @@ cudaError_t launch_unsplit(int dtype, int scheme, const void *in, void *out, con
     g.sz = ndim == 3 ? s[2] : 0.0;
     g.status = status;
     g.tz = ndim == 3 ? (lc.tz > 0 ? lc.tz : default_tz(dtype, ndim, dims)) : 1;
+    // more than 64 planes per item leave too few items to even out (FEC, 512^3: 925 us
+    // with 64, 987 with 256)
+    if (lc.tz <= 0 && scheme == 1 && g.tz > 64) g.tz = 64;
     if (g.tz > g.nz) g.tz = g.nz;
     g.chunks = (g.nz + g.tz - 1) / g.tz;
     g.tiles_x = (g.nx + 31) / 32;

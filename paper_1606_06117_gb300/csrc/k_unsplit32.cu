@@ -25,8 +25,9 @@
 // Measured (CUDA events, us per step, k_unsplit.cu -> here):
 //   rows of no 16-byte multiple, 187 x 150 x 131: CIR 88 -> 24, FEC 132 -> 41,
 //   BEC 188 -> 56; 65 x 40 x 30: CIR 39.9 -> 4.8, BEC 33.7 -> 10.6;
-//   whole chunks: 64^3 FEC 20.8 -> 8.7, BEC 19.9 -> 12.6; 128^3 FEC 29 -> 26, BEC 49 -> 38; but 256^3 FEC 154 -> 182, 384^3 BEC 751 -> 808,
-//   so large grids of whole chunks keep k_unsplit.cu (unsplit32_serves).
+//   whole chunks: 64^3 FEC 18.4 -> 8.5, BEC 14.0 -> 12.7, 188 x 150 x 131 BEC
+//   60.5 -> 56.2; but 192^3 FEC 65 -> 82, BEC 102 -> 111, so larger grids of whole
+//   chunks keep k_unsplit.cu (unsplit32_serves).
 #include <type_traits>
 
 #include "sl_internal.h"
@@ -349,11 +350,11 @@ bool unsplit32_serves(int scheme, int ndim, const int64_t dims[3], bool vec)
 {
     if (ndim != 3) return false;
     if (!vec) return true;
-    // planes per share of two CTAs per SM: FEC crosses over between 26 (160^3: 45.1
-    // against 48.7 us) and 45 (192^3: 83 against 74), BEC between 45 (192^3: 115
-    // against 119) and some 50 (8 M cells: 121 against 118)
+    // by the (column tile, plane) pairs of the grid: FEC crosses over between 2600
+    // (48 x 200 x 100: 20.4 against 21.6 us) and 4096 (128^3: 25.4 against 24.9), BEC
+    // between 8000 (160^3: 61.3 against 62.6) and 11200 (256 x 100 x 200: 91 against 87)
     const int64_t pairs = ((dims[0] + TX - 1) / TX) * ((dims[1] + TY - 1) / TY) * dims[2];
-    return pairs < (scheme == 2 ? 46 : 28) * 2 * 152;
+    return pairs < (scheme == 2 ? 9000 : 3000);
 }
 
 cudaError_t launch_unsplit32(int scheme, Geo g, int grid, const void *in, void *out, const void *vel,
