@@ -475,9 +475,13 @@ cudaError_t launch_unsplit(int dtype, int scheme, const void *in, void *out, con
     g.sz = ndim == 3 ? s[2] : 0.0;
     g.status = status;
     g.tz = ndim == 3 ? (lc.tz > 0 ? lc.tz : default_tz(dtype, ndim, dims)) : 1;
-    // more than 64 planes per item leave too few items to even out (FEC, 512^3: 925 us
-    // with 64, 987 with 256)
-    if (lc.tz <= 0 && scheme == 1 && g.tz > 64) g.tz = 64;
+    // FEC items: 64 planes at most where that leaves items for six rounds of the 608
+    // resident CTAs, else 40 (512^3: 925 us with 64, 987 with 256; 384^3: 403 with 38,
+    // 421 with 64)
+    if (lc.tz <= 0 && scheme == 1) {
+        const int64_t items = (dims[0] + 31) / 32 * ((dims[1] + 15) / 16) * ((dims[2] + 63) / 64);
+        g.tz = g.tz < 40 ? g.tz : (items >= 6 * 608 ? 64 : 40);
+    }
     if (g.tz > g.nz) g.tz = g.nz;
     g.chunks = (g.nz + g.tz - 1) / g.tz;
     g.tiles_x = (g.nx + 31) / 32;
