@@ -244,7 +244,8 @@ int sl_field_load(const char *path, void *field, int ndim, const int64_t dims[3]
  *   SL_KERNEL_UNSPLIT      generic CIR / FEC / BEC kernels: on large FP32 3D grids
  *                          with dims[0] % 4 == 0 and aligned buffers tile height
  *                          8, 16 or 32 (otherwise a fixed height) and planes per
- *                          work item, or for 3D BEC and the other FP32 3D grids
+ *                          work item, or for 3D BEC, the other FP32 3D grids and
+ *                          3D steps in SL_F64 and SL_F32_D64
  *                          (persistent equal shares) CTAs per SM.
  * A choice is cached per (dims, scheme, dtype) in the process and used by
  * sl_advect, sl_advect_multi, sl_advect_host and sl_batch_create whenever the

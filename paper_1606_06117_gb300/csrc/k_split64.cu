@@ -30,31 +30,6 @@ namespace {
 constexpr int TX = 32;
 
 // -------------------------------------------------- bit-pattern operations
-__device__ __forceinline__ double widen(double v) { return v; }
-// Exact float to double without the conversion instruction, for normal numbers
-// and zeros; denormals, infinities and NaN take the instruction.
-__device__ __forceinline__ double widen(float v)
-{
-    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
-    if (m - 1u < 0x007fffffu || m >= 0x7f800000u) return (double)v;
-    const unsigned hi = (b & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u);
-    return __hiloint2double((int)hi, (int)(b << 29));
-}
-
-// sgn C (a NaN counts as its sign bit says: every use ends in a NaN anyway)
-__device__ __forceinline__ int sgn_bits(double c)
-{
-    const int hi = __double2hiint(c);
-    return ((hi & 0x7fffffff) | __double2loint(c)) == 0 ? 0 : (hi < 0 ? -1 : 1);
-}
-
-// |C| > 1 (false for a NaN, like the comparison)
-__device__ __forceinline__ bool beyond_one(double c)
-{
-    const unsigned long long a = (unsigned long long)__double_as_longlong(c) & 0x7fffffffffffffffull;
-    return a > 0x3ff0000000000000ull && a <= 0x7ff0000000000000ull;
-}
-
 __device__ __forceinline__ double pick(int s, double pos, double neg, double zero)
 {
     return s > 0 ? pos : (s < 0 ? neg : zero);

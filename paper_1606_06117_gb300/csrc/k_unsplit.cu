@@ -38,14 +38,14 @@ namespace {
 template <typename A, bool HAS_Z, typename S>
 __device__ __forceinline__ A mlerp(const S *q0, const S *q1, int o, int ox, int oy, A wx, A wy, A wz)
 {
-    const A a00 = A(q0[o]), a10 = A(q0[o + ox]), a01 = A(q0[o + oy]), a11 = A(q0[o + oy + ox]);
+    const A a00 = to<A>(q0[o]), a10 = to<A>(q0[o + ox]), a01 = to<A>(q0[o + oy]), a11 = to<A>(q0[o + oy + ox]);
     const A b0 = a10 + wx * (a00 - a10);
     const A b1 = a11 + wx * (a01 - a11);
     const A c0 = b1 + wy * (b0 - b1);
     if constexpr (!HAS_Z) {
         return c0;
     } else {
-        const A e00 = A(q1[o]), e10 = A(q1[o + ox]), e01 = A(q1[o + oy]), e11 = A(q1[o + oy + ox]);
+        const A e00 = to<A>(q1[o]), e10 = to<A>(q1[o + ox]), e01 = to<A>(q1[o + oy]), e11 = to<A>(q1[o + oy + ox]);
         const A f0 = e10 + wx * (e00 - e10);
         const A f1 = e11 + wx * (e01 - e11);
         const A c1 = f1 + wy * (f0 - f1);
@@ -219,9 +219,11 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
     // tile.  A tile's pairs are numbered from a tile-dependent plane, so that
     // the share boundaries of all tiles fall on the same planes (neighbouring
     // tiles are then processed at the same z and their shared halo rows stay in
-    // L2); planes are taken modulo nz.  CIR and FEC (more CTAs per SM): one
-    // (column tile, z chunk of g.tz planes) item per CTA, items over the grid.
-    constexpr bool PERSIST = NST == 3 && HAS_Z;
+    // L2); planes are taken modulo nz.  So do all 3D steps in double arithmetic
+    // (bound by the FP64 pipe; items of 16 planes left a 64^3 FEC step 64 CTAs).  CIR
+    // and FEC in FP32 (more CTAs per SM): one (column tile, z chunk of g.tz planes)
+    // item per CTA, items over the grid.
+    constexpr bool PERSIST = HAS_Z && (NST == 3 || sizeof(D) == 8);
     const int nzz = HAS_Z ? g.nz : 1;
     const int64_t total = PERSIST ? (int64_t)g.tiles_x * g.tiles_y * nzz : (int64_t)g.tiles_x * g.tiles_y * g.chunks;
     const int64_t G = gridDim.x;
@@ -315,14 +317,14 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                 for (int k = 0; k < c1.K; ++k) {
                     const int o = c1.o[k];
                     if ((k >= c1.KI || TX * TY % NT != 0) && o < 0) continue;
-                    const D cx = D(cP[o]) * sxd, cy = D(cP[SC + o]) * syd;
-                    const D cz = HAS_Z ? D(cP[2 * SC + o]) * szd : D(0);
+                    const D cx = to<D>(cP[o]) * sxd, cy = to<D>(cP[SC + o]) * syd;
+                    const D cz = HAS_Z ? to<D>(cP[2 * SC + o]) * szd : D(0);
                     const int ox = by_sign(cx, -1, 1, 0), oy = by_sign(cy, -PW, PW, 0);
                     const T *phi1 = HAS_Z ? by_sign<D, const T *>(cz, phim, php, phi0) : phi0;
                     const D v = mlerp<D, HAS_Z>(phi0, phi1, o, ox, oy, D(1) - fabs(cx), D(1) - fabs(cy),
                                                 D(1) - fabs(cz));
                     if constexpr (NST == 1) {
-                        bad |= fabs(cx) > D(1) || fabs(cy) > D(1) || fabs(cz) > D(1);
+                        bad |= beyond_one(cx) || beyond_one(cy) || beyond_one(cz);
                         store(k, q, T(v));
                     } else {
                         lq[o] = v;
@@ -343,19 +345,19 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                     for (int k = 0; k < c2.K; ++k) {
                         const int o = c2.o[k];
                         if ((k >= c2.KI || TX * TY % NT != 0) && o < 0) continue;
-                        const D cx = D(cP[o]) * sxd, cy = D(cP[SC + o]) * syd;
-                        const D cz = HAS_Z ? D(cP[2 * SC + o]) * szd : D(0);
+                        const D cx = to<D>(cP[o]) * sxd, cy = to<D>(cP[SC + o]) * syd;
+                        const D cz = HAS_Z ? to<D>(cP[2 * SC + o]) * szd : D(0);
                         // reversed flow: departure x + u dt, corners toward +s
                         const int ox = by_sign(cx, 1, -1, 0), oy = by_sign(cy, PW, -PW, 0);
                         const D *l1 = HAS_Z ? by_sign<D, const D *>(cz, lp, lm, l0) : l0;
                         const D bar = mlerp<D, HAS_Z>(l0, l1, o, ox, oy, D(1) - fabs(cx), D(1) - fabs(cy),
                                                       D(1) - fabs(cz));
-                        const D delta = D(phiq[o]) - bar;
+                        const D phi = to<D>(phiq[o]), delta = phi - bar;
                         if constexpr (NST == 2) {
-                            bad |= fabs(cx) > D(1) || fabs(cy) > D(1) || fabs(cz) > D(1);
+                            bad |= beyond_one(cx) || beyond_one(cy) || beyond_one(cz);
                             store(k, q, T(l0[o] + delta * D(0.5)));
                         } else {
-                            pq[o] = T(D(phiq[o]) + delta * D(0.5));
+                            pq[o] = T(phi + delta * D(0.5));
                         }
                     }
                 }
@@ -372,9 +374,9 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
                     for (int k = 0; k < c3.K; ++k) {
                         const int o = c3.o[k];
                         if (TX * TY % NT != 0 && o < 0) continue;
-                        const T cx = T(D(cP[o]) * sxd), cy = T(D(cP[SC + o]) * syd);
-                        const T cz = HAS_Z ? T(D(cP[2 * SC + o]) * szd) : T(0);
-                        bad |= fabs(cx) > T(1) || fabs(cy) > T(1) || fabs(cz) > T(1);
+                        const T cx = T(to<D>(cP[o]) * sxd), cy = T(to<D>(cP[SC + o]) * syd);
+                        const T cz = HAS_Z ? T(to<D>(cP[2 * SC + o]) * szd) : T(0);
+                        bad |= beyond_one(cx) || beyond_one(cy) || beyond_one(cz);
                         const int ox = by_sign(cx, -1, 1, 0), oy = by_sign(cy, -PW, PW, 0);
                         const T *p1 = HAS_Z ? by_sign<T, const T *>(cz, pm, pp, p0) : p0;
                         const T v = mlerp<T, HAS_Z>(p0, p1, o, ox, oy, T(1) - fabs(cx), T(1) - fabs(cy),
@@ -414,11 +416,13 @@ cudaError_t go(Geo g, int grid, const void *in, void *out, const void *vel, cons
         per_dev[dev] = sms * (per_sm > 0 ? per_sm : 1);
     }
     g.tiles_y = (g.ny + TY - 1) / TY;
-    const bool persist = NST == 3 && HAS_Z;
+    const bool persist = HAS_Z && (NST == 3 || sizeof(D) == 8);
     const int64_t total = (int64_t)g.tiles_x * g.tiles_y * (persist ? g.nz : g.chunks);
     int gr = grid > 0 ? grid : (int)total;
-    if (persist && grid <= 0)   // a plane of one CTA per SM takes 0.7 of a plane of two (256^3)
-        gr = (int)plan_ctas((int64_t)g.tiles_x * g.tiles_y, g.nz, 2 * NST, 0.7, per_dev[dev] / sm_count[dev],
+    // a plane of one CTA per SM takes 0.7 of a plane of two (FP32 BEC, 256^3), or
+    // little more than half where they share the FP64 pipe
+    if (persist && grid <= 0)
+        gr = (int)plan_ctas((int64_t)g.tiles_x * g.tiles_y, g.nz, 2 * NST, sizeof(D) == 8 ? 0.55 : 0.7, per_dev[dev] / sm_count[dev],
                             sm_count[dev], fs.n);
     if (gr > total) gr = (int)total;
     kern<<<dim3(gr, fs.n), K::NT, K::smem(), st>>>(static_cast<const T *>(in), static_cast<T *>(out),

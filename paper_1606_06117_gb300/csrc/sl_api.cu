@@ -839,7 +839,7 @@ int sl_autotune_scheme(void *out, const void *in, const void *vel, int ndim, con
             std::vector<int> tys = {0};
             if (dtype == SL_F32 && ndim == 3) tys = {8, 16, 32};
             for (int ty : tys) {
-                if (scheme == SL_BEC && ndim == 3)
+                if (ndim == 3 && (scheme == SL_BEC || dtype != SL_F32))
                     for (int k = 1; k <= 3; ++k) cands.push_back({ty, 0, k});
                 else
                     for (int tz : tzs) cands.push_back({ty, tz, 0});

@@ -88,9 +88,55 @@ __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.lau
 // keeps the cell.  D is the arithmetic type (float, or double with float
 // storage for SL_F32_D64).
 
+// GB300 issues about two double operations per clock and SM, comparisons and
+// float-to-double conversions included, so double signs, bounds and widenings go
+// through the bit patterns.
+//
+// sgn C (a NaN counts as its sign bit says: every use ends in a NaN anyway)
+__device__ __forceinline__ int sgn_bits(double c)
+{
+    const int hi = __double2hiint(c);
+    return ((hi & 0x7fffffff) | __double2loint(c)) == 0 ? 0 : (hi < 0 ? -1 : 1);
+}
+
+// |C| > 1 (false for a NaN, like the comparison)
+__device__ __forceinline__ bool beyond_one(float c) { return fabsf(c) > 1.f; }
+__device__ __forceinline__ bool beyond_one(double c)
+{
+    const unsigned long long a = (unsigned long long)__double_as_longlong(c) & 0x7fffffffffffffffull;
+    return a > 0x3ff0000000000000ull && a <= 0x7ff0000000000000ull;
+}
+
+// Exact conversion to the arithmetic type: float to double without the conversion
+// instruction for normal numbers and zeros; denormals, infinities and NaN take it.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v)
+{
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m - 1u < 0x007fffffu || m >= 0x7f800000u) return (double)v;
+    const unsigned hi = (b & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+template <typename D, typename T>
+__device__ __forceinline__ D to(T v)
+{
+    if constexpr (sizeof(D) == 8)
+        return widen(v);
+    else
+        return D(v);
+}
+
 // by the sign of C: C > 0, C < 0, C == 0
 template <typename D, typename V>
-__device__ __forceinline__ V by_sign(D C, V pos, V neg, V zero) { return C > D(0) ? pos : (C < D(0) ? neg : zero); }
+__device__ __forceinline__ V by_sign(D C, V pos, V neg, V zero)
+{
+    if constexpr (sizeof(D) == 8) {
+        const int s = sgn_bits(C);
+        return s > 0 ? pos : (s < 0 ? neg : zero);
+    } else {
+        return C > D(0) ? pos : (C < D(0) ? neg : zero);
+    }
+}
 
 // Outputs o[0..R) of a line segment from p[0..R+6) = Phi at offsets -3..R+2
 // and c[0..R+4) = Courant numbers at offsets -2..R+1.
