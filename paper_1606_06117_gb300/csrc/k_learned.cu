@@ -298,6 +298,16 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b
         "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
+// The same with A in tensor memory: row = lane, two BF16 elements along K per column.
+__device__ __forceinline__ void mma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t idesc, int accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(b), "r"(idesc), "r"(accumulate));
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t *bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -331,10 +341,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, unsigned parity
     return false;
 }
 
-// 32 lanes x 32 consecutive TMEM columns into v[0..32) (this thread's lane).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
+// 32 lanes x 64 consecutive TMEM columns into v[0..64) (this thread's lane), both
+// loads in flight before the wait.
+__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[32])
 {
-    uint32_t r[32];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
         "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
@@ -343,10 +353,43 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+// Waits for the loads; the registers pass through the wait, so that nothing reads
+// them before it.
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                   "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]),
+                   "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]),
+                   "+r"(r[30]), "+r"(r[31])::"memory");
+}
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64])
+{
+    uint32_t a[32], b[32];
+    tmem_ld32_issue(taddr, a);
+    tmem_ld32_issue(taddr + 32, b);
+    tmem_wait(a);
+    tmem_wait(b);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        v[i] = __uint_as_float(a[i]);
+        v[32 + i] = __uint_as_float(b[i]);
+    }
+}
+
+// 16 consecutive TMEM columns of this thread's lane <- r; tmem_wait_st before they are read.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n" ::"r"(
+            taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
@@ -365,56 +408,91 @@ __device__ __forceinline__ uint32_t pack_bf16_relu(float a, float b)
 
 constexpr int MT = 128;                      // cells per tile (MMA M)
 constexpr int BX = 32, BY = 4;               // tile = 32 x 4 cells of one plane
-constexpr int HX = BX + 8, HY = BY + 4, HZ = 5;   // staged block: x halo 4 (16-byte chunks), y, z halo 2
-constexpr int CPR = HX / 4;                         // 16-byte chunks per staged row
-constexpr int A1_BYTES = MT * KP1 * 2, A2_BYTES = MT * NH * 2;
-constexpr int W1_BYTES = NH * KP1 * 2, W2_BYTES = NH * NH * 2;
+constexpr int HX = 64, HY = BY + 4, HZ = 5;   // staged block: x halo 4 (16-byte chunks), y, z halo 2
+static_assert(BX == 32 && HY == 8 && MT == 128, "the staging threads' shares");
+constexpr int KS = KP1 - NH;                                     // K columns 64..79, staged in shared memory
+constexpr int A_BYTES = MT * KS * 2, W_BYTES = NH * KP1 * 2;   // operand images, K = 80 in both layers
 constexpr int BLK_FLOATS = HX * HY * HZ;
-// layout of the dynamic shared memory (bytes); about 54 KB, so four CTAs fit on
-// an SM and take all 512 of its tensor-memory columns.  The layer-2 operand A2
-// reuses A1's space: layer 1's MMA has finished reading A1 (its commit was
-// waited for) before epilogue 1 writes A2, and layer 2's MMA has finished
-// before the next tile's features are written to A1.
-constexpr int CTAS_PER_SM = 4;
-static_assert(CTAS_PER_SM * 128 <= 512, "tensor-memory columns of the resident CTAs");
-static_assert(A2_BYTES <= A1_BYTES, "A2 fits in A1's space");
-constexpr int S_A1 = 0, S_A2 = S_A1, S_W1 = S_A1 + A1_BYTES, S_W2 = S_W1 + W1_BYTES;
-constexpr int S_F = S_W2 + W2_BYTES;                          // FP32: b1, b2, w3, b3
 constexpr int STAGE_FLOATS = BLK_FLOATS + 3 * MT;              // Phi block + the tile's three u components
-constexpr int S_BLK = S_F + 4 * (3 * NH + 4);                  // two stages (double buffer)
-constexpr int S_BAR = S_BLK + 2 * 4 * STAGE_FLOATS;
-constexpr int S_TM = S_BAR + 16;
+// One CTA per SM of WGS warpgroups that share the weights; each warpgroup works
+// on tiles of its own (its operands, staging buffers, mbarrier, 96 TMEM columns
+// and named barrier), so that one's gathers and epilogues run under another's
+// tensor-core and copy latencies.
+//  - A's columns 0 to 63 go from registers to tensor memory (BF16 pairs, one row per
+//    lane) and are read there by the MMAs of both layers; only columns 64 to 79 pass
+//    through shared memory, once.
+//  - The biases enter through the GEMMs: K is padded from 67 to 80 anyway, columns
+//    67 to 69 are 1, and the weight images hold each bias there as three BF16
+//    parts that add up to its 24 bits.  Layer 2 overwrites columns 0 to 63 and leaves
+//    those behind them as they are (its weights for columns 64 to 66 are zero).
+//  - Layer 2 accumulates into the TMEM columns of layer 1, which the epilogue
+//    between them has read.
+//  - Rows of the staged block are 64 floats apart: a cell's bank depends on x alone,
+//    so neighbours that step to different rows do not collide.
+// What bounds it: instruction issue (about 60% of the cycles) with waits at the
+// barriers of a tile's two GEMMs; registers allow no sixth warpgroup (80 each spill,
+// 786 us).  Measured, 256^3: 825 us with four CTAs of one warpgroup and biases added
+// from shared memory; 688 with five warpgroups in one CTA, 666 with 64 accumulators
+// per TMEM read, 628 with A in tensor memory, 571 with whole lines per copy
+// instruction and no divisions in the staging, 559 with rows 64 floats apart.
+// Blocks staged two tiles ahead and one barrier less per tile took 568.
+constexpr int WGS = 5, NT_STEP = WGS * MT, TM_COLS = 512, TM_WG = NH + NH / 2;   // D, then A's columns 0..63
+static_assert(WGS * TM_WG <= TM_COLS, "tensor-memory columns of the warpgroups");
+constexpr int S_A = 0, S_W1 = S_A + WGS * A_BYTES, S_W2 = S_W1 + W_BYTES;   // operands on 128-byte boundaries
+constexpr int S_BLK = S_W2 + W_BYTES;                         // two stages per warpgroup
+constexpr int S_F = S_BLK + WGS * 2 * 4 * STAGE_FLOATS;       // w3, b3 in FP32
+constexpr int S_BAR = S_F + 4 * (NH + 4);
+constexpr int S_TM = S_BAR + (8 * WGS + 15) / 16 * 16;
 constexpr int SMEM_BYTES = S_TM + 16;
-// a fifth resident CTA would wait forever for tensor-memory columns; its shared
+static_assert(A_BYTES % 128 == 0 && W_BYTES % 128 == 0 && S_F % 16 == 0, "alignment");
+// a second resident CTA would wait forever for tensor-memory columns; its shared
 // memory (with the 1 KB per-CTA reserve) cannot fit in the SM's 228 KB
-static_assert((CTAS_PER_SM + 1) * (SMEM_BYTES + 1024) > 228 * 1024, "at most CTAS_PER_SM resident CTAs");
+static_assert(2 * (SMEM_BYTES + 1024) > 228 * 1024 && SMEM_BYTES <= 227 * 1024, "one resident CTA");
 
-// One learned step over the grid; persistent CTAs of 128 threads (4 warps),
-// one cell per thread per tile.  wb points at the BF16 operand images of W1
-// and W2 (already in the core-matrix layout) followed by b1, b2, w3, b3 in FP32.
-__global__ void __launch_bounds__(MT) k_learned_step(const float *__restrict__ phi, float *__restrict__ out,
-                                                     const float *__restrict__ vel, int nx, int ny, int nz,
-                                                     float sx, float sy, float sz,
-                                                     const unsigned char *__restrict__ wb, unsigned *status)
+// The barrier of one warpgroup, and the same with an OR over its threads.
+__device__ __forceinline__ void wg_sync(int g) { asm volatile("barrier.cta.sync %0, 128;\n" ::"r"(g + 1) : "memory"); }
+__device__ __forceinline__ bool wg_or(int g, bool v)
+{
+    unsigned r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.or.pred q, %2, 128, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}\n"
+        : "=r"(r)
+        : "r"((unsigned)v), "r"(g + 1)
+        : "memory");
+    return r != 0;
+}
+
+// One learned step over the grid; one cell per thread per tile.  wb points at
+// the BF16 operand images of W1 and W2 (already in the core-matrix layout, biases
+// included) followed by w3, b3 in FP32.
+__global__ void __launch_bounds__(NT_STEP, 1)
+k_learned_step(const float *__restrict__ phi, float *__restrict__ out, const float *__restrict__ vel, int nx, int ny,
+               int nz, float sx, float sy, float sz, const unsigned char *__restrict__ wb, unsigned *status)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    const int tid = threadIdx.x, warp = tid >> 5;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + S_BAR);
+    const int wg = threadIdx.x >> 7, tid = threadIdx.x & (MT - 1), warp = tid >> 5;   // within the warpgroup
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + S_BAR) + wg;
     uint32_t *tm_slot = reinterpret_cast<uint32_t *>(smem + S_TM);
     float *fw = reinterpret_cast<float *>(smem + S_F);
-    float *blk = reinterpret_cast<float *>(smem + S_BLK);
+    float *blk = reinterpret_cast<float *>(smem + S_BLK) + wg * 2 * STAGE_FLOATS;
+    unsigned char *A = smem + S_A + wg * A_BYTES;
     const int64_t plane = (int64_t)nx * ny, ncell = plane * nz;
 
     // weights once per CTA (operand images are copied verbatim)
     {
         const uint4 *src = reinterpret_cast<const uint4 *>(wb);
         uint4 *dst = reinterpret_cast<uint4 *>(smem + S_W1);
-        for (int i = tid; i < (W1_BYTES + W2_BYTES) / 16; i += MT) dst[i] = src[i];
-        const float *fsrc = reinterpret_cast<const float *>(wb + W1_BYTES + W2_BYTES);
-        for (int i = tid; i < 3 * NH + 1; i += MT) fw[i] = fsrc[i];
+        for (int i = threadIdx.x; i < 2 * W_BYTES / 16; i += NT_STEP) dst[i] = src[i];
+        const float *fsrc = reinterpret_cast<const float *>(wb + 2 * W_BYTES);
+        for (int i = threadIdx.x; i < NH + 1; i += NT_STEP) fw[i] = fsrc[i];
+        *reinterpret_cast<uint4 *>(A + core_off(tid, 1, MT / 8)) = make_uint4(0u, 0u, 0u, 0u);   // columns 72..79
     }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;\n" ::"r"(smem_u32(tm_slot)));
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tm_slot)),
+                     "n"(TM_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
     }
     if (tid == 0) mbar_init1(bar);
@@ -422,53 +500,86 @@ __global__ void __launch_bounds__(MT) k_learned_step(const float *__restrict__ p
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tm_slot;
-    const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+    const uint32_t tmem = *tm_slot + wg * TM_WG, tmem_a = tmem + NH;
+    const uint32_t lanes = (uint32_t)(warp * 32) << 16;
     const uint32_t idesc = instr_desc(MT, NH);
-    const uint32_t a1 = smem_u32(smem + S_A1), a2 = smem_u32(smem + S_A2);
-    const uint32_t w1 = smem_u32(smem + S_W1), w2 = smem_u32(smem + S_W2);
+    const uint32_t a0 = smem_u32(A), w1 = smem_u32(smem + S_W1), w2 = smem_u32(smem + S_W2);
     unsigned phase = 0;
     bool timeout = false;
 
+    // tile (tx, ty, z) of this warpgroup, and the step to its next one
     const int tiles_x = nx / BX, tiles_y = ny / BY;
-    const int64_t ntiles = (int64_t)tiles_x * tiles_y * nz;
-    // the Phi block x in [x0-2, x0+34), y in [y0-2, y0+6), z in [z-2, z+3) and
-    // the tile's velocity, staged with 4-byte cp.async one tile ahead
-    auto issue_block = [&](int64_t tt, int b) {
-        const int tx_ = (int)(tt % tiles_x);
-        const int ty_ = (int)((tt / tiles_x) % tiles_y);
-        const int z_ = (int)(tt / ((int64_t)tiles_x * tiles_y));
-        float *dst = blk + b * STAGE_FLOATS;
-        // x in [x0-4, x0+36) in 16-byte chunks: nx is a multiple of 32, so a
-        // chunk never straddles the periodic seam and every source is aligned
-        for (int i = tid; i < BLK_FLOATS / 4; i += MT) {
-            const int cx4 = i % CPR, row = i / CPR, by = row % HY, bz = row / HY;
-            int gx = tx_ * BX - 4 + 4 * cx4, gy = ty_ * BY - 2 + by, gz = z_ - 2 + bz;   // at most one period away
-            gx += gx < 0 ? nx : (gx >= nx ? -nx : 0);
-            gy += gy < 0 ? ny : (gy >= ny ? -ny : 0);
-            gz += gz < 0 ? nz : (gz >= nz ? -nz : 0);
-            cp_async16(dst + 4 * i, phi + (int64_t)gz * plane + (int64_t)gy * nx + gx);
+    const int64_t ntiles = (int64_t)tiles_x * tiles_y * nz, hop = (int64_t)gridDim.x * WGS;
+    const int64_t first = (int64_t)blockIdx.x * WGS + wg;
+    const int hx = (int)(hop % tiles_x), hy = (int)(hop / tiles_x % tiles_y), hz = (int)(hop / ((int64_t)tiles_x * tiles_y));
+    int tx = (int)(first % tiles_x), ty = (int)(first / tiles_x % tiles_y), z = (int)(first / ((int64_t)tiles_x * tiles_y));
+    auto advance = [&](int &x, int &y, int &zz) {
+        x += hx;
+        y += hy;
+        zz += hz;
+        if (x >= tiles_x) {
+            x -= tiles_x;
+            ++y;
         }
-        const int64_t cell_ = (int64_t)z_ * plane + (int64_t)(ty_ * BY + tid / BX) * nx + tx_ * BX + tid % BX;
-        cp_async4(dst + BLK_FLOATS + tid, vel + cell_);
-        cp_async4(dst + BLK_FLOATS + MT + tid, vel + ncell + cell_);
-        cp_async4(dst + BLK_FLOATS + 2 * MT + tid, vel + 2 * ncell + cell_);
+        if (y >= tiles_y) {
+            y -= tiles_y;
+            ++zz;
+        }
+    };
+    // the Phi block x in [x0-4, x0+36), y in [y0-2, y0+6), z in [z-2, z+3) and
+    // the tile's velocity, staged with cp.async one tile ahead.  nx is a multiple of
+    // 32, so a 16-byte chunk never straddles the periodic seam and every source is
+    // aligned.  Chunk c of the 32 inner cells of rows (y, z) = (r, q), (r, q + 2),
+    // (r, q + 4): eight threads read a whole line of a row; then the outer chunks,
+    // two per row, by the first 80 threads.
+    auto issue_block = [&](int tx_, int ty_, int z_, int b) {
+        float *dst = blk + b * STAGE_FLOATS;
+        auto wrapped = [](int v, int n) { return v + (v < 0 ? n : (v >= n ? -n : 0)); };   // at most one period away
+        const int c = tid & 7, r = (tid >> 3) & 7, q = tid >> 6;
+        const float *src = phi + (int64_t)wrapped(ty_ * BY - 2 + r, ny) * nx + tx_ * BX + 4 * c;
+        float *d = dst + (q * HY + r) * HX + 4 + 4 * c;
+#pragma unroll
+        for (int k = 0; k < HZ; k += 2)
+            if (q + k < HZ) cp_async16(d + k * HY * HX, src + wrapped(z_ - 2 + q + k, nz) * plane);
+        if (tid < 2 * HY * HZ) {
+            const int er = (tid >> 1) & 7, ez = tid >> 4, ex = (tid & 1) * (BX + 4);
+            cp_async16(dst + (ez * HY + er) * HX + ex, phi + wrapped(z_ - 2 + ez, nz) * plane +
+                                                           (int64_t)wrapped(ty_ * BY - 2 + er, ny) * nx +
+                                                           wrapped(tx_ * BX - 4 + ex, nx));
+        }
+        const float *v = vel + (z_ * plane + (int64_t)(ty_ * BY + tid / BX) * nx + tx_ * BX + tid % BX);
+        cp_async4(dst + BLK_FLOATS + tid, v);
+        cp_async4(dst + BLK_FLOATS + MT + tid, v + ncell);
+        cp_async4(dst + BLK_FLOATS + 2 * MT + tid, v + 2 * ncell);
         cp_async_commit();
     };
-    if ((int64_t)blockIdx.x < ntiles) issue_block(blockIdx.x, 0);
+    // D = A (128 x 80) * W^T, both operands K-major, issued by one thread: columns
+    // 64..79 of A first (shared memory), then 0..63 (tensor memory)
+    auto gemm = [&](uint32_t w) {
+        if (tid == 0) {
+            auto db = [&](int k) { return smem_desc(w + k * 2 * (NH / 8) * 128, (NH / 8) * 128, 128); };
+            mma_bf16(tmem, smem_desc(a0, (MT / 8) * 128, 128), db(NH / 16), idesc, 0);
+#pragma unroll
+            for (int k = 0; k < NH / 16; ++k) mma_bf16_ta(tmem, tmem_a + k * 8, db(k), idesc, 1);
+            mma_commit(bar);
+        }
+        if (!mbar_wait_bounded(bar, phase)) timeout = true;
+        phase ^= 1u;
+        tc_fence_after();
+    };
+    if (first < ntiles) issue_block(tx, ty, z, 0);
     int it = 0;
-    for (int64_t t = blockIdx.x; t < ntiles && !timeout; t += gridDim.x, ++it) {
-        const int tx = (int)(t % tiles_x);
-        const int ty = (int)((t / tiles_x) % tiles_y);
-        const int z = (int)(t / ((int64_t)tiles_x * tiles_y));
-        const int x0 = tx * BX, y0 = ty * BY;
+    for (int64_t t = first; t < ntiles; t += hop, ++it) {
+        const int x0 = tx * BX, y0 = ty * BY, z0 = z;
         const float *sb = blk + (it & 1) * STAGE_FLOATS;
         cp_async_wait_all();
-        __syncthreads();
-        if (t + gridDim.x < ntiles) issue_block(t + gridDim.x, (it & 1) ^ 1);
-        // ---- features of this thread's cell -> row tid of A1 (BF16)
+        timeout = wg_or(wg, timeout);   // the block is there, and every warp is done with the tile before
+        if (timeout) break;
+        advance(tx, ty, z);
+        if (t + hop < ntiles) issue_block(tx, ty, z, (it & 1) ^ 1);
+        // ---- features of this thread's cell -> row tid of A (BF16)
         const int cxl = tid % BX, cyl = tid / BX;
-        const int64_t cell = (int64_t)z * plane + (int64_t)(y0 + cyl) * nx + x0 + cxl;
+        const int64_t cell = (int64_t)z0 * plane + (int64_t)(y0 + cyl) * nx + x0 + cxl;
         const float cx = sb[BLK_FLOATS + tid] * sx, cy = sb[BLK_FLOATS + MT + tid] * sy,
                     cz = sb[BLK_FLOATS + 2 * MT + tid] * sz;
         if (fabsf(cx) > 1.f || fabsf(cy) > 1.f || fabsf(cz) > 1.f) atomicOr(status, 1u);
@@ -476,111 +587,67 @@ __global__ void __launch_bounds__(MT) k_learned_step(const float *__restrict__ p
                     ccz = fminf(fmaxf(cz, -1.f), 1.f);
         auto at = [&](int xx, int yy, int zz) {
             // xx, yy, zz are global indices within 2 cells of the cell
-            return sb[((zz - z + 2) * HY + (yy - y0 + 2)) * HX + (xx - x0 + 4)];
+            return sb[((zz - z0 + 2) * HY + (yy - y0 + 2)) * HX + (xx - x0 + 4)];
         };
         float feat[NIN], m, s;
-        cell_features(at, x0 + cxl, y0 + cyl, z, ccx, ccy, ccz, feat, m, s);
-        {
-            unsigned char *A = smem + S_A1;
+        cell_features(at, x0 + cxl, y0 + cyl, z0, ccx, ccy, ccz, feat, m, s);
 #pragma unroll
-            for (int kg = 0; kg < KP1 / 8; ++kg) {
-                float q[8];
+        for (int h = 0; h < 2; ++h) {
+            uint32_t q[16];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) q[e] = (kg * 8 + e < NIN) ? feat[kg * 8 + e] : 0.f;
-                uint4 pk = make_uint4(pack_bf16(q[0], q[1]), pack_bf16(q[2], q[3]), pack_bf16(q[4], q[5]),
-                                      pack_bf16(q[6], q[7]));
-                *reinterpret_cast<uint4 *>(A + core_off(tid, kg, MT / 8)) = pk;
-            }
+            for (int k = 0; k < 16; ++k) q[k] = pack_bf16(feat[32 * h + 2 * k], feat[32 * h + 2 * k + 1]);
+            tmem_st16(tmem_a + lanes + 16 * h, q);
         }
+        // columns 67..69 are the biases' ones
+        *reinterpret_cast<uint4 *>(A + core_off(tid, 0, MT / 8)) =
+            make_uint4(pack_bf16(feat[64], feat[65]), pack_bf16(feat[66], 1.f), pack_bf16(1.f, 1.f), 0u);
+        tmem_wait_st();
         fence_async_smem();
         tc_fence_before();
-        __syncthreads();
+        wg_sync(wg);
         tc_fence_after();
-        // ---- layer 1 on the tensor cores: D[0:64) = A1 (128 x 80) * W1^T
-        if (tid == 0) {
-#pragma unroll
-            for (int k = 0; k < KP1 / 16; ++k) {
-                const uint64_t da = smem_desc(a1 + k * 2 * (MT / 8) * 128, (MT / 8) * 128, 128);
-                const uint64_t db = smem_desc(w1 + k * 2 * (NH / 8) * 128, (NH / 8) * 128, 128);
-                mma_bf16(tmem, da, db, idesc, k > 0);
-            }
-            mma_commit(bar);
-        }
-        if (!mbar_wait_bounded(bar, phase)) timeout = true;
-        phase ^= 1u;
-        tc_fence_after();
-        // ---- epilogue 1: bias, ReLU, BF16 -> A2
+        gemm(w1);
+        // ---- epilogue 1: ReLU, BF16 -> columns 0..63 of A
         {
-            unsigned char *A = smem + S_A2;
+            float v[NH];
+            tmem_ld64(tmem + lanes, v);
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                float v[32];
-                tmem_ld32(lane_base + half * 32, v);
-                const float4 *b1v = reinterpret_cast<const float4 *>(fw + half * 32);
+            for (int h = 0; h < 2; ++h) {
+                uint32_t q[16];
 #pragma unroll
-                for (int kg = 0; kg < 4; ++kg) {
-                    const float4 ba = b1v[2 * kg], bb = b1v[2 * kg + 1];
-                    const float2 bias[4] = {make_float2(ba.x, ba.y), make_float2(ba.z, ba.w), make_float2(bb.x, bb.y),
-                                            make_float2(bb.z, bb.w)};
-                    uint32_t w[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {   // bias on pairs (FADD2), ReLU folded into the conversion
-                        const float2 h = __fadd2_rn(make_float2(v[kg * 8 + 2 * e], v[kg * 8 + 2 * e + 1]), bias[e]);
-                        w[e] = pack_bf16_relu(h.x, h.y);
-                    }
-                    const uint4 pk = make_uint4(w[0], w[1], w[2], w[3]);
-                    *reinterpret_cast<uint4 *>(A + core_off(tid, half * 4 + kg, MT / 8)) = pk;
-                }
+                for (int k = 0; k < 16; ++k)   // ReLU folded into the conversion
+                    q[k] = pack_bf16_relu(v[32 * h + 2 * k], v[32 * h + 2 * k + 1]);
+                tmem_st16(tmem_a + lanes + 16 * h, q);
             }
+            tmem_wait_st();
         }
-        fence_async_smem();
         tc_fence_before();
-        __syncthreads();
+        wg_sync(wg);
         tc_fence_after();
-        // ---- layer 2: D[64:128) = A2 (128 x 64) * W2^T
-        if (tid == 0) {
+        gemm(w2);
+        // ---- epilogue 2: ReLU, output layer, Phi_new = m + s y
+        float2 ya01 = make_float2(fw[NH], 0.f), ya23 = make_float2(0.f, 0.f);   // four accumulation chains
+        {
+            float v[NH];
+            tmem_ld64(tmem + lanes, v);
+            const float4 *w3v = reinterpret_cast<const float4 *>(fw);
 #pragma unroll
-            for (int k = 0; k < NH / 16; ++k) {
-                const uint64_t da = smem_desc(a2 + k * 2 * (MT / 8) * 128, (MT / 8) * 128, 128);
-                const uint64_t db = smem_desc(w2 + k * 2 * (NH / 8) * 128, (NH / 8) * 128, 128);
-                mma_bf16(tmem + NH, da, db, idesc, k > 0);
-            }
-            mma_commit(bar);
-        }
-        if (!mbar_wait_bounded(bar, phase)) timeout = true;
-        phase ^= 1u;
-        tc_fence_after();
-        // ---- epilogue 2: bias, ReLU, output layer, Phi_new = m + s y
-        float2 ya01 = make_float2(fw[3 * NH], 0.f), ya23 = make_float2(0.f, 0.f);   // four accumulation chains
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            float v[32];
-            tmem_ld32(lane_base + NH + half * 32, v);
-            const float4 *b2v = reinterpret_cast<const float4 *>(fw + NH + half * 32);
-            const float4 *w3v = reinterpret_cast<const float4 *>(fw + 2 * NH + half * 32);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                // bias and weight pairs: packed FADD2 / FFMA2, ReLU per lane
-                const float4 bb = b2v[q], ww = w3v[q];
-                float2 h01 = __fadd2_rn(make_float2(v[4 * q], v[4 * q + 1]), make_float2(bb.x, bb.y));
-                float2 h23 = __fadd2_rn(make_float2(v[4 * q + 2], v[4 * q + 3]), make_float2(bb.z, bb.w));
-                h01 = make_float2(fmaxf(h01.x, 0.f), fmaxf(h01.y, 0.f));
-                h23 = make_float2(fmaxf(h23.x, 0.f), fmaxf(h23.y, 0.f));
+            for (int q = 0; q < NH / 4; ++q) {
+                const float4 ww = w3v[q];
+                const float2 h01 = make_float2(fmaxf(v[4 * q], 0.f), fmaxf(v[4 * q + 1], 0.f));
+                const float2 h23 = make_float2(fmaxf(v[4 * q + 2], 0.f), fmaxf(v[4 * q + 3], 0.f));
                 ya01 = __ffma2_rn(h01, make_float2(ww.x, ww.y), ya01);
                 ya23 = __ffma2_rn(h23, make_float2(ww.z, ww.w), ya23);
             }
         }
         const float y = (ya01.x + ya01.y) + (ya23.x + ya23.y);
         out[cell] = m + s * y;
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        timeout = __syncthreads_or(timeout);
     }
     cp_async_wait_all();   // a block prefetched for a tile that was not run
-    if (timeout && tid == 0) atomicOr(status, 2u);
+    if (timeout) atomicOr(status, 2u);
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;\n" ::"r"(tmem));
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(*tm_slot), "n"(TM_COLS));
 }
 
 // Failure-detection self-test: waits on an mbarrier that no thread or copy
@@ -609,29 +676,35 @@ __global__ void k_wait_selftest(unsigned polls, unsigned *status, unsigned *gave
     }
 }
 
-// FP32 parameters -> the inference weight image: W1 (64 x 80, K zero-padded)
-// and W2 (64 x 64) as BF16 K-major core matrices, then b1, b2, w3, b3 in FP32.
+// Element (n, k) of a layer's weight image: its weight for k < nin, for k = 67 to
+// 69 the three BF16 parts of its bias (cut off, not rounded, so that they add up to
+// the FP32 value; a bias that is not finite stays whole), else 0.
+__device__ __forceinline__ float image_value(const float *w, const float *b, int nin, int n, int k)
+{
+    if (k < nin) return w[n * nin + k];
+    if (k < NIN || k >= NIN + 3) return 0.f;
+    const float v = b[n];
+    if (!isfinite(v)) return k == NIN ? v : 0.f;
+    const float hi = __uint_as_float(__float_as_uint(v) & 0xffff0000u), r = v - hi;
+    const float mid = __uint_as_float(__float_as_uint(r) & 0xffff0000u);
+    return k == NIN ? hi : (k == NIN + 1 ? mid : r - mid);
+}
+
+// FP32 parameters -> the inference weight image: W1 and W2 (64 x 80 each, biases
+// in columns 67 to 69) as BF16 K-major core matrices, then w3, b3 in FP32.
 __global__ void k_pack(const float *__restrict__ params, unsigned char *__restrict__ wb)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     __nv_bfloat16 *w1 = reinterpret_cast<__nv_bfloat16 *>(wb);
-    __nv_bfloat16 *w2 = reinterpret_cast<__nv_bfloat16 *>(wb + W1_BYTES);
-    float *f = reinterpret_cast<float *>(wb + W1_BYTES + W2_BYTES);
+    __nv_bfloat16 *w2 = reinterpret_cast<__nv_bfloat16 *>(wb + W_BYTES);
+    float *f = reinterpret_cast<float *>(wb + 2 * W_BYTES);
     if (i < NH * KP1) {
-        const int n = i / KP1, k = i % KP1;
-        const float v = k < NIN ? params[O_W1 + n * NIN + k] : 0.f;
-        w1[core_off(n, k / 8, NH / 8) / 2 + k % 8] = __float2bfloat16_rn(v);
+        const int n = i / KP1, k = i % KP1, o = core_off(n, k / 8, NH / 8) / 2 + k % 8;
+        w1[o] = __float2bfloat16_rn(image_value(params + O_W1, params + O_B1, NIN, n, k));
+        w2[o] = __float2bfloat16_rn(image_value(params + O_W2, params + O_B2, NH, n, k));
     }
-    if (i < NH * NH) {
-        const int n = i / NH, k = i % NH;
-        w2[core_off(n, k / 8, NH / 8) / 2 + k % 8] = __float2bfloat16_rn(params[O_W2 + n * NH + k]);
-    }
-    if (i < NH) {
-        f[i] = params[O_B1 + i];
-        f[NH + i] = params[O_B2 + i];
-        f[2 * NH + i] = params[O_W3 + i];
-    }
-    if (i == 0) f[3 * NH] = params[O_B3];
+    if (i < NH) f[i] = params[O_W3 + i];
+    if (i == 0) f[NH] = params[O_B3];
 }
 
 }  // namespace lrn
@@ -683,7 +756,7 @@ int sl_corrector_create(sl_corrector **out, uint64_t seed)
     sl_corrector *c = new (std::nothrow) sl_corrector();
     if (!c) return lfail(SL_ERR_NOMEM, "host allocation");
     c->device = ctx->device;
-    const size_t wbytes = W1_BYTES + W2_BYTES + 4 * (3 * NH + 4);
+    const size_t wbytes = 2 * W_BYTES + 4 * (NH + 4);
     void *p = nullptr;
     if (cudaMalloc(&p, 4 * (size_t)NPARAM * 4 + 256 + wbytes) != cudaSuccess) {
         delete c;
@@ -857,15 +930,15 @@ int sl_advect_learned(sl_corrector *c, void *out, const void *in, const void *ve
         if (!smem_set[ctx->device]) {
             if (cudaFuncSetAttribute(k_learned_step, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess)
                 return cudaErrorInvalidValue;
-            // all of the SM's unified L1 / shared memory as shared, so four CTAs fit
+            // all of the SM's unified L1 / shared memory as shared
             if (cudaFuncSetAttribute(k_learned_step, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
                 return cudaErrorInvalidValue;
             smem_set[ctx->device] = 1;
         }
         const int64_t tiles = (dims[0] / BX) * (dims[1] / BY) * dims[2];
-        int grid = ctx->num_sms * CTAS_PER_SM;   // never more: each CTA holds 128 TMEM columns
-        if (grid > tiles) grid = (int)tiles;
-        k_learned_step<<<grid, MT, SMEM_BYTES, st>>>(
+        const int64_t ctas = (tiles + WGS - 1) / WGS;
+        const int grid = ctas < ctx->num_sms ? (int)ctas : ctx->num_sms;   // one per SM: each holds its TMEM
+        k_learned_step<<<grid, NT_STEP, SMEM_BYTES, st>>>(
             static_cast<const float *>(in), static_cast<float *>(dst), static_cast<const float *>(vel), (int)dims[0],
             (int)dims[1], (int)dims[2], (float)(dt / spacing[0]), (float)(dt / spacing[1]), (float)(dt / spacing[2]),
             c->wb, ctx->status);

@@ -259,3 +259,64 @@ def test_corrupted_weights_fall_back_to_the_plain_step(bad):
         assert torch.isfinite(out).all()
     finally:
         sl.sl_corrector_destroy(c)
+
+
+# tiles of 32 x 4 cells: fewer than the warpgroups of one CTA, one more than they are, a remainder of a
+# row of tiles, and two rounds of every CTA with a remainder
+@pytest.mark.parametrize("dims", [(32, 4, 3), (32, 8, 3), (96, 12, 5), (64, 16, 191)])
+def test_learned_step_on_every_cell_and_all_bits_of_the_biases(dims):
+    """With W1 = 0 the network's output is the same for every cell and rounds nothing
+    but its sums: b1 is rounded to BF16 as layer 2's operand (each lies 2^-12 off a
+    BF16 value, far from a tie), W2 is BF16, b2, w3 and b3 use all 24 bits.  67 products added in
+    FP32 with truncation are within 67 2^-23 < 2^-16 of the sum of their magnitudes; m and s come from
+    FP32 interpolation of values of magnitude up to max|Phi| (a dozen roundings)."""
+    nx, ny, nz = dims
+    rng = np.random.default_rng(nx + nz)
+    phi = torch.from_numpy(rng.standard_normal((nz, ny, nx))).float()
+    sp, dt = [0.1, 0.2, 0.15], 0.05
+    vel = torch.from_numpy(np.stack([rng.uniform(-0.95, 0.95, (nz, ny, nx)) * sp[d] / dt for d in range(3)])).float()
+    b1 = (bf16(rng.standard_normal(NH)) * (1 + 2.0 ** -12)).astype(np.float32)
+    W2 = bf16(rng.standard_normal((NH, NH)) * 0.2)
+    b2, w3, b3 = [rng.standard_normal(n).astype(np.float32) for n in (NH, NH, 1)]
+    params = np.concatenate([np.zeros(NH * NIN), b1, W2.ravel(), b2, w3, b3]).astype(np.float32)
+    c = sl.sl_corrector_create(5)
+    try:
+        sl.sl_corrector_set_params(c, params)
+        out = torch.empty((nz, ny, nx), device=DEV)
+        used, _ = sl.sl_advect_learned(c, out, phi.to(DEV), vel.to(DEV), 3, list(dims), sp, dt)
+        torch.cuda.synchronize()
+        assert used == 0
+    finally:
+        sl.sl_corrector_destroy(c)
+    h1 = np.maximum(bf16(b1), 0.0)
+    h2 = np.maximum(W2 @ h1 + b2.astype(np.float64), 0.0)
+    y = float(h2 @ w3.astype(np.float64)) + float(b3[0])
+    mag = float(np.abs(w3).astype(np.float64) @ (np.abs(W2) @ h1 + np.abs(b2))) + abs(float(b3[0]))
+    # departure points as the kernel rounds them (FP32), the rest in FP64
+    idx = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")[::-1]   # x, y, z
+    base, frac = [], []
+    for d in range(3):
+        cfl = vel[d].numpy() * np.float32(dt / sp[d])
+        X = idx[d].astype(np.float32) - cfl
+        b = np.minimum(np.floor(X).astype(np.int64), idx[d])
+        base.append(b)
+        frac.append((X - b.astype(np.float32)).astype(np.float64))
+    p64 = phi.numpy().astype(np.float64)
+
+    def at(a, b, k):
+        return p64[(base[2] + k) % nz, (base[1] + b) % ny, (base[0] + a) % nx]
+
+    m = np.zeros((nz, ny, nx))
+    for a in range(2):
+        for b in range(2):
+            for k in range(2):
+                w = [(frac[d] if e else 1 - frac[d]) for d, e in enumerate((a, b, k))]
+                m += w[0] * w[1] * w[2] * at(a, b, k)
+    s = np.full((nz, ny, nx), 1e-30)
+    for a in range(-1, 3):
+        for b in range(-1, 3):
+            for k in range(-1, 3):
+                s = np.maximum(s, np.abs(at(a, b, k) - m))
+    err = np.abs(out.cpu().numpy() - (m + s * y))
+    bound = s * (2.0 ** -16 * mag) + 12 * 2.0 ** -23 * np.abs(p64).max() * (1 + 2 * abs(y))
+    assert (err <= bound).all(), (err / bound).max()
