@@ -37,9 +37,15 @@
 // tile, plane) pairs of all grids are numbered and every CTA takes one
 // contiguous, equal share, marching along z in each column tile.  Each plane
 // bundle (the field and velocity rows a plane needs, with their periodic halo)
-// is staged by the tensor-memory accelerator, one 2D box per array and row
-// band, issued by one thread and counted by the slot's mbarrier; three slots
-// are in flight.  One block barrier per plane in either order.
+// is staged by the tensor-memory accelerator, one 2D box per array (tiles at the
+// periodic seam in y: per array and row band), counted by the slot's mbarrier; three
+// slots are in flight.  One thread of each of four warps issues the boxes of one
+// array: the four warps sit on the SM's four schedulers.  Measured, 512^3, x,y,z /
+// z,y,x: 612 / 928 us with one thread issuing row bands (603 / 927 with one box per
+// array), 611 / 886 with two warps, 561 / 816 with four, 560 / 780 with four and one
+// box per array, 593 / 830 with four warps on two schedulers, 611 / 840 with eight
+// warps and row bands, 621 / 1299 with a warp of its own (registers: 96 a thread).
+// One block barrier per plane in either order.
 //   x,y,z: x sweep on the tile widened by the y halo (scalar runs of 8 in
 //          registers, into a double-buffered shared plane); y sweep on pairs
 //          of adjacent columns in packed f32x2 arithmetic, feeding per-column
@@ -435,7 +441,8 @@ __device__ __forceinline__ int wrapz(int p, int nz) { return ((p % nz) + nz) % n
 // ------------------------------------------------------------------ staging
 // Staged rows of 44 floats run from x0 - 4 to x0 + 40 (row stride 44 floats,
 // so the 16-byte blocks of runs in different rows fall on different banks).
-// Rows are copied in bands [y0 - 8, y0), [y0, y0 + 32) and [y0 + 32, y0 + 32
+// A tile away from the periodic seam in y takes one box of the rows it reads, from
+// y0 - 3 on.  At the seam rows are copied in bands [y0 - 8, y0), [y0, y0 + 32) and [y0 + 32, y0 + 32
 // + b): each band lies within [0, ny) after the periodic wrap (ny is a
 // multiple of 32) and starts on a 128-byte boundary in shared memory (8 rows
 // of 176 bytes = 11 x 128).  At the periodic seam in x (x0 == 0 or x0 + 32 ==
@@ -486,11 +493,11 @@ __device__ __forceinline__ void tma3(float *dst, const CUtensorMap *m, int x, in
 // Tensor maps of one instance: box shapes (width x rows) over the field
 // tensor [nz][ny][nx] (F) and the velocity tensor [3 nz][ny][nx] (V).
 enum {
-    M_F44_8, M_F44_32, M_F44_3, M_F40_4, M_F40_32, M_F40_3, M_F4_8, M_F4_32, M_F4_3,
+    M_F44_8, M_F44_32, M_F44_3, M_F40_4, M_F40_32, M_F40_3, M_F4_8, M_F4_32, M_F4_3, M_F44_38, M_F40_38, M_F4_38,
     M_V44_8, M_V44_32, M_V44_3, M_V40_4, M_V40_32, M_V40_3, M_V40_2, M_V4_8, M_V4_32, M_V4_3, M_V4_2,
-    M_V32_2, M_V32_32, NMAPS
+    M_V32_2, M_V32_32, M_V44_38, M_V40_38, M_V4_38, M_V40_36, M_V4_36, M_V32_36, NMAPS
 };
-constexpr int NFMAPS = M_F4_3 + 1;   // the field's maps come first
+constexpr int NFMAPS = M_F4_38 + 1;   // the field's maps come first
 struct FastMaps {
     CUtensorMap m[NMAPS];                          // field 0 and the velocity
     CUtensorMap fx[kFastFields - 1][NFMAPS];       // fields 1 .. nf-1
@@ -620,38 +627,60 @@ __device__ __forceinline__ void x_run(const float *pbase, const Blocks &pb, cons
 namespace xyz {
 constexpr int RX = 8, NXI = (TY + 6) * (TX / RX);    // 152 x-run items
 // slot layout (floats; every part starts on a 128-byte boundary): Phi and u_x
-// rows [-8, TY+3) at stride PW, u_y rows [-2, TY+2) and u_z rows [0, TY) at
-// stride TX, and the seam side buffers of Phi and u_x (rows [-8, TY+3), 4 wide)
+// rows [-8, TY+3) (one box: from row -3 on) at stride PW, u_y rows [-2, TY+2) and u_z
+// rows [0, TY) at stride TX, and the seam side buffers of Phi and u_x (the same rows, 4 wide)
 constexpr int O_PHI = 0, O_UX = 1920, O_UY = 3840, O_UZ = O_UY + (TY + 4) * TX, O_SP = O_UZ + TY * TX,
               O_SX = O_SP + 192, SLOT = O_SX + 192;
 static_assert(43 * PW <= 1920 && 43 * 4 <= 192 && SLOT % 32 == 0, "slot layout");
 constexpr int XW = 36;                                // x-swept row stride (bank-conflict-free stores)
 constexpr int SZ_X = (TY + 6) * XW;                   // one x-swept plane, rows [-3, TY+3)
 constexpr unsigned BYTES = 4u * (2 * 43 * PW + (TY + 4) * TX + TY * TX), BYTES_SEAM = 4u * 2 * 43 * 4;
+constexpr unsigned BYTES_IN = 4u * (2 * 38 * PW + (TY + 4) * TX + TY * TX), BYTES_IN_SEAM = 4u * 2 * 38 * 4;   // one box per array
 constexpr int tab_size(int ch) { return ch ? 38 * PW / ch : 0; }   // copied rows: whole shared rows
 template <int NS, int CH>
 constexpr size_t smem() { return sizeof(float) * (NS * SLOT + 2 * SZ_X + tab_size(CH)) + 128; }
 }  // namespace xyz
 
 // Stages the bundle of plane pz (reduced modulo nz) for the x,y,z order into
-// slot sb: Phi, u_x and u_y at pz, u_z at pz - 1 (one thread).
+// slot sb: Phi, u_x and u_y at pz, u_z at pz - 1.  Part `part` of the issuing threads'
+// four (one array each; part 0 arms the slot's mbarrier; a box that lands before that
+// is counted all the same, the phase ends with the arming arrival at the earliest).
 __device__ __forceinline__ void xyz_issue(float *sb, uint64_t *b, const CUtensorMap *fm, const CUtensorMap *m,
-                                          int x0, int y0, int nx, int ny, int nz, int pz, bool seam)
+                                          int x0, int y0, int nx, int ny, int nz, int pz, bool seam, bool yseam,
+                                          int part)
 {
     using namespace xyz;
     const int yt = y0 - 8 < 0 ? y0 - 8 + ny : y0 - 8, yb = y0 + TY >= ny ? y0 + TY - ny : y0 + TY;
     const int yt2 = y0 - 2 < 0 ? y0 - 2 + ny : y0 - 2;
     const int pz1 = pz == 0 ? nz - 1 : pz - 1;
     const int xs = x0 == 0 ? nx - 4 : 0;
-    bar_arm(b, BYTES + (seam ? BYTES_SEAM : 0u));
-    const Band3 fb{M_F44_8, M_F44_32, M_F44_3, M_F4_8, M_F4_32, M_F4_3, 3};
-    const Band3 vb{M_V44_8, M_V44_32, M_V44_3, M_V4_8, M_V4_32, M_V4_3, 3};
-    stage_rows(sb + O_PHI, sb + O_SP, fm, fb, x0, xs, yt, y0, yb, pz, seam, b);
-    stage_rows(sb + O_UX, sb + O_SX, m, vb, x0, xs, yt, y0, yb, pz, seam, b);
-    tma3(sb + O_UY, &m[M_V32_2], x0, yt2, nz + pz, b);
-    tma3(sb + O_UY + 2 * TX, &m[M_V32_32], x0, y0, nz + pz, b);
-    tma3(sb + O_UY + 34 * TX, &m[M_V32_2], x0, yb, nz + pz, b);
-    tma3(sb + O_UZ, &m[M_V32_32], x0, y0, 2 * nz + pz1, b);
+    if (!yseam) {   // one box per array, from row -3 (u_y: -2, u_z: 0) on
+        if (part == 0) {
+            bar_arm(b, BYTES_IN + (seam ? BYTES_IN_SEAM : 0u));
+            tma3(sb + O_PHI, &fm[M_F44_38], x0 - 4, y0 - 3, pz, b);
+            if (seam) tma3(sb + O_SP, &fm[M_F4_38], xs, y0 - 3, pz, b);
+        } else if (part == 1) {
+            tma3(sb + O_UX, &m[M_V44_38], x0 - 4, y0 - 3, pz, b);
+            if (seam) tma3(sb + O_SX, &m[M_V4_38], xs, y0 - 3, pz, b);
+        } else if (part == 2) {
+            tma3(sb + O_UY, &m[M_V32_36], x0, y0 - 2, nz + pz, b);
+        } else {
+            tma3(sb + O_UZ, &m[M_V32_32], x0, y0, 2 * nz + pz1, b);
+        }
+    } else if (part == 0) {
+        const Band3 fb{M_F44_8, M_F44_32, M_F44_3, M_F4_8, M_F4_32, M_F4_3, 3};
+        bar_arm(b, BYTES + (seam ? BYTES_SEAM : 0u));
+        stage_rows(sb + O_PHI, sb + O_SP, fm, fb, x0, xs, yt, y0, yb, pz, seam, b);
+    } else if (part == 1) {
+        const Band3 vb{M_V44_8, M_V44_32, M_V44_3, M_V4_8, M_V4_32, M_V4_3, 3};
+        stage_rows(sb + O_UX, sb + O_SX, m, vb, x0, xs, yt, y0, yb, pz, seam, b);
+    } else if (part == 2) {
+        tma3(sb + O_UY, &m[M_V32_2], x0, yt2, nz + pz, b);
+        tma3(sb + O_UY + 2 * TX, &m[M_V32_32], x0, y0, nz + pz, b);
+        tma3(sb + O_UY + 34 * TX, &m[M_V32_2], x0, yb, nz + pz, b);
+    } else {
+        tma3(sb + O_UZ, &m[M_V32_32], x0, y0, 2 * nz + pz1, b);
+    }
 }
 
 // The same bundle by copies of CH floats (all threads): Phi and u_x rows
@@ -732,7 +761,7 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
     const int yu = O_UY + yr * TX + 2 * cp;           // u_y of row yr - 2 (staged row y + 2)
     const int yx = yr * XW + 2 * cp;                  // x-swept row yr - 3 (row y + 3)
     const int zu = O_UZ + yr * TX + 2 * cp;           // u_z of row yr
-    constexpr int ISSUER = NT - 1;                    // idle in the x phase
+    const bool issuer = (tid & 31) == 31 && tid >= NT / 2;   // of array 7 - tid / 32
     __shared__ uint64_t bars[NS];
     if (tid == 0) {
         for (int k = 0; k < NS; ++k) bar_init(&bars[k], CH ? NT : 1);
@@ -740,9 +769,9 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
     }
     __syncthreads();
     unsigned par = 0;                     // bit k: parity of slot k's next completion
-    unsigned armed = 0;                   // issuer: slots armed and not seen complete
+    unsigned armed = 0;                   // issuers: slots with boxes issued and not seen complete
     // Poll budget of a wait.  Once a wait has given up, later waits poll once
-    // and the issuer stops issuing: the kernel runs to its end on stale shared
+    // and the issuers stop issuing: the kernel runs to its end on stale shared
     // data (every access stays in bounds, every thread meets every barrier).
     unsigned polls = kPolls;
     bool tmo = false;
@@ -761,8 +790,11 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
         const int pfirst = sg.z0 - 3, plast = sg.z1 + 2;
         const bool sl = CH == 0 && x0 == 0, sr = CH == 0 && x0 + TX == I.nx, seam = sl || sr;
         Blocks bp, bu;
-        bp.set(O_PHI + (xrow + 5) * PW, O_SP + 4 * (xrow + 5), xr, sl, sr);
-        bu.set(O_UX + (xrow + 5) * PW, O_SX + 4 * (xrow + 5), xr, sl, sr);
+        // the staged row -3: the first one, or behind the rest of the upper row band
+        const bool yseam = CH || y0 == 0 || y0 + TY == I.ny;
+        const int srow = xrow + (yseam ? 5 : 0);
+        bp.set(O_PHI + srow * PW, O_SP + 4 * srow, xr, sl, sr);
+        bu.set(O_UX + srow * PW, O_SX + 4 * srow, xr, sl, sr);
         float *const obase = (BATCH ? I.out : I.fout[fld]) + (int64_t)(y0 + yr) * I.nx + x0 + 2 * cp;
         const int onx = I.nx;
         auto issue = [&](int pz, int s) {
@@ -770,8 +802,9 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
                 if (!tmo)
                     xyz_copy<CH>(buf + s * SLOT, &bars[s], offs, tid, I.fin[fld], I.vel, I.ncell, pz * plane_n,
                                  (pz == 0 ? nz - 1 : pz - 1) * plane_n);
-            } else if (tid == ISSUER && !tmo) {
-                xyz_issue(buf + s * SLOT, &bars[s], fmaps, maps, x0, y0, I.nx, I.ny, nz, pz, seam);
+            } else if (issuer && !tmo) {
+                xyz_issue(buf + s * SLOT, &bars[s], fmaps, maps, x0, y0, I.nx, I.ny, nz, pz, seam, yseam,
+                          7 - (tid >> 5));
                 armed |= 1u << s;
             }
         };
@@ -808,7 +841,7 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
             if (!ok) {
                 polls = 1;
                 tmo = true;
-            } else if (tid == ISSUER) {
+            } else if (issuer) {
                 armed &= ~(1u << s);
             }
             par ^= 1u << s;
@@ -897,7 +930,7 @@ k_cec_xyz_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
     }
     if constexpr (CH)
         cp_async_wait_all();
-    else if (tid == ISSUER && armed)
+    else if (issuer && armed)
         drain<NS>(bars, armed, par);
     if (tmo) atomicOr(status, 2u);
     flag_cfl(status, bad);
@@ -912,7 +945,8 @@ constexpr int RY = 4, RX = 4;                         // a warp's y and x sweeps
 // slot layout (floats, 128-byte aligned parts): Phi(p) and u_z(p-1) rows
 // [-4, TY+3), u_y(p-3) rows [-4, TY+2), u_x(p-3) rows [0, TY), row r at
 // (r + 4) ZS (u_x: r ZS); the seam side buffers hold row r at 32 + 4 r
-// (rows from -8, so that the bands of 8, 32 and 2 or 3 rows are contiguous).
+// (rows from -8, so that the bands of 8, 32 and 2 or 3 rows are contiguous).  One
+// box per array puts its first row, -3 or -2, first in the array and its side buffer.
 // u_z and its side buffer lie DZ after Phi and its side buffer.
 constexpr int O_PHI = 0, O_SP = 1568, DZ = 1760, O_UZ = O_PHI + DZ, O_SZ = O_SP + DZ, O_UY = 3520, O_SY = 5056,
               O_UX = 5248, O_SX = 6528, SLOT = 6688;
@@ -922,6 +956,7 @@ static_assert(39 * ZS <= O_SP && O_SP + 192 <= DZ && O_SZ + 192 <= O_UY && O_UY 
 constexpr int SZ_Z = (TY + 6) * ZS;                   // one z-swept plane, rows [-3, TY+3)
 constexpr int SZ_Y = TY * ZS;                         // y-swept rows [0, TY)
 constexpr unsigned BYTES = 4u * (39 + 39 + 38 + 32) * ZS, BYTES_SEAM = 4u * 4 * (43 + 43 + 42 + 32);
+constexpr unsigned BYTES_IN = 4u * (38 + 38 + 36 + 32) * ZS, BYTES_IN_SEAM = 4u * 4 * (38 + 38 + 36 + 32);   // one box per array
 constexpr int tab_size(int ch) { return ch ? 38 * ZS / ch : 0; }
 template <int NS, int CH>
 constexpr size_t smem() { return sizeof(float) * (NS * SLOT + 2 * SZ_Z + SZ_Y + tab_size(CH)) + 128; }
@@ -961,9 +996,10 @@ __device__ __forceinline__ void stage40(float *dst, float *side, const CUtensorM
 }
 
 // Stages the bundle of plane pz (reduced modulo nz) for the z,y,x order into
-// slot sb: Phi at pz, u_z at pz - 1, u_y and u_x at pz - 3 (one thread).
+// slot sb: Phi at pz, u_z at pz - 1, u_y and u_x at pz - 3 (parts as above).
 __device__ __forceinline__ void zyx_issue(float *sb, uint64_t *b, const CUtensorMap *fm, const CUtensorMap *m,
-                                          int x0, int y0, int nx, int ny, int nz, int pz, bool seam)
+                                          int x0, int y0, int nx, int ny, int nz, int pz, bool seam, bool yseam,
+                                          int part)
 {
     using namespace zyx;
     const int yt4 = y0 - 4 < 0 ? y0 - 4 + ny : y0 - 4, yt8 = y0 - 8 < 0 ? y0 - 8 + ny : y0 - 8;
@@ -971,15 +1007,35 @@ __device__ __forceinline__ void zyx_issue(float *sb, uint64_t *b, const CUtensor
     const int pz1 = pz == 0 ? nz - 1 : pz - 1;
     const int pz3 = pz >= 3 ? pz - 3 : pz - 3 + nz;
     const int xs = x0 == 0 ? nx - 4 : 0;
-    bar_arm(b, BYTES + (seam ? BYTES_SEAM : 0u));
-    stage40(sb + O_PHI, sb + O_SP, fm, M_F40_4, M_F40_32, M_F40_3, M_F4_8, M_F4_32, M_F4_3, x0, xs, yt4, yt8, y0,
-            yb, pz, seam, b);
-    stage40(sb + O_UZ, sb + O_SZ, m, M_V40_4, M_V40_32, M_V40_3, M_V4_8, M_V4_32, M_V4_3, x0, xs, yt4, yt8, y0,
-            yb, 2 * nz + pz1, seam, b);
-    stage40(sb + O_UY, sb + O_SY, m, M_V40_4, M_V40_32, M_V40_2, M_V4_8, M_V4_32, M_V4_2, x0, xs, yt4, yt8, y0,
-            yb, nz + pz3, seam, b);
-    tma3(sb + O_UX, &m[M_V40_32], x0 - 4, y0, pz3, b);
-    if (seam) tma3(sb + O_SX + 32, &m[M_V4_32], xs, y0, pz3, b);
+    if (!yseam) {   // one box per array, from row -3 (u_y: -2, u_x: 0) on
+        if (part == 0) {
+            bar_arm(b, BYTES_IN + (seam ? BYTES_IN_SEAM : 0u));
+            tma3(sb + O_PHI, &fm[M_F40_38], x0 - 4, y0 - 3, pz, b);
+            if (seam) tma3(sb + O_SP, &fm[M_F4_38], xs, y0 - 3, pz, b);
+        } else if (part == 1) {
+            tma3(sb + O_UZ, &m[M_V40_38], x0 - 4, y0 - 3, 2 * nz + pz1, b);
+            if (seam) tma3(sb + O_SZ, &m[M_V4_38], xs, y0 - 3, 2 * nz + pz1, b);
+        } else if (part == 2) {
+            tma3(sb + O_UY, &m[M_V40_36], x0 - 4, y0 - 2, nz + pz3, b);
+            if (seam) tma3(sb + O_SY, &m[M_V4_36], xs, y0 - 2, nz + pz3, b);
+        } else {
+            tma3(sb + O_UX, &m[M_V40_32], x0 - 4, y0, pz3, b);
+            if (seam) tma3(sb + O_SX + 32, &m[M_V4_32], xs, y0, pz3, b);
+        }
+    } else if (part == 0) {
+        bar_arm(b, BYTES + (seam ? BYTES_SEAM : 0u));
+        stage40(sb + O_PHI, sb + O_SP, fm, M_F40_4, M_F40_32, M_F40_3, M_F4_8, M_F4_32, M_F4_3, x0, xs, yt4, yt8, y0,
+                yb, pz, seam, b);
+    } else if (part == 1) {
+        stage40(sb + O_UZ, sb + O_SZ, m, M_V40_4, M_V40_32, M_V40_3, M_V4_8, M_V4_32, M_V4_3, x0, xs, yt4, yt8, y0,
+                yb, 2 * nz + pz1, seam, b);
+    } else if (part == 2) {
+        stage40(sb + O_UY, sb + O_SY, m, M_V40_4, M_V40_32, M_V40_2, M_V4_8, M_V4_32, M_V4_2, x0, xs, yt4, yt8, y0,
+                yb, nz + pz3, seam, b);
+    } else {
+        tma3(sb + O_UX, &m[M_V40_32], x0 - 4, y0, pz3, b);
+        if (seam) tma3(sb + O_SX + 32, &m[M_V4_32], xs, y0, pz3, b);
+    }
 }
 
 // The same bundle by copies of CH floats (all threads): Phi and u_z rows
@@ -1071,7 +1127,7 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
     bool bad = false;
     int hint = 0;
     Seg sg;
-    constexpr int ISSUER = NT - 1;                    // idle in the y phase
+    const bool issuer = (tid & 31) == 31 && tid >= NT / 2;   // of array 7 - tid / 32
     __shared__ uint64_t bars[NS];
     if (tid == 0) {
         for (int k = 0; k < NS; ++k) bar_init(&bars[k], CH ? NT : 1);
@@ -1112,13 +1168,18 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
         const int pfirst = sg.z0 - 3, plast = sg.z1 + 2;
         const bool sl = CH == 0 && x0 == 0, sr = CH == 0 && x0 + TX == I.nx, seam = sl || sr;
         const int edge = (sl ? 1 : 0) | (sr ? 2 : 0);
+        // staged rows of row -3 of Phi and u_z, row -2 of u_y: the first, or behind the
+        // rest of the upper row band
+        const bool yseam = CH || y0 == 0 || y0 + TY == I.ny;
+        const int rz = yseam ? 1 : 0, ry = yseam ? 2 : 0;
         auto issue = [&](int pz, int s) {
             if constexpr (CH) {
                 if (!tmo)
                     zyx_copy<CH>(buf + s * SLOT, &bars[s], offs, tid, I.fin[fld], I.vel, I.ncell, pz * plane_n,
                                  (pz == 0 ? nz - 1 : pz - 1) * plane_n, (pz >= 3 ? pz - 3 : pz - 3 + nz) * plane_n);
-            } else if (tid == ISSUER && !tmo) {
-                zyx_issue(buf + s * SLOT, &bars[s], fmaps, maps, x0, y0, I.nx, I.ny, nz, pz, seam);
+            } else if (issuer && !tmo) {
+                zyx_issue(buf + s * SLOT, &bars[s], fmaps, maps, x0, y0, I.nx, I.ny, nz, pz, seam, yseam,
+                          7 - (tid >> 5));
                 armed |= 1u << s;
             }
         };
@@ -1131,12 +1192,12 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
             int zr, zc;
             zpair(q, zr, zc);
             const bool side = ((zc < 2 ? 1 : (zc >= 18 ? 2 : 0)) & edge) != 0;
-            zop[k] = q >= NZP ? 0 : (side ? O_SP + 20 + 4 * zr + 2 * (zc & 1) : O_PHI + (zr + 1) * ZS + 2 * zc);
+            zop[k] = q >= NZP ? 0 : (side ? O_SP + 20 * rz + 4 * zr + 2 * (zc & 1) : O_PHI + (zr + rz) * ZS + 2 * zc);
         }
         // u_y of the y item: row yg - 2 + k at uyo + k ust
         const bool yside = ((lane < 2 ? 1 : (lane >= 18 ? 2 : 0)) & edge) != 0;
         const int ust = yside ? 4 : ZS;
-        const int uyo = yside ? O_SY + 24 + 4 * yg + 2 * (lane & 1) : O_UY + (yg + 2) * ZS + 2 * lane;
+        const int uyo = yside ? O_SY + 12 * ry + 4 * yg + 2 * (lane & 1) : O_UY + (yg + ry) * ZS + 2 * lane;
         Blocks3 bu;
         bu.set(O_UX + xrow * ZS, O_SX + 32 + 4 * xrow, xr, sl, sr);
         float *const obase = (BATCH ? I.out : I.fout[fld]) + (int64_t)(y0 + xrow) * I.nx + x0 + xr;
@@ -1169,7 +1230,7 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
             if (!ok) {
                 polls = 1;
                 tmo = true;
-            } else if (tid == ISSUER) {
+            } else if (issuer) {
                 armed &= ~(1u << s);
             }
             par ^= 1u << s;
@@ -1278,7 +1339,7 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
     }
     if constexpr (CH)
         cp_async_wait_all();
-    else if (tid == ISSUER && armed)
+    else if (issuer && armed)
         drain<NS>(bars, armed, par);
     if (tmo) atomicOr(status, 2u);
     flag_cfl(status, bad);
@@ -1381,8 +1442,10 @@ cudaError_t encode_maps(FastMaps &fm, const FastInst &f)
     if (!enc) return cudaErrorNotSupported;
     static const int shape[NMAPS][3] = {
         {0, 44, 8}, {0, 44, 32}, {0, 44, 3}, {0, 40, 4}, {0, 40, 32}, {0, 40, 3}, {0, 4, 8}, {0, 4, 32}, {0, 4, 3},
+        {0, 44, 38}, {0, 40, 38}, {0, 4, 38},
         {1, 44, 8}, {1, 44, 32}, {1, 44, 3}, {1, 40, 4}, {1, 40, 32}, {1, 40, 3}, {1, 40, 2}, {1, 4, 8},
-        {1, 4, 32}, {1, 4, 3}, {1, 4, 2}, {1, 32, 2}, {1, 32, 32}};
+        {1, 4, 32}, {1, 4, 3}, {1, 4, 2}, {1, 32, 2}, {1, 32, 32},
+        {1, 44, 38}, {1, 40, 38}, {1, 4, 38}, {1, 40, 36}, {1, 4, 36}, {1, 32, 36}};
     for (int k = 0; k < NMAPS; ++k) {
         const bool v = shape[k][0] == 1;
         const cuuint64_t dims[3] = {(cuuint64_t)f.nx, (cuuint64_t)f.ny, (cuuint64_t)f.nz * (v ? 3 : 1)};

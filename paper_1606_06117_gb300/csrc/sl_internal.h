@@ -144,7 +144,7 @@ struct FastInst {
 constexpr int kFastHaloBelow = 6, kFastHaloAbove = 3;
 // Bytes of one instance's tensor maps (22 maps of the first field and the
 // velocity, 9 for each further field; 128 bytes each, 64-byte aligned).
-constexpr size_t kFastMapsBytes = (22 + 9 * (kFastFields - 1)) * 128;
+constexpr size_t kFastMapsBytes = (31 + 12 * (kFastFields - 1)) * 128;
 // Encodes the tensor maps of an instance into dst (host memory, kFastMapsBytes).
 cudaError_t fast_encode_maps(void *dst, const FastInst &f);
 bool fast_eligible(const int64_t dims[3], int ndim, int dtype, bool aligned);

@@ -58,3 +58,26 @@ def test_shares_and_field_groups_keep_the_bits(tmp_path, nx):
             for o, r in zip(outs, refs):
                 assert torch.equal(o, r), (tz, parity)
     assert sl.sl_device_status() == 0
+
+
+# (nz, ny, nx): no tile row, one and three tile rows away from the periodic seam in y, at either seam in x
+# and between them; one field and groups of fields
+@pytest.mark.parametrize("fields", [1, 3])
+@pytest.mark.parametrize("shape", [(8, 32, 64), (9, 64, 96), (12, 96, 64), (10, 160, 128)])
+def test_boxes_of_inner_and_seam_tiles_give_the_bits_of_the_copies(shape, fields):
+    nz, ny, nx = shape
+    phi, vel, sp, dt = random_case(shape, seed=sum(shape), dtype="f32")
+    n, vel, dims = phi.numel(), vel.to(DEV), [nx, ny, nz]
+    store = torch.randn((fields,) + shape, device=DEV)
+    store[0] = phi.to(DEV)
+    for parity in (0, 1):
+        outs = torch.empty((fields,) + shape, device=DEV)
+        sl.sl_advect_multi(list(outs), list(store), vel, 3, dims, sp, dt, sl.CEC, sl.F32, parity)
+        for f in range(fields):
+            buf = torch.empty(n + 1, dtype=torch.float32, device=DEV)
+            buf[1:] = store[f].view(-1)     # one float off 16 bytes: copied element by element
+            ref = torch.empty(n, dtype=torch.float32, device=DEV)
+            sl.sl_advect(ref, buf.data_ptr() + 4, vel, 3, dims, sp, dt, sl.CEC, sl.F32, parity)
+            torch.cuda.synchronize()
+            assert torch.equal(outs[f].view(-1), ref), (parity, f)
+    assert sl.sl_device_status() == 0
