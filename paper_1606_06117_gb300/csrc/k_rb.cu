@@ -27,16 +27,21 @@
 // clock and SM), so the step is arranged to spend few FP64 operations and to
 // spread them over many SMs: each producer writes its cells' ghost images
 // itself (no separate fill pass), the forces kernel also gives the divergence,
-// the per-cell kernels use small CTAs, and the transforms run one CTA per mode or
+// the forces' CTAs hold 32 cells, and the transforms run one CTA per mode or
 // row: all that stays within a z mode in one kernel (both x transforms), the
 // inverse z transform in the projection, which needs a row of phi and the
 // difference of its neighbours only.  That makes four launches per step (the
 // advection of the three fields in one).  At 50 x 50 the step is a chain of small
 // kernels, so each is launched while its predecessor runs (programmatic dependent
 // launch), sets up what does not depend on it, copies its constant operands and
-// then waits; long runs replay the step from a CUDA graph.
-// Measured, 50 x 50 FP64 CEC, us per step: 29.9 with five launches one after the
-// other, 23.9 with the double-precision sweeps of k_split64.cu, 23.0 now.
+// then waits; long runs replay the step from a CUDA graph.  A kernel lets the next
+// one in only when most of its work is done: CTAs that come in earlier take their
+// places while the SMs are full, two or more end on one SM, and the FP64 pipe of
+// that SM is what the step then waits for.
+// Measured, FP64 CEC, us per step at 50 x 50 (128 x 128): 29.9 (65.5) with five
+// launches one after the other, 23.9 with the double-precision sweeps of
+// k_split64.cu, 23.0 (108) with four launches that overlap from their start, 21.5
+// (100) with the forces' terms on warps of their own, 17.8 (58) with the late release.
 #include <cmath>
 #include <new>
 #include <vector>
@@ -108,32 +113,61 @@ __device__ __forceinline__ void store_mirrored(T *pl, int k, int i, T v, int nx,
 // velocities (averages of the adjacent cells of (u2, w2), zero on the walls)
 // into d (nz x nx).  A cell evaluates u2 and w2 of its neighbours itself (the
 // same expressions), so that no second pass is needed for the divergence.
+// What bounds it at the paper's 50^2: FP64 issue, about 60 cycles of a scheduler per
+// warp instruction, with one warp of 32 cells per SM.  So each of a CTA's 7 warps takes
+// one of the terms (u2 here and on either side, w2 here and above and below, theta') of
+// the same 32 cells, and the divergence is put together through shared memory.
+// Measured, 50^2 FP64: 23.2 us per step with one thread per cell, 21.5 with
+// the terms apart.
+constexpr int kRbTerms = 7;
 template <typename T>
-__global__ void k_rb_forces(const T *u, const T *w, const T *th, const T *au, const T *aw, const T *at, T *o_u, T *o_w,
-                            T *o_t, T *d, int nx, int nz, T dt, T Ra, T Pr, T idx2, T idz2, T idx, T idz)
+__global__ void __launch_bounds__(32 * kRbTerms)
+k_rb_forces(const T *u, const T *w, const T *th, const T *au, const T *aw, const T *at, T *o_u, T *o_w, T *o_t, T *d,
+            int nx, int nz, T dt, T Ra, T Pr, T idx2, T idz2, T idx, T idz)
 {
-    const int px = rb_px(nx);
-    const int n = nx * nz;
-    auto lap = [&](const T *f, int64_t o) {
-        return (f[o + 1] - T(2) * f[o] + f[o - 1]) * idx2 + (f[o + px] - T(2) * f[o] + f[o - px]) * idz2;
+    __shared__ T val[kRbTerms][32];
+    const int px = rb_px(nx), lane = threadIdx.x & 31, term = threadIdx.x >> 5;
+    const int c = blockIdx.x * 32 + lane;
+    const bool in = c < nx * nz;
+    const int k = c / nx, i = c - k * nx;
+    const int64_t o = (int64_t)(k + RBG) * px + i + RBG;
+    auto lap = [&](const T *f, int64_t q) {
+        return (f[q + 1] - T(2) * f[q] + f[q - 1]) * idx2 + (f[q + px] - T(2) * f[q] + f[q - px]) * idz2;
     };
-    auto u2 = [&](int64_t o) { return au[o] + dt * (Pr * lap(u, o)); };
-    auto w2 = [&](int64_t o) { return aw[o] + dt * (Ra * Pr * th[o] + Pr * lap(w, o)); };
-    pdl_release();
     pdl_wait();
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-        const int k = c / nx, i = c - (c / nx) * nx;
-        const int64_t o = (int64_t)(k + RBG) * px + i + RBG;
-        const T uc = u2(o), wc = w2(o);
-        o_u[o] = uc;
-        o_w[o] = wc;
+    if (term < 3) {
+        // u2 at the cell (term 0), its east (1) and west neighbour (2)
+        if (in && (term == 0 || (term == 1 ? i + 1 < nx : i > 0))) {
+            const int64_t q = o + (term == 1) - (term == 2);
+            const T v = au[q] + dt * (Pr * lap(u, q));
+            val[term][lane] = v;
+            if (term == 0) o_u[o] = v;
+        }
+    } else if (term < 6) {
+        // w2 at the cell (term 3), above (4) and below it (5)
+        if (in && (term == 3 || (term == 4 ? k + 1 < nz : k > 0))) {
+            const int64_t q = o + (term == 4 ? px : 0) - (term == 5 ? px : 0);
+            const T v = aw[q] + dt * (Ra * Pr * th[q] + Pr * lap(w, q));
+            val[term][lane] = v;
+            if (term == 3) o_w[o] = v;
+        }
+    } else if (in) {
         store_mirrored(o_t, k, i, at[o] + dt * (w[o] + lap(th, o)), nx, nz, T(1), T(-1));
-        const T ue = i + 1 < nx ? T(0.5) * (uc + u2(o + 1)) : T(0);
-        const T uw = i > 0 ? T(0.5) * (u2(o - 1) + uc) : T(0);
-        const T wn = k + 1 < nz ? T(0.5) * (wc + w2(o + px)) : T(0);
-        const T ws = k > 0 ? T(0.5) * (w2(o - px) + wc) : T(0);
-        d[c] = (ue - uw) * idx + (wn - ws) * idz;
     }
+    pdl_release();
+    __syncthreads();
+    T part = T(0);
+    if (term == 0 && in) {
+        const T ue = i + 1 < nx ? T(0.5) * (val[0][lane] + val[1][lane]) : T(0);
+        const T uw = i > 0 ? T(0.5) * (val[2][lane] + val[0][lane]) : T(0);
+        part = (ue - uw) * idx;
+    } else if (term == 3 && in) {
+        const T wn = k + 1 < nz ? T(0.5) * (val[3][lane] + val[4][lane]) : T(0);
+        const T ws = k > 0 ? T(0.5) * (val[5][lane] + val[3][lane]) : T(0);
+        val[6][lane] = (wn - ws) * idz;
+    }
+    __syncthreads();
+    if (term == 0 && in) d[c] = part + val[6][lane];
 }
 
 constexpr int kRbRowThreads = 256;
@@ -219,7 +253,6 @@ k_rb_modes(const T *D, const T *cz, const T *cx, const T *cxT, const T *lx, cons
     T *part = reinterpret_cast<T *>(rb_smem), *R = part + kRbRowThreads, *F = R + rb_pad<T>(nx);
     T *az = F + rb_pad<T>(nx), *sD = az + rb_pad<T>(nz), *sC = sD + rb_pad<T>((int64_t)nz * nx);
     const int k = blockIdx.x, px = rb_pitch(nx);
-    pdl_release();
     for (int m = threadIdx.x; m < nz; m += kRbRowThreads) az[m] = cz[(int64_t)k * nz + m];
     if constexpr (STAGED)
         for (int e = threadIdx.x; e < nx * nx; e += kRbRowThreads) sC[(e / nx) * px + e % nx] = cx[e];
@@ -236,6 +269,7 @@ k_rb_modes(const T *D, const T *cz, const T *cx, const T *cxT, const T *lx, cons
     rb_vecmat<1>(a1, STAGED ? sC : cxT, STAGED ? 1 : nx, STAGED ? px : 1, nx, nx, part,
                  [&](int, int j, T v) { F[j] = (k == 0 && j == 0) ? T(0) : v / (lk + lx[j]); });
     T *Gk = G + (int64_t)k * nx;
+    pdl_release();
     rb_vecmat<1>(a2, STAGED ? sC : cx, STAGED ? px : nx, 1, nx, nx, part, [&](int, int i, T v) { Gk[i] = v; });
 }
 
@@ -253,7 +287,6 @@ k_rb_project(const T *u2, const T *w2, const T *G, const T *czT, const T *zT, T 
     T *part = reinterpret_cast<T *>(rb_smem), *phi = part + 2 * kRbRowThreads, *dphi = phi + rb_pad<T>(nx);
     T *a = dphi + rb_pad<T>(nx), *z = a + rb_pad<T>(nz), *sG = z + rb_pad<T>(nz);
     const int m = blockIdx.x, px = rb_px(nx);
-    pdl_release();
     for (int k = threadIdx.x; k < nz; k += kRbRowThreads) {
         a[k] = czT[(int64_t)m * nz + k];
         z[k] = zT[(int64_t)m * nz + k];
@@ -267,6 +300,7 @@ k_rb_project(const T *u2, const T *w2, const T *G, const T *czT, const T *zT, T 
     __syncthreads();
     const T *const az[2] = {a, z};
     rb_vecmat<2>(az, STAGED ? sG : G, nx, 1, nz, nx, part, [&](int q, int i, T v) { (q ? dphi : phi)[i] = v; });
+    pdl_release();
     for (int i = threadIdx.x; i < nx; i += kRbRowThreads) {
         const int64_t o = (int64_t)(m + RBG) * px + i + RBG;
         const T dx = phi[i + 1 < nx ? i + 1 : i] - phi[i > 0 ? i - 1 : i];
@@ -309,23 +343,13 @@ __global__ void k_rb_copy(const T *src, T *dst, int nx, int nz, bool to_padded)
 
 int blocks_for(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 4096); }
 
-// Threads per CTA for the per-cell kernels: FP64 arithmetic is scarce per SM,
-// so small boxes spread over as many SMs as the device has before CTAs grow.
-int cell_block(int64_t n, int sms)
-{
-    int b = 32;
-    while (b < 256 && (n + b - 1) / b > 4 * sms) b *= 2;
-    return b;
-}
-int cell_grid(int64_t n, int b) { return (int)std::min<int64_t>((n + b - 1) / b, 4096); }
-
 }  // namespace
 }  // namespace sl
 
 using namespace sl;
 
 struct sl_rb {
-    int device = -1, sms = 1;
+    int device = -1;
     bool staged = false;   // transforms with staged operands (small boxes)
     int nx = 0, nz = 0, scheme = SL_CEC, dtype = SL_F64;
     double Lx = 2.0, Lz = 1.0, Ra = 0.0, Pr = 1.0;
@@ -367,7 +391,6 @@ int rb_step_t(sl_rb *r, double dt, int nsteps, cudaStream_t st)
     const double dx = r->Lx / nx, dz = r->Lz / nz;
     const int64_t pdims[3] = {px, pz, 1};
     const double sp[3] = {dx, dz, 1.0};
-    const int cbk = cell_block(n, r->sms), cgr = cell_grid(n, cbk);
     const size_t msm = rb_modes_smem<T>(nx, nz, r->staged), psm = rb_project_smem<T>(nx, nz, r->staged);
     auto modes = r->staged ? k_rb_modes<T, true> : k_rb_modes<T, false>;
     auto project = r->staged ? k_rb_project<T, true> : k_rb_project<T, false>;
@@ -382,7 +405,7 @@ int rb_step_t(sl_rb *r, double dt, int nsteps, cudaStream_t st)
         if (rc) return rc;
         // forces: u2, w2 into the work planes, theta' (with ghosts) into the
         // next state, the face divergence D into d
-        cudaError_t e = launch_kernel(k_rb_forces<T>, dim3(cgr), cbk, 0, st, true, S0, S0 + P, S0 + 2 * P, A, A + P,
+        cudaError_t e = launch_kernel(k_rb_forces<T>, dim3((n + 31) / 32), 32 * kRbTerms, 0, st, true, S0, S0 + P, S0 + 2 * P, A, A + P,
                                       A + 2 * P, Wk, Wk + P, S1 + 2 * P, d, nx, nz, T(dt), T(r->Ra), T(r->Pr),
                                       T(1.0 / (dx * dx)), T(1.0 / (dz * dz)), T(1.0 / dx), T(1.0 / dz));
         // G = [(C_z D C_x^T) / lam] C_x
@@ -491,7 +514,6 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
     sl_rb *r = new (std::nothrow) sl_rb();
     if (!r) return set_error(SL_ERR_NOMEM, "host allocation");
     r->device = c->device;
-    r->sms = c->num_sms > 0 ? c->num_sms : 1;
     r->nx = nx;
     r->nz = nz;
     r->Lx = Lx;

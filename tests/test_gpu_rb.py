@@ -302,3 +302,9 @@ def test_steps_on_a_side_stream_equal_steps_on_the_default_stream():
             g.close()
     for x, y in zip(*res):
         assert torch.equal(x, y)
+
+
+# one group of 32 cells exactly, four cells more, rows that straddle the groups, a box too large to be staged
+@pytest.mark.parametrize("nx,nz", [(8, 4), (9, 4), (31, 5), (33, 7), (112, 8)])
+def test_boxes_at_the_edges_of_the_cell_groups_match_the_oracle(nx, nz):
+    test_plume_steps_match_the_oracle("CEC", nx, nz, 3)
