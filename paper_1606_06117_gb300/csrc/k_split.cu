@@ -29,7 +29,7 @@ namespace {
 template <typename T, int TX, int TY>
 struct Shape {
     static constexpr int HW = TX + 8;                    // staged x in [-4, TX+4)
-    static constexpr int PW = HW + (sizeof(T) == 4 ? 4 : 2);   // row stride
+    static constexpr int PW = HW + 4;   // row stride
     static constexpr int PH = TY + 6;                    // staged y in [-3, TY+3)
 };
 
@@ -37,35 +37,20 @@ struct Shape {
 template <typename T, int N>
 __device__ __forceinline__ void lds_vec(const T *src, T (&dst)[N])
 {
-    if constexpr (sizeof(T) == 4) {
-        static_assert(N % 4 == 0, "");
+    static_assert(sizeof(T) == 4 && N % 4 == 0, "");
 #pragma unroll
-        for (int i = 0; i < N / 4; ++i) {
-            const float4 v = reinterpret_cast<const float4 *>(src)[i];
-            dst[4 * i] = v.x; dst[4 * i + 1] = v.y; dst[4 * i + 2] = v.z; dst[4 * i + 3] = v.w;
-        }
-    } else {
-        static_assert(N % 2 == 0, "");
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i) {
-            const double2 v = reinterpret_cast<const double2 *>(src)[i];
-            dst[2 * i] = v.x; dst[2 * i + 1] = v.y;
-        }
+    for (int i = 0; i < N / 4; ++i) {
+        const float4 v = reinterpret_cast<const float4 *>(src)[i];
+        dst[4 * i] = v.x; dst[4 * i + 1] = v.y; dst[4 * i + 2] = v.z; dst[4 * i + 3] = v.w;
     }
 }
 
 template <typename T, int N>
 __device__ __forceinline__ void sts_vec(T *dst, const T (&src)[N])
 {
-    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-        for (int i = 0; i < N / 4; ++i)
-            reinterpret_cast<float4 *>(dst)[i] = make_float4(src[4 * i], src[4 * i + 1], src[4 * i + 2], src[4 * i + 3]);
-    } else {
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i)
-            reinterpret_cast<double2 *>(dst)[i] = make_double2(src[2 * i], src[2 * i + 1]);
-    }
+    for (int i = 0; i < N / 4; ++i)
+        reinterpret_cast<float4 *>(dst)[i] = make_float4(src[4 * i], src[4 * i + 1], src[4 * i + 2], src[4 * i + 3]);
 }
 
 // Stages a rectangle of rows [r0, r0+NR) (relative to the tile origin) and
@@ -409,12 +394,7 @@ __device__ __forceinline__ void zyx_item(const Geo &g, int item, const T *__rest
             if (gy < g.ny) {
                 T *dst = out + (int64_t)kz * g.plane + (int64_t)gy * g.nx + x0 + xr;
                 if (VEC && x0 + xr + RX <= g.nx) {
-                    if constexpr (sizeof(T) == 4) {
-                        reinterpret_cast<float4 *>(dst)[0] = make_float4(o[0], o[1], o[2], o[3]);
-                    } else {
-                        reinterpret_cast<double2 *>(dst)[0] = make_double2(o[0], o[1]);
-                        reinterpret_cast<double2 *>(dst)[1] = make_double2(o[2], o[3]);
-                    }
+                    reinterpret_cast<float4 *>(dst)[0] = make_float4(o[0], o[1], o[2], o[3]);
                 } else {
 #pragma unroll
                     for (int i = 0; i < RX; ++i)
