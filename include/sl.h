@@ -492,7 +492,8 @@ int sl_advect_learned(sl_corrector *c, void *out, const void *in, const void *ve
  * sl_rb_create: nx, nz in [4, 4096]; Lx, Lz > 0; Ra finite; Pr >= 0;
  *   scheme sl_scheme; dtype SL_F64 or SL_F32 (the arithmetic of every step).
  *   Allocates all device buffers on the current device (about
- *   12 (nx + 6)(nz + 6) + 2 nx nz + 2 nx^2 + 3 nz^2 elements); the state starts at
+ *   12 (nx + 6)(nz + 6) + 2 nx nz + 2 nx^2 + 3 nz^2 elements, and nx^2 nz more for small
+ *   FP32 boxes and for FP64 boxes where these stay below 256 MB and the device has them); the state starts at
  *   rest (U = 0, theta = 0).  Errors: SL_ERR_ARG, SL_ERR_UNSUPPORTED,
  *   SL_ERR_NOMEM, SL_ERR_CUDA.
  * sl_rb_set_state / sl_rb_get_state: DEVICE arrays of nz x nx elements of the

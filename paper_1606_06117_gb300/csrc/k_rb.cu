@@ -28,11 +28,11 @@
 // spread them over many SMs: each producer writes its cells' ghost images
 // itself (no separate fill pass), the forces kernel also gives the divergence,
 // the forces' CTAs hold 32 cells, and the transforms run one CTA per mode or
-// row: all that stays within a z mode in one kernel (both x transforms), the
+// row: all that stays within a z mode in one kernel (the x solve), the
 // inverse z transform in the projection, which needs a row of phi and the
 // difference of its neighbours only.  That makes four launches per step (the
 // advection of the three fields in one).  At 50 x 50 the step is a chain of small
-// kernels, so each is launched while its predecessor runs (programmatic dependent
+// kernels, so on small boxes each is launched while its predecessor runs (programmatic dependent
 // launch), sets up what does not depend on it, copies its constant operands and
 // then waits; long runs replay the step from a CUDA graph.  A kernel lets the next
 // one in only when most of its work is done: CTAs that come in earlier take their
@@ -41,7 +41,9 @@
 // Measured, FP64 CEC, us per step at 50 x 50 (128 x 128): 29.9 (65.5) with five
 // launches one after the other, 23.9 with the double-precision sweeps of
 // k_split64.cu, 23.0 (108) with four launches that overlap from their start, 21.5
-// (100) with the forces' terms on warps of their own, 17.8 (58) with the late release.
+// (100) with the forces' terms on warps of their own, 17.8 (58) with the late release,
+// 16.3 (51) with one matrix per z mode for its x solve, 16.3 (42.5) with the overlap on
+// small boxes only.
 #include <cmath>
 #include <new>
 #include <vector>
@@ -233,44 +235,70 @@ __host__ __device__ constexpr int64_t rb_pad(int64_t n)
     return (n + 16 / (int64_t)sizeof(T) - 1) / (16 / (int64_t)sizeof(T)) * (16 / (int64_t)sizeof(T));
 }
 
-// Row pitch of C_x in shared memory: odd, so that reading it along either index
-// keeps the lanes on distinct banks.
-__host__ __device__ constexpr int rb_pitch(int nx) { return nx | 1; }
-
 // Everything of the Poisson solve that stays within one z mode, one CTA per mode k:
 //   R[i] = sum_m C_z[k][m] D[m][i],  F[j] = sum_i R[i] C_x[j][i] / lam_kj,
 //   G[k][i] = sum_j F[j] C_x[j][i]
 // (lam_kj = lz[k] + lx[j]; the constant mode F[0] of k = 0 is 0); phi = C_z^T G is
-// left to the projection.  STAGED (small boxes): D and C_x are copied to shared
-// memory first, so that the sums do not wait on L2; what does not depend on the
-// predecessor is copied while that still runs.  Otherwise C_x enters transposed
-// for the second sum (cxT), so that every load is coalesced or a broadcast.
-template <typename T, bool STAGED>
+// left to the projection.  The last two are one linear map of a row, so
+//   G[k] = R M_k,  M_k[i][i'] = sum_{j, lam_kj != 0} C_x[j][i] C_x[j][i'] / lam_kj
+// with the matrices M_k computed once per box: a third of the FP64 sums and all
+// divisions less per step (FP64 CEC, 50 x 50: 17.8 -> 16.3 us per step, 128 x 128: 58 ->
+// 51, 400 x 50: 175 -> 110).  Forms:
+//   kLarge   M would take more than kRbGreenMax, or FP32 boxes that are not staged
+//            (their sums are cheap and C_x stays closer than M: 128 x 128 33 us against
+//            38): both x transforms, C_x entering transposed for the first, so that
+//            every load is coalesced or a broadcast;
+//   kGreen   M_k read from global memory;
+//   kStaged  small boxes: D and M_k are copied to shared memory first, so that the
+//            sums do not wait on L2; M_k while the predecessor still runs.
+enum RbForm { kLarge, kGreen, kStaged };
+template <typename T, int FORM>
 __global__ void __launch_bounds__(kRbRowThreads)
-k_rb_modes(const T *D, const T *cz, const T *cx, const T *cxT, const T *lx, const T *lz, T *G, int nx, int nz)
+k_rb_modes(const T *D, const T *cz, const T *cx, const T *cxT, const T *M, const T *lx, const T *lz, T *G, int nx, int nz)
 {
     extern __shared__ __align__(16) unsigned char rb_smem[];
     T *part = reinterpret_cast<T *>(rb_smem), *R = part + kRbRowThreads, *F = R + rb_pad<T>(nx);
-    T *az = F + rb_pad<T>(nx), *sD = az + rb_pad<T>(nz), *sC = sD + rb_pad<T>((int64_t)nz * nx);
-    const int k = blockIdx.x, px = rb_pitch(nx);
+    T *az = F + rb_pad<T>(nx), *sD = az + rb_pad<T>(nz), *sM = sD + rb_pad<T>((int64_t)nz * nx);
+    const int k = blockIdx.x;
     for (int m = threadIdx.x; m < nz; m += kRbRowThreads) az[m] = cz[(int64_t)k * nz + m];
-    if constexpr (STAGED)
-        for (int e = threadIdx.x; e < nx * nx; e += kRbRowThreads) sC[(e / nx) * px + e % nx] = cx[e];
-    const T lk = lz[k];
+    const T *const Mk = FORM == kLarge ? nullptr : M + k * rb_pad<T>((int64_t)nx * nx);
+    if constexpr (FORM == kStaged) rb_stage(sM, Mk, (int64_t)nx * nx);
     pdl_wait();
-    if constexpr (STAGED) {
+    if constexpr (FORM == kStaged) {
         rb_stage(sD, D, (int64_t)nz * nx);
         cp_async_commit();
         cp_async_wait_all();
     }
     __syncthreads();
     const T *const a0[1] = {az}, *const a1[1] = {R}, *const a2[1] = {F};
-    rb_vecmat<1>(a0, STAGED ? sD : D, nx, 1, nz, nx, part, [&](int, int i, T v) { R[i] = v; });
-    rb_vecmat<1>(a1, STAGED ? sC : cxT, STAGED ? 1 : nx, STAGED ? px : 1, nx, nx, part,
-                 [&](int, int j, T v) { F[j] = (k == 0 && j == 0) ? T(0) : v / (lk + lx[j]); });
     T *Gk = G + (int64_t)k * nx;
+    rb_vecmat<1>(a0, FORM == kStaged ? sD : D, nx, 1, nz, nx, part, [&](int, int i, T v) { R[i] = v; });
+    if constexpr (FORM == kLarge) {
+        const T lk = lz[k];
+        rb_vecmat<1>(a1, cxT, nx, 1, nx, nx, part,
+                     [&](int, int j, T v) { F[j] = (k == 0 && j == 0) ? T(0) : v / (lk + lx[j]); });
+    }
     pdl_release();
-    rb_vecmat<1>(a2, STAGED ? sC : cx, STAGED ? px : nx, 1, nx, nx, part, [&](int, int i, T v) { Gk[i] = v; });
+    rb_vecmat<1>(FORM == kLarge ? a2 : a1, FORM == kLarge ? cx : (FORM == kStaged ? sM : Mk), nx, 1, nx, nx, part,
+                 [&](int, int i, T v) { Gk[i] = v; });
+}
+
+// M of one box, summed in double: thread (i, i') of mode k = blockIdx.y; the CTA's
+// 1 / lam_kj once in shared memory (a division per term took most of the time).
+template <typename T>
+__global__ void k_rb_green(const T *cx, const T *lx, const T *lz, T *M, int nx)
+{
+    extern __shared__ __align__(16) unsigned char rb_smem[];
+    double *inv = reinterpret_cast<double *>(rb_smem);
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nn = (int64_t)nx * nx;
+    const int k = blockIdx.y, i = (int)(e / nx), i2 = (int)(e % nx);
+    for (int j = threadIdx.x; j < nx; j += blockDim.x)
+        inv[j] = k == 0 && j == 0 ? 0.0 : 1.0 / ((double)lz[k] + (double)lx[j]);
+    __syncthreads();
+    if (e >= nn) return;
+    double acc = 0.0;
+    for (int j = 0; j < nx; ++j) acc += (double)cx[(int64_t)j * nx + i] * inv[j] * (double)cx[(int64_t)j * nx + i2];
+    M[k * rb_pad<T>(nn) + e] = T(acc);
 }
 
 // Projection, one CTA per row m: phi[m][i] = sum_k C_z[k][m] G[k][i] and the
@@ -279,17 +307,32 @@ k_rb_modes(const T *D, const T *cz, const T *cx, const T *cxT, const T *lx, cons
 // there).  Cells take the average of their two faces' gradient corrections
 // (face gradient (phi_{i+1} - phi_i) / dx inside, zero on the walls); the result
 // is the new u, w with their ghost images.  czT, zT: C_z and Z transposed.
-template <typename T, bool STAGED>
+// PAIR: one CTA for the rows m and nz - 1 - m, whose sums differ in the signs of the odd
+// modes only (C_z[k][nz-1-m] = (-1)^k C_z[k][m], Z with a minus), so that the even
+// and the odd half-sums serve both: half the FP64 work, on half as many CTAs.  It
+// is for boxes of more rows than kRbPairRows, the SMs they would otherwise share.
+// Measured, CEC, us per step without and with: 300 x 200 FP64 240 / 232, FP32 127 / 105.
+constexpr int kRbPairRows = 152;
+// Boxes of at most half as many rows as there are SMs launch each kernel while its
+// predecessor runs: the CTAs of two kernels then find an SM each.  On larger boxes
+// the next kernel's CTAs crowd on the SMs that finish first, and the FP64 pipe of
+// those SMs is what the step waits for.  Measured, FP64 CEC, us per step with and
+// without the overlap: 50 x 50 16.3 / 17.0, 80 x 80 30.6 / 29.9, 100 x 100 41.7 / 36.0,
+// 128 x 128 50.9 / 42.5, 512 x 256 702 / 535.
+constexpr int kRbEarlyRows = 76;
+template <typename T, bool STAGED, bool PAIR>
 __global__ void __launch_bounds__(kRbRowThreads)
 k_rb_project(const T *u2, const T *w2, const T *G, const T *czT, const T *zT, T *u, T *w, int nx, int nz, T idx, T idz)
 {
     extern __shared__ __align__(16) unsigned char rb_smem[];
-    T *part = reinterpret_cast<T *>(rb_smem), *phi = part + 2 * kRbRowThreads, *dphi = phi + rb_pad<T>(nx);
-    T *a = dphi + rb_pad<T>(nx), *z = a + rb_pad<T>(nz), *sG = z + rb_pad<T>(nz);
-    const int m = blockIdx.x, px = rb_px(nx);
-    for (int k = threadIdx.x; k < nz; k += kRbRowThreads) {
-        a[k] = czT[(int64_t)m * nz + k];
-        z[k] = zT[(int64_t)m * nz + k];
+    constexpr int H = PAIR ? 2 : 1;   // interleaved halves of the sums over k
+    T *part = reinterpret_cast<T *>(rb_smem), *phi = part + 2 * kRbRowThreads, *dphi = phi + H * rb_pad<T>(nx);
+    T *a = dphi + H * rb_pad<T>(nx), *z = a + rb_pad<T>(nz) + rb_pad<T>(H), *sG = z + rb_pad<T>(nz) + rb_pad<T>(H);
+    const int m = blockIdx.x, px = rb_px(nx), nh = (nz + H - 1) / H;
+    for (int k = threadIdx.x; k < nz; k += kRbRowThreads) {   // even k, then odd k
+        const int at = PAIR ? (k & 1) * nh + (k >> 1) : k;
+        a[at] = czT[(int64_t)m * nz + k];
+        z[at] = zT[(int64_t)m * nz + k];
     }
     pdl_wait();
     if constexpr (STAGED) {
@@ -298,14 +341,30 @@ k_rb_project(const T *u2, const T *w2, const T *G, const T *czT, const T *zT, T 
         cp_async_wait_all();
     }
     __syncthreads();
-    const T *const az[2] = {a, z};
-    rb_vecmat<2>(az, STAGED ? sG : G, nx, 1, nz, nx, part, [&](int q, int i, T v) { (q ? dphi : phi)[i] = v; });
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        const T *const az[2] = {a + h * nh, z + h * nh};
+        T *ph = phi + h * rb_pad<T>(nx), *dp = dphi + h * rb_pad<T>(nx);
+        rb_vecmat<2>(az, (STAGED ? sG : G) + h * nx, H * nx, 1, h ? nz / 2 : nh, nx, part,
+                     [&](int q, int i, T v) { (q ? dp : ph)[i] = v; });
+    }
     pdl_release();
+    auto correct = [&](int row, int i, T dx, T dz) {
+        const int64_t o = (int64_t)(row + RBG) * px + i + RBG;
+        store_mirrored(u, row, i, u2[o] - T(0.5) * (dx * idx), nx, nz, T(-1), T(-1));
+        store_mirrored(w, row, i, w2[o] - T(0.5) * (dz * idz), nx, nz, T(-1), T(-1));
+    };
     for (int i = threadIdx.x; i < nx; i += kRbRowThreads) {
-        const int64_t o = (int64_t)(m + RBG) * px + i + RBG;
-        const T dx = phi[i + 1 < nx ? i + 1 : i] - phi[i > 0 ? i - 1 : i];
-        store_mirrored(u, m, i, u2[o] - T(0.5) * (dx * idx), nx, nz, T(-1), T(-1));
-        store_mirrored(w, m, i, w2[o] - T(0.5) * (dphi[i] * idz), nx, nz, T(-1), T(-1));
+        const int ie = i + 1 < nx ? i + 1 : i, iw = i > 0 ? i - 1 : i;
+        const T dx = phi[ie] - phi[iw];
+        if constexpr (!PAIR) {
+            correct(m, i, dx, dphi[i]);
+        } else {
+            const T *po = phi + rb_pad<T>(nx);
+            const T dxo = po[ie] - po[iw], dzo = dphi[rb_pad<T>(nx) + i];
+            correct(m, i, dx + dxo, dphi[i] + dzo);
+            if (nz - 1 - m != m) correct(nz - 1 - m, i, dx - dxo, dzo - dphi[i]);
+        }
     }
 }
 
@@ -314,16 +373,20 @@ template <typename T>
 size_t rb_modes_smem(int nx, int nz, bool staged)
 {
     return sizeof(T) * (size_t)(kRbRowThreads + 2 * rb_pad<T>(nx) + rb_pad<T>(nz) +
-                                (staged ? rb_pad<T>((int64_t)nz * nx) + (int64_t)nx * rb_pitch(nx) : 0));
+                                (staged ? rb_pad<T>((int64_t)nz * nx) + rb_pad<T>((int64_t)nx * nx) : 0));
 }
 template <typename T>
 size_t rb_project_smem(int nx, int nz, bool staged)
 {
-    return sizeof(T) * (size_t)(2 * kRbRowThreads + 2 * rb_pad<T>(nx) + 2 * rb_pad<T>(nz) +
+    const int h = nz > kRbPairRows ? 2 : 1;
+    return sizeof(T) * (size_t)(2 * kRbRowThreads + 2 * h * rb_pad<T>(nx) + 2 * (rb_pad<T>(nz) + rb_pad<T>(2)) +
                                 (staged ? rb_pad<T>((int64_t)nz * nx) : 0));
 }
-// (an unstaged FP64 box of 4096 x 4096 takes 132 KB in the projection)
-constexpr size_t kRbStagedMax = 96 * 1024, kRbSmemMax = 136 * 1024;
+// (an unstaged FP64 box of 4096 x 4096 takes 197 KB in the projection)
+constexpr size_t kRbStagedMax = 96 * 1024, kRbSmemMax = 200 * 1024;
+// The most M takes.  FP64 boxes gain up to where it is read from HBM every step (144 MB,
+// 300 x 200: 285 -> 240 us) and break even at 537 MB (512 x 256).  Every staged box is below.
+constexpr size_t kRbGreenMax = 256u << 20;
 
 // interior <-> padded copies
 template <typename T>
@@ -363,9 +426,10 @@ struct sl_rb {
     void *S[2] = {nullptr, nullptr}, *A = nullptr, *W = nullptr;
     // interior arrays (nz x nx): the face divergence D, and phi in z modes (G)
     void *d = nullptr, *G = nullptr;
-    // orthonormal DCT-II matrices C_x and C_z and their transposes, the row
-    // differences of C_z (transposed, k_rb_project); eigenvalues per axis
+    // orthonormal DCT-II matrices C_x and C_z, their transposes (C_x's without M only), the
+    // row differences of C_z (transposed, k_rb_project); eigenvalues per axis
     void *cx = nullptr, *cxT = nullptr, *cz = nullptr, *czT = nullptr, *zT = nullptr, *lx = nullptr, *lz = nullptr;
+    void *M = nullptr;      // the z modes' x solves (k_rb_modes), unless too large
     int *signs = nullptr;   // sx of (u, w, theta), then sz of (u, w, theta)
     // long runs replay kRbGraphSteps steps from one CUDA graph, captured for
     // one dt and one starting buffer on a stream of the box's own
@@ -387,13 +451,15 @@ int rb_step_t(sl_rb *r, double dt, int nsteps, cudaStream_t st)
     T *d = static_cast<T *>(r->d), *G = static_cast<T *>(r->G);
     const T *cx = static_cast<const T *>(r->cx), *cxT = static_cast<const T *>(r->cxT);
     const T *cz = static_cast<const T *>(r->cz), *czT = static_cast<const T *>(r->czT), *zT = static_cast<const T *>(r->zT);
-    const T *lx = static_cast<const T *>(r->lx), *lz = static_cast<const T *>(r->lz);
+    const T *lx = static_cast<const T *>(r->lx), *lz = static_cast<const T *>(r->lz), *M = static_cast<const T *>(r->M);
     const double dx = r->Lx / nx, dz = r->Lz / nz;
     const int64_t pdims[3] = {px, pz, 1};
     const double sp[3] = {dx, dz, 1.0};
     const size_t msm = rb_modes_smem<T>(nx, nz, r->staged), psm = rb_project_smem<T>(nx, nz, r->staged);
-    auto modes = r->staged ? k_rb_modes<T, true> : k_rb_modes<T, false>;
-    auto project = r->staged ? k_rb_project<T, true> : k_rb_project<T, false>;
+    auto modes = r->staged ? k_rb_modes<T, kStaged> : (M ? k_rb_modes<T, kGreen> : k_rb_modes<T, kLarge>);
+    const bool pair = nz > kRbPairRows, early = nz <= kRbEarlyRows;
+    auto project = r->staged ? (pair ? k_rb_project<T, true, true> : k_rb_project<T, true, false>)
+                             : (pair ? k_rb_project<T, false, true> : k_rb_project<T, false, false>);
     for (int s = 0; s < nsteps; ++s) {
         // S0 holds step n with its ghost layers (the walls' mirror images)
         T *S0 = static_cast<T *>(r->S[r->cur]), *S1 = static_cast<T *>(r->S[r->cur ^ 1]);
@@ -401,19 +467,19 @@ int rb_step_t(sl_rb *r, double dt, int nsteps, cudaStream_t st)
         // CEC alternates its sweep order with the step index
         const void *ins[3] = {S0, S0 + P, S0 + 2 * P};
         void *outs[3] = {A, A + P, A + 2 * P};
-        int rc = advect_fields(outs, ins, 3, S0, 2, pdims, sp, dt, r->scheme, r->dtype, (int)(r->step & 1), st, true);
+        int rc = advect_fields(outs, ins, 3, S0, 2, pdims, sp, dt, r->scheme, r->dtype, (int)(r->step & 1), st, early);
         if (rc) return rc;
         // forces: u2, w2 into the work planes, theta' (with ghosts) into the
         // next state, the face divergence D into d
-        cudaError_t e = launch_kernel(k_rb_forces<T>, dim3((n + 31) / 32), 32 * kRbTerms, 0, st, true, S0, S0 + P, S0 + 2 * P, A, A + P,
+        cudaError_t e = launch_kernel(k_rb_forces<T>, dim3((n + 31) / 32), 32 * kRbTerms, 0, st, early, S0, S0 + P, S0 + 2 * P, A, A + P,
                                       A + 2 * P, Wk, Wk + P, S1 + 2 * P, d, nx, nz, T(dt), T(r->Ra), T(r->Pr),
                                       T(1.0 / (dx * dx)), T(1.0 / (dz * dz)), T(1.0 / dx), T(1.0 / dz));
         // G = [(C_z D C_x^T) / lam] C_x
         if (e == cudaSuccess)
-            e = launch_kernel(modes, dim3(nz), kRbRowThreads, msm, st, true, d, cz, cx, cxT, lx, lz, G, nx, nz);
+            e = launch_kernel(modes, dim3(nz), kRbRowThreads, msm, st, early, d, cz, cx, cxT, M, lx, lz, G, nx, nz);
         // the projected u, w (with ghosts) of the next state
         if (e == cudaSuccess)
-            e = launch_kernel(project, dim3(nz), kRbRowThreads, psm, st, true, Wk, Wk + P, G, czT, zT, S1, S1 + P, nx, nz,
+            e = launch_kernel(project, dim3(pair ? (nz + 1) / 2 : nz), kRbRowThreads, psm, st, early, Wk, Wk + P, G, czT, zT, S1, S1 + P, nx, nz,
                               T(1.0 / dx), T(1.0 / dz));
         if (e != cudaSuccess) return set_error(SL_ERR_CUDA, cudaGetErrorString(e));
         r->cur ^= 1;
@@ -528,9 +594,22 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
     r->plane = (int64_t)rb_px(nx) * (nz + 2 * RBG);
     auto round64 = [](int64_t k) { return (k + 63) / 64 * 64; };
     const int64_t n = (int64_t)nx * nz;
-    const int64_t elems = 4 * round64(3 * r->plane) + 2 * round64(n) + 2 * round64((int64_t)nx * nx) +
-                          3 * round64((int64_t)nz * nz) + round64(nx) + round64(nz) + 64;
-    if (cudaMalloc(&r->mem, r->esz * elems) != cudaSuccess) {
+    const int64_t mstride = dtype == SL_F64 ? rb_pad<double>((int64_t)nx * nx) : rb_pad<float>((int64_t)nx * nx);
+    r->staged = (dtype == SL_F64 ? rb_modes_smem<double>(nx, nz, true) : rb_modes_smem<float>(nx, nz, true)) <= kRbStagedMax;
+    int64_t melems = r->staged || (dtype == SL_F64 && (size_t)(nz * mstride) * r->esz <= kRbGreenMax) ? nz * mstride : 0;
+    auto elements = [&] {
+        return (melems ? round64(melems) : round64((int64_t)nx * nx)) + round64((int64_t)nx * nx) + round64(nx) +
+               round64(nz) + 4 * round64(3 * r->plane) + 2 * round64(n) + 3 * round64((int64_t)nz * nz) + 64;
+    };
+    if (cudaMalloc(&r->mem, r->esz * elements()) != cudaSuccess && melems) {
+        cudaGetLastError();   // without M and staging the box takes less
+        r->mem = nullptr;
+        r->staged = false;
+        melems = 0;
+        cudaMalloc(&r->mem, r->esz * elements());
+    }
+    const int64_t elems = elements();
+    if (!r->mem) {
         delete r;
         return set_error(SL_ERR_NOMEM, "device buffers of the box");
     }
@@ -547,12 +626,13 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
     r->d = take(n);
     r->G = take(n);
     r->cx = take((int64_t)nx * nx);
-    r->cxT = take((int64_t)nx * nx);
+    if (!melems) r->cxT = take((int64_t)nx * nx);
+    r->lx = take(nx);
+    r->lz = take(nz);
     r->cz = take((int64_t)nz * nz);
     r->czT = take((int64_t)nz * nz);
     r->zT = take((int64_t)nz * nz);
-    r->lx = take(nx);
-    r->lz = take(nz);
+    if (melems) r->M = take(melems);
     r->signs = reinterpret_cast<int *>(p);
     std::vector<double> cxm, czm, cxt((size_t)nx * nx), lxv(nx), lzv(nz);
     dct_matrix(cxm, nx);
@@ -581,30 +661,46 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
         }
     };
     up(r->cx, cxm);
-    up(r->cxT, cxt);
+    if (!melems) up(r->cxT, cxt);
+    up(r->lx, lxv);
+    up(r->lz, lzv);
     up(r->cz, czm);
     up(r->czT, czt);
     up(r->zT, zt);
-    up(r->lx, lxv);
-    up(r->lz, lzv);
+    if (e == cudaSuccess && r->M) {
+        const dim3 grid((unsigned)(((int64_t)nx * nx + 255) / 256), (unsigned)nz);
+        if (dtype == SL_F64)
+            k_rb_green<<<grid, 256, 8 * nx>>>(static_cast<const double *>(r->cx), static_cast<const double *>(r->lx),
+                                              static_cast<const double *>(r->lz), static_cast<double *>(r->M), nx);
+        else
+            k_rb_green<<<grid, 256, 8 * nx>>>(static_cast<const float *>(r->cx), static_cast<const float *>(r->lx),
+                                              static_cast<const float *>(r->lz), static_cast<float *>(r->M), nx);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    }
     if (e == cudaSuccess) e = cudaMemcpy(r->signs, signs, sizeof signs, cudaMemcpyHostToDevice);
     // small boxes stage the transforms' operands in shared memory; the kernels'
     // limit is per function, not per box, so it is raised to the cap that every
     // box fits under
-    r->staged = (dtype == SL_F64 ? rb_modes_smem<double>(nx, nz, true) : rb_modes_smem<float>(nx, nz, true)) <= kRbStagedMax;
     auto raise = [&](auto kern) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRbSmemMax);
     };
     if (dtype == SL_F64) {
-        raise(k_rb_modes<double, true>);
-        raise(k_rb_modes<double, false>);
-        raise(k_rb_project<double, true>);
-        raise(k_rb_project<double, false>);
+        raise(k_rb_modes<double, kStaged>);
+        raise(k_rb_modes<double, kGreen>);
+        raise(k_rb_modes<double, kLarge>);
+        raise(k_rb_project<double, true, false>);
+        raise(k_rb_project<double, false, false>);
+        raise(k_rb_project<double, true, true>);
+        raise(k_rb_project<double, false, true>);
     } else {
-        raise(k_rb_modes<float, true>);
-        raise(k_rb_modes<float, false>);
-        raise(k_rb_project<float, true>);
-        raise(k_rb_project<float, false>);
+        raise(k_rb_modes<float, kStaged>);
+        raise(k_rb_modes<float, kGreen>);
+        raise(k_rb_modes<float, kLarge>);
+        raise(k_rb_project<float, true, false>);
+        raise(k_rb_project<float, false, false>);
+        raise(k_rb_project<float, true, true>);
+        raise(k_rb_project<float, false, true>);
     }
     if (e != cudaSuccess) {
         cudaFree(r->mem);

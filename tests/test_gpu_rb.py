@@ -308,3 +308,11 @@ def test_steps_on_a_side_stream_equal_steps_on_the_default_stream():
 @pytest.mark.parametrize("nx,nz", [(8, 4), (9, 4), (31, 5), (33, 7), (112, 8)])
 def test_boxes_at_the_edges_of_the_cell_groups_match_the_oracle(nx, nz):
     test_plume_steps_match_the_oracle("CEC", nx, nz, 3)
+
+
+# an unstaged FP32 box (both x transforms), and one whose rows are projected in pairs
+@pytest.mark.parametrize("nx,nz", [(160, 8), (6, 155)])
+def test_float32_boxes_of_every_form_track_the_oracle(nx, nz):
+    got, ref = run_both(nx, nz, "CEC", plume_start(nx, nz, seed=nx), 2e-4, 3, Ra=1e5, dtype=torch.float32)
+    for name, a, b in zip(("u", "w", "theta"), got, ref):
+        assert_parity(a, b, "f32", f"{nx}x{nz} {name}", allowance(nx, nz, 3, f64=False))
