@@ -110,9 +110,8 @@ int sl_advect(void *out, const void *in, const void *vel, int ndim,
  * bit to one sl_advect call per field.  Same arguments and errors as
  * sl_advect; every outs[f] must differ from every ins[g] and from the other
  * outs.  Since L_U is linear in Phi for a fixed velocity (Sec. 2), every field
- * shares the departure points and CEC weights; an SL_CEC step in FP32 on the
- * geometry of the persistent kernel (see sl_autotune) advances up to 4 fields
- * per launch: the launch's CTAs form groups, one CTA per field, that walk the
+ * shares the departure points and CEC weights; an SL_CEC step in FP32 on a 3D
+ * grid of 8 planes or more advances up to 4 fields per launch: the launch's CTAs form groups, one CTA per field, that walk the
  * same (column tile, plane) sequence, so that a group's velocity reads can be
  * served from L2 after the first one.  Otherwise fields stored at uniform
  * strides (ins[f] = ins[0] + f * a, outs[f] = outs[0] + f * b, whole elements)

@@ -563,8 +563,8 @@ __device__ __forceinline__ void build_table(int *tab, int tid, int x0, int y0, i
     }
 }
 
-// A wait gave up (no copy arrived within kPolls polls): the issuing thread
-// waits (bounded) for the phase of every slot it armed and that has not
+// A wait gave up (no copy arrived within kPolls polls): an issuing thread
+// waits (bounded) for the phase of every slot it filled and that has not
 // completed, so that no copy lands in shared memory after the CTA has left,
 // and records the timeout.
 template <int NS>
