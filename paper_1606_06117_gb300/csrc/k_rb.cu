@@ -601,18 +601,22 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
         return (melems ? round64(melems) : round64((int64_t)nx * nx)) + round64((int64_t)nx * nx) + round64(nx) +
                round64(nz) + 4 * round64(3 * r->plane) + 2 * round64(n) + 3 * round64((int64_t)nz * nz) + 64;
     };
-    if (cudaMalloc(&r->mem, r->esz * elements()) != cudaSuccess && melems) {
-        cudaGetLastError();   // without M and staging the box takes less
-        r->mem = nullptr;
+    auto allocate = [&] {
+        if (cudaMalloc(&r->mem, r->esz * elements()) == cudaSuccess) return true;
+        cudaGetLastError();
+        return false;
+    };
+    bool got = allocate();
+    if (!got && melems) {   // without M and staging the box takes less
         r->staged = false;
         melems = 0;
-        cudaMalloc(&r->mem, r->esz * elements());
+        got = allocate();
     }
-    const int64_t elems = elements();
-    if (!r->mem) {
+    if (!got) {
         delete r;
         return set_error(SL_ERR_NOMEM, "device buffers of the box");
     }
+    const int64_t elems = elements();
     char *p = static_cast<char *>(r->mem);
     auto take = [&](int64_t k) {
         void *q = p;
