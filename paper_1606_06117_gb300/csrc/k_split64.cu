@@ -20,7 +20,7 @@
 // on 32 x 16 tiles, where register runs with double comparisons took 121 and
 // more.  Two and three CTAs of 256 threads per SM cover each other's barriers.
 // Measured (CUDA events), a step of each order: 256^3 SL_F64 6.56 ms before
-// (32 x 16 and 32 x 8 tiles, 32-plane items), 2.96 ms now; the Rayleigh-Benard step of a 50 x 50 box, which
+// (32 x 16 and 32 x 8 tiles, 32-plane items), 2.90 ms now; the Rayleigh-Benard step of a 50 x 50 box, which
 // advects three fields with this kernel, 29.9 -> 23.9 us.
 #include "sl_internal.h"
 
@@ -36,42 +36,53 @@ __device__ __forceinline__ double pick(int s, double pos, double neg, double zer
 }
 
 // ------------------------------------------------------- the sweep's stages
-// The 1D scheme of sl_common.cuh with d_j = Phi_j - Phi_{j-s_j} carried along:
-//   L_j = Phi_j - U_j d_j,   delta_j = Phi_j - L_j - U_j (L_{j+s_j} - L_j) = U_j (d_j - (L_{j+s_j} - L_j)),
+// The 1D scheme of sl_common.cuh with L_U[Phi] written from the cell,
+//   L_j = Phi_j - U_j (Phi_j - Phi_{j-s_j}),   delta_j = (Phi_j - L_j) - U_j (L_{j+s_j} - L_j),
 // one operation less than from W = 1 - U.  U = 1 takes the neighbour itself, so
 // that an integer Courant number stays an exact shift (delta is then exactly
-// zero); d = 0 keeps constants and C = 0 exact.
-__device__ __forceinline__ double lu(double c, double p, double nb, double &d)
+// zero); equal neighbours keep constants and C = 0 exact.  delta starts from the rounded
+// L_j: half of L_j's rounding error then cancels in the result (U ((Phi_j -
+// Phi_{j-s_j}) - (L_{j+s_j} - L_j)), as many operations, left smooth fields 4 %
+// further from the exact step).
+__device__ __forceinline__ double lu(double c, double p, double nb)
 {
-    d = p - nb;
     const bool unit = (__double2hiint(c) & 0x7fffffff) == 0x3ff00000 && __double2loint(c) == 0;
-    return unit ? nb : fma(-fabs(c), d, p);
+    return unit ? nb : fma(-fabs(c), p - nb, p);
 }
-__device__ __forceinline__ double delta_of(double c, double d, double L, double Ln) { return fabs(c) * (d - (Ln - L)); }
+__device__ __forceinline__ double delta_of(double c, double p, double L, double Ln)
+{
+    return fma(-fabs(c), Ln - L, p - L);
+}
 __device__ __forceinline__ double cec_of(double c, double L, double d, double dn)
 {
     return fma(fma(fabs(c), 1.0 / 6.0, 1.0 / 6.0), dn - d, fma(0.5, d, L));
 }
 
+// Phi of a cell for the two stages of an in-plane sweep that use it: a float is widened
+// once and kept in the cell's place for delta until delta replaces it (widened again,
+// SL_F32_D64 took 3.98 ms for 3.86 at 256^3, a step of each order), a double is read again.
+__device__ __forceinline__ double keep(double v, double &) { return v; }
+__device__ __forceinline__ double keep(float v, double &place) { return place = widen(v); }
+__device__ __forceinline__ double kept(const double &v, double) { return v; }
+__device__ __forceinline__ double kept(const float &, double place) { return place; }
+
 // Sliding window of the sweep along z for one column (ZWin of sl_common.cuh):
 // after a push of Phi_p and C_{p-1} the result is the value at p - 3.
 template <typename T>
 struct ZWin64 {
-    double ph[2], df, L[2], c[2], dl[2];   // Phi at p-2, p-1; d at p-2; L, C at p-3, p-2; delta at p-4, p-3
+    double ph[2], L[2], c[2], dl[2];   // Phi at p-2, p-1; L, C at p-3, p-2; delta at p-4, p-3
 
     __device__ __forceinline__ void init()
     {
-        ph[0] = ph[1] = df = L[0] = L[1] = c[0] = c[1] = dl[0] = dl[1] = 0.0;
+        ph[0] = ph[1] = L[0] = L[1] = c[0] = c[1] = dl[0] = dl[1] = 0.0;
     }
     __device__ __forceinline__ T push(double phi, double cn)
     {
-        double d;
-        const double Ln = lu(cn, ph[1], pick(sgn_bits(cn), ph[0], phi, ph[1]), d);
-        const double dn = delta_of(c[1], df, L[1], pick(sgn_bits(c[1]), Ln, L[0], L[1]));
+        const double Ln = lu(cn, ph[1], pick(sgn_bits(cn), ph[0], phi, ph[1]));
+        const double dn = delta_of(c[1], ph[0], L[1], pick(sgn_bits(c[1]), Ln, L[0], L[1]));
         const T out = T(cec_of(c[0], L[0], dl[1], pick(sgn_bits(c[0]), dl[0], dn, dl[1])));
         ph[0] = ph[1];
         ph[1] = phi;
-        df = d;
         L[0] = L[1];
         L[1] = Ln;
         c[0] = c[1];
@@ -233,7 +244,7 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
                     const double c = widen(s1[r * PW + j + 2]) * sx;
                     const T *q = sP + r * PW + j + 2;
                     sC[r * (TX + 4) + j] = c;
-                    sL[r * (TX + 4) + j] = lu(c, widen(q[0]), widen(q[-sgn_bits(c)]), sD[r * (TX + 4) + j]);
+                    sL[r * (TX + 4) + j] = lu(c, keep(q[0], sD[r * (TX + 4) + j]), widen(q[-sgn_bits(c)]));
                     if (j >= 2 && j < TX + 2) bad |= beyond_one(c);
                 });
                 __syncthreads();
@@ -241,7 +252,7 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
                     const double c = sC[r * (TX + 4) + j + 1];
                     const double *l = sL + r * (TX + 4) + j + 1;
                     double &d = sD[r * (TX + 4) + j + 1];
-                    d = delta_of(c, d, l[0], l[sgn_bits(c)]);
+                    d = delta_of(c, kept(sP[r * PW + j + 3], d), l[0], l[sgn_bits(c)]);
                 });
                 __syncthreads();
                 each<NT, TY + 6, TX>(tid, [&](int r, int x) {
@@ -255,7 +266,7 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
                     const double c = widen(s2[r * TX + x]) * sy;
                     const T *q = sS + (r + 1) * TX + x;
                     sC[r * TX + x] = c;
-                    sL[r * TX + x] = lu(c, widen(q[0]), widen(q[-sgn_bits(c) * TX]), sD[r * TX + x]);
+                    sL[r * TX + x] = lu(c, keep(q[0], sD[r * TX + x]), widen(q[-sgn_bits(c) * TX]));
                     if (r >= 2 && r < TY + 2) bad |= beyond_one(c);
                 });
                 __syncthreads();
@@ -263,7 +274,7 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
                     const double c = sC[(r + 1) * TX + x];
                     const double *l = sL + (r + 1) * TX + x;
                     double &d = sD[(r + 1) * TX + x];
-                    d = delta_of(c, d, l[0], l[sgn_bits(c) * TX]);
+                    d = delta_of(c, kept(sS[(r + 2) * TX + x], d), l[0], l[sgn_bits(c) * TX]);
                 });
                 __syncthreads();
                 // ---- the y sweep's value, then the cell's z window
@@ -303,7 +314,7 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
                     const double c = widen(s2[r * PW + j + 1]) * sy;
                     const T *q = src + (r + 1) * SW + j;
                     sC[r * CW + j] = c;
-                    sL[r * CW + j] = lu(c, widen(q[0]), widen(q[-sgn_bits(c) * SW]), sD[r * CW + j]);
+                    sL[r * CW + j] = lu(c, keep(q[0], sD[r * CW + j]), widen(q[-sgn_bits(c) * SW]));
                     if (r >= 2 && r < TY + 2 && j >= 3 && j < TX + 3) bad |= beyond_one(c);
                 });
                 __syncthreads();
@@ -311,7 +322,7 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
                     const double c = sC[(r + 1) * CW + j];
                     const double *l = sL + (r + 1) * CW + j;
                     double &d = sD[(r + 1) * CW + j];
-                    d = delta_of(c, d, l[0], l[sgn_bits(c) * CW]);
+                    d = delta_of(c, kept(src[(r + 2) * SW + j], d), l[0], l[sgn_bits(c) * CW]);
                 });
                 __syncthreads();
                 each<NT, TY, CW>(tid, [&](int r, int j) {                  // over sS: its z-swept values are spent
@@ -325,7 +336,7 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
                     const double c = widen(s3[r * PW + j + 2]) * sx;
                     const T *q = sS + r * CW + j + 1;
                     sC[r * (TX + 4) + j] = c;
-                    sL[r * (TX + 4) + j] = lu(c, widen(q[0]), widen(q[-sgn_bits(c)]), sD[r * (TX + 4) + j]);
+                    sL[r * (TX + 4) + j] = lu(c, keep(q[0], sD[r * (TX + 4) + j]), widen(q[-sgn_bits(c)]));
                     if (j >= 2 && j < TX + 2) bad |= beyond_one(c);
                 });
                 __syncthreads();
@@ -333,7 +344,7 @@ k_cec64(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel
                     const double c = sC[r * (TX + 4) + j + 1];
                     const double *l = sL + r * (TX + 4) + j + 1;
                     double &d = sD[r * (TX + 4) + j + 1];
-                    d = delta_of(c, d, l[0], l[sgn_bits(c)]);
+                    d = delta_of(c, kept(sS[r * CW + j + 2], d), l[0], l[sgn_bits(c)]);
                 });
                 __syncthreads();
                 each<NT, TY, TX>(tid, [&](int r, int x) {
