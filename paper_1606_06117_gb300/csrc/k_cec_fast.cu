@@ -1352,7 +1352,6 @@ k_cec_zyx_fast(const __grid_constant__ FastInst one, const __grid_constant__ Map
 #define SL_ZYX_SLOTS 3     // staged plane slots per CTA, z,y,x order
 #endif
 
-// Shared-memory opt-in and persistent grid size of one kernel, once per device.
 template <bool ZYX, bool BATCH, int CH>
 constexpr auto kernel_of()
 {
@@ -1363,43 +1362,26 @@ constexpr auto kernel_of()
 }
 
 template <bool ZYX, bool BATCH, int CH>
-cudaError_t prepare(int &grid, int &nsm)
+cudaError_t prepare(Residency &r)
 {
-    static int cached[64] = {}, count[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (cached[dev] == 0) {
-        auto kern = kernel_of<ZYX, BATCH, CH>();
-        const size_t smem = ZYX ? zyx::smem<SL_ZYX_SLOTS, CH>() : xyz::smem<SL_XYZ_SLOTS, CH>();
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
-        if (e != cudaSuccess) return e;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        count[dev] = sms;
-        cached[dev] = sms * (per_sm > 0 ? per_sm : 1);
-    }
-    grid = cached[dev];
-    nsm = count[dev];
-    return cudaSuccess;
+    static ResidencyCache cache;
+    return residency(cache, kernel_of<ZYX, BATCH, CH>(), NT,
+                     ZYX ? zyx::smem<SL_ZYX_SLOTS, CH>() : xyz::smem<SL_XYZ_SLOTS, CH>(), false, r);
 }
 
 template <bool ZYX, bool BATCH, int CH>
 cudaError_t go_fast(const FastInst &one, const MapsOf<CH> &maps, const FastInst *tab, int ninst, int64_t total,
                     unsigned *status, int grid_req, cudaStream_t st)
 {
-    int grid = 0, sms = 1;
-    cudaError_t e = prepare<ZYX, BATCH, CH>(grid, sms);
+    Residency res;
+    cudaError_t e = prepare<ZYX, BATCH, CH>(res);
     if (e != cudaSuccess) return e;
+    int grid = res.sms * res.per_sm;
     const int nf = tab ? 1 : one.nf;
     if (grid_req > 0)
         grid = grid_req;
     else if (!tab)   // a plane of one CTA per SM takes 0.7 of a plane of two (300^3)
-        grid = (int)plan_ctas(one.ntiles, one.nzr, kFastHaloBelow, 0.7, grid / sms, sms, nf) * nf;
+        grid = (int)plan_ctas(one.ntiles, one.nzr, kFastHaloBelow, 0.7, res.per_sm, res.sms, nf) * nf;
     if (grid > total) grid = (int)total;
     grid = grid >= nf ? grid / nf * nf : nf;   // whole groups of nf CTAs
     if (grid > total * nf) grid = (int)(total * nf);
@@ -1600,9 +1582,9 @@ cudaError_t launch_cec_fast(const FastInst &one, const FastInst *dev_table, int 
 
 int fast_grid(int parity)
 {
-    int g = 0, sms = 0;
-    if (((parity & 1) ? prepare<true, false, 0>(g, sms) : prepare<false, false, 0>(g, sms)) != cudaSuccess) return 0;
-    return g;
+    Residency r;
+    if (((parity & 1) ? prepare<true, false, 0>(r) : prepare<false, false, 0>(r)) != cudaSuccess) return 0;
+    return r.sms * r.per_sm;
 }
 
 }  // namespace sl

@@ -366,30 +366,17 @@ cudaError_t go(Geo g, const Launch &lc, const void *in, void *out, const void *v
 {
     using K = Lay<T, TY, HAS_Z, ZYX>;
     auto kern = k_cec64<T, TY, NT, HAS_Z, VEC, ZYX>;
-    // shared-memory opt-in and resident CTAs of the GPU, once per device
-    static int resident[64] = {}, sms[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static ResidencyCache cache;
+    Residency res;
+    const cudaError_t e = residency(cache, kern, NT, K::smem(), true, res);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (resident[dev] == 0) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem());
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, K::smem());
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        sms[dev] = n;
-        resident[dev] = n * (per_sm > 0 ? per_sm : 1);
-    }
     g.tiles_x = (g.nx + TX - 1) / TX;
     g.tiles_y = (g.ny + TY - 1) / TY;
     const int64_t tiles = (int64_t)g.tiles_x * g.tiles_y;
     const int64_t total = tiles * (g.tz > 0 ? g.chunks : g.nz);
     int64_t gr = total;
     if (HAS_Z && g.tz == 0)   // the FP64 pipe is shared: one CTA per SM is hardly slower per plane than half of two
-        gr = plan_ctas(tiles, g.nz, 6, 0.55, resident[dev] / sms[dev], sms[dev], fs.n);
+        gr = plan_ctas(tiles, g.nz, 6, 0.55, res.per_sm, res.sms, fs.n);
     if (lc.grid > 0 && lc.grid < gr) gr = lc.grid;
     if (gr < 1) gr = 1;
     if (gr > 0x7fffffff) return cudaErrorInvalidConfiguration;

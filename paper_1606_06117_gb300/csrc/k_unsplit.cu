@@ -398,23 +398,10 @@ cudaError_t go(Geo g, int grid, const void *in, void *out, const void *vel, cons
 {
     using K = Cfg<T, D, NST, TX, TY, HAS_Z>;
     auto kern = k_unsplit<T, D, NST, TX, TY, HAS_Z, VEC>;
-    // shared-memory opt-in and resident CTAs per SM, once per device
-    static int per_dev[64] = {}, sm_count[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static ResidencyCache cache;
+    Residency res;
+    const cudaError_t e = residency(cache, kern, K::NT, K::smem(), true, res);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (per_dev[dev] == 0) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem());
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, K::NT, K::smem());
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        sm_count[dev] = sms;
-        per_dev[dev] = sms * (per_sm > 0 ? per_sm : 1);
-    }
     g.tiles_y = (g.ny + TY - 1) / TY;
     const bool persist = HAS_Z && (NST == 3 || sizeof(D) == 8);
     const int64_t total = (int64_t)g.tiles_x * g.tiles_y * (persist ? g.nz : g.chunks);
@@ -422,8 +409,8 @@ cudaError_t go(Geo g, int grid, const void *in, void *out, const void *vel, cons
     // a plane of one CTA per SM takes 0.7 of a plane of two (FP32 BEC, 256^3), or
     // little more than half where they share the FP64 pipe
     if (persist && grid <= 0)
-        gr = (int)plan_ctas((int64_t)g.tiles_x * g.tiles_y, g.nz, 2 * NST, sizeof(D) == 8 ? 0.55 : 0.7, per_dev[dev] / sm_count[dev],
-                            sm_count[dev], fs.n);
+        gr = (int)plan_ctas((int64_t)g.tiles_x * g.tiles_y, g.nz, 2 * NST, sizeof(D) == 8 ? 0.55 : 0.7, res.per_sm, res.sms,
+                            fs.n);
     if (gr > total) gr = (int)total;
     kern<<<dim3(gr, fs.n), K::NT, K::smem(), st>>>(static_cast<const T *>(in), static_cast<T *>(out),
                                                    static_cast<const T *>(vel), g, fs.fin, fs.fout);

@@ -328,30 +328,17 @@ cudaError_t go(Geo g, int grid, const float *in, float *out, const float *vel, c
 {
     using K = Lay<NST>;
     auto kern = k_unsplit32<NST, BIG>;
-    // shared-memory opt-in and resident CTAs of the GPU, once per device
-    static int resident[64] = {}, sms[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static ResidencyCache cache;
+    Residency res;
+    const cudaError_t e = residency(cache, kern, K::NT, K::SMEM, true, res);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (resident[dev] == 0) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, K::NT, K::SMEM);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        sms[dev] = n;
-        resident[dev] = n * (per_sm > 0 ? per_sm : 1);
-    }
     g.tiles_x = (g.nx + TX - 1) / TX;
     g.tiles_y = (g.ny + TY - 1) / TY;
     const int64_t total = (int64_t)g.tiles_x * g.tiles_y * (g.tz > 0 ? g.chunks : g.nz);
     int64_t gr = total;
     // a plane of one CTA per SM takes 0.58 of a plane of two (BEC, 256^3)
     if (g.tz == 0)
-        gr = plan_ctas((int64_t)g.tiles_x * g.tiles_y, g.nz, 2 * NST, 0.58, resident[dev] / sms[dev], sms[dev], fs.n);
+        gr = plan_ctas((int64_t)g.tiles_x * g.tiles_y, g.nz, 2 * NST, 0.58, res.per_sm, res.sms, fs.n);
     if (grid > 0 && grid < total) gr = grid;
     if (gr < 1) gr = 1;
     if (gr > 0x7fffffff) return cudaErrorInvalidConfiguration;

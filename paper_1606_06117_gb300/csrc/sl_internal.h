@@ -5,6 +5,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "per_device.h"
 #include "sl_common.cuh"
 
 namespace sl {
@@ -47,6 +48,26 @@ cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, int block, size_t smem,
     cfg.attrs = &at;
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
+// Shared-memory opt-in of a kernel on the current device (carveout: all of the SM's
+// unified memory as shared, too) and its residency, once per device.
+template <typename K>
+cudaError_t residency(ResidencyCache &cache, K kern, int block, size_t smem, bool carveout, Residency &r)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= ResidencyCache::kDevices) return cudaErrorInvalidDevice;
+    if (cache.get(dev, r)) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && carveout) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.per_sm, kern, block, smem);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (r.per_sm < 1) r.per_sm = 1;
+    cache.set(dev, r);
+    return cudaSuccess;
 }
 
 // Several fields advected by one velocity in one launch: field f reads
