@@ -233,11 +233,16 @@ int sl_field_load(const char *path, void *field, int ndim, const int64_t dims[3]
  * dimensionality, sizes, 16-byte alignment); the autotuner chooses, by timing
  * on the caller's buffers, among launch shapes of that kernel that change only
  * how cells are grouped into work, never a cell's arithmetic, so every choice
- * gives bitwise the same results:
+ * gives bitwise the same results.  The launch an untuned step makes is always
+ * among them and is kept unless another one is faster:
  *   SL_KERNEL_CEC_FAST     persistent FP32 split CEC kernel (32 x 32 column
- *                          tiles): CTAs per SM, 1 or 2.
- *   SL_KERNEL_CEC_SPLIT    generic split CEC kernel: planes per work item, or for
- *                          SL_F64 and SL_F32_D64 in 3D persistent equal shares.
+ *                          tiles): CTAs per SM, 1 or 2 (2: the kernel's own
+ *                          division of the work, as untuned).
+ *   SL_KERNEL_CEC_SPLIT    split CEC on all other grids: planes per work item, or for
+ *                          SL_F64 and SL_F32_D64 in 3D persistent equal shares (0
+ *                          planes, as untuned).  In FP32 on 8 planes or more, 32
+ *                          planes (all, if there are fewer) stand for the kernel's
+ *                          own division of the work, as untuned.
  *   SL_KERNEL_CIR_GROUPS   FP32 CIR kernel on four-cell groups: tile height
  *                          16 or 32, planes per work item.
  *   SL_KERNEL_UNSPLIT      generic CIR / FEC / BEC kernels: on large FP32 3D grids
@@ -261,8 +266,8 @@ typedef struct {
     int kernel;       /* SL_KERNEL_*                                         */
     int tile_x;       /* column tile of a work item, cells along x           */
     int tile_y;       /*                             cells along y           */
-    int tile_z;       /* planes per work item; 0: persistent equal shares    */
-    int ctas_per_sm;  /* CTAs per SM of a persistent launch; 0: one per item  */
+    int tile_z;       /* planes per work item; 0: the kernel's own division  */
+    int ctas_per_sm;  /* CTAs per SM of a persistent launch; 0: not chosen   */
     float ms;         /* measured time of one step, milliseconds             */
 } sl_tuning;
 

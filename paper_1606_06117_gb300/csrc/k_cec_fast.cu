@@ -1378,7 +1378,7 @@ cudaError_t go_fast(const FastInst &one, const MapsOf<CH> &maps, const FastInst 
     if (e != cudaSuccess) return e;
     int grid = res.sms * res.per_sm;
     const int nf = tab ? 1 : one.nf;
-    if (grid_req > 0)
+    if (grid_req > 0 && grid_req != grid)   // all resident CTAs asked for: the default below
         grid = grid_req;
     else if (!tab)   // a plane of one CTA per SM takes 0.7 of a plane of two (300^3)
         grid = (int)plan_ctas(one.ntiles, one.nzr, kFastHaloBelow, 0.7, res.per_sm, res.sms, nf) * nf;
@@ -1508,6 +1508,8 @@ bool any_eligible(const int64_t dims[3], int ndim, int dtype)
     return dtype == 0 && ndim == 3 && dims[2] >= 8;
 }
 
+int any_default_tz(const int64_t dims[3]) { return (int)std::min<int64_t>(32, dims[2]); }
+
 cudaError_t launch_cec_any(const void *in, void *out, const void *vel, const int64_t dims[3], const double s[3],
                            int parity, Launch lc, unsigned *status, const FieldSet &fs, cudaStream_t st)
 {
@@ -1524,7 +1526,9 @@ cudaError_t launch_cec_any(const void *in, void *out, const void *vel, const int
             one.fin[i] = static_cast<const float *>(in) + (f0 + i) * fs.fin;
             one.fout[i] = static_cast<float *>(out) + (f0 + i) * fs.fout;
         }
-        int64_t grid = lc.tz > 0 ? (total + lc.tz - 1) / lc.tz * one.nf : 0;   // shares of lc.tz planes
+        // shares of lc.tz planes; any_default_tz stands for the default division
+        const bool shares = lc.tz > 0 && lc.tz != any_default_tz(dims);
+        int64_t grid = shares ? (total + lc.tz - 1) / lc.tz * one.nf : 0;
         if (grid > 0x7fffffff) grid = 0x7fffffff;
         cudaError_t e;
         if (parity & 1)

@@ -803,7 +803,9 @@ int sl_autotune_scheme(void *out, const void *in, const void *vel, int ndim, con
     const bool aligned = aligned16(out) && aligned16(in) && aligned16(vel);
     const int fam = family_of(scheme, dtype, ndim, dims, aligned);
 
-    // candidates: (tile height, planes per item, CTAs per SM); 0 = the default
+    // candidates: (tile height, planes per item, CTAs per SM); 0 = the default.  The
+    // first is the launch an untuned step makes, so that tuning never loses it; the
+    // family's numbers for it are those that launch_for turns back into that launch.
     struct Cand {
         int ty, tz, ctas;
     };
@@ -818,15 +820,16 @@ int sl_autotune_scheme(void *out, const void *in, const void *vel, int ndim, con
     }
     if (fam == SL_KERNEL_CEC_FAST) {
         const int occ = std::max(1, fast_grid(0) / c->num_sms);
-        for (int k = 1; k <= std::min(occ, 2); ++k) cands.push_back({0, 0, k});
+        for (int k = occ; k >= 1; --k) cands.push_back({0, 0, k});
     } else if (fam == SL_KERNEL_CEC_SPLIT) {
-        if (dtype != SL_F32 && ndim == 3) cands.push_back({0, 0, 0});   // equal shares
-        if (any_eligible(dims, ndim, dtype)) {                          // the default shares, as planes
-            const int64_t pairs = (dims[0] + 31) / 32 * ((dims[1] + 31) / 32) * dims[2], ctas = 2 * c->num_sms;
-            cands.push_back({0, (int)std::max<int64_t>(1, (pairs + ctas - 1) / ctas), 0});
-        }
-        for (int tz : tzs) cands.push_back({0, tz, 0});
+        const int own = any_eligible(dims, ndim, dtype) ? any_default_tz(dims)
+                        : dtype != SL_F32 && ndim == 3  ? 0   // equal shares
+                                                        : default_tz(dtype, ndim, dims);
+        cands.push_back({0, own, 0});
+        for (int tz : tzs)
+            if (tz != own) cands.push_back({0, tz, 0});
     } else if (fam == SL_KERNEL_CIR_GROUPS) {
+        cands.push_back({0, 0, 0});
         for (int ty : {16, 32})
             if (ty == 16 || dims[1] >= 32)
                 for (int tz : tzs) cands.push_back({ty, tz, 0});
@@ -836,6 +839,7 @@ int sl_autotune_scheme(void *out, const void *in, const void *vel, int ndim, con
             for (int k = 0; k <= 2; ++k) cands.push_back({0, 0, k});   // equal shares
             for (int tz : tzs) cands.push_back({0, tz, 0});
         } else {
+            if (ndim == 3) cands.push_back({0, 0, 0});
             std::vector<int> tys = {0};
             if (dtype == SL_F32 && ndim == 3) tys = {8, 16, 32};
             for (int ty : tys) {

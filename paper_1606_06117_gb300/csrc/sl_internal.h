@@ -175,8 +175,12 @@ cudaError_t launch_cec_fast(const FastInst &one, const FastInst *dev_table, int 
                             unsigned *status, int grid_req, cudaStream_t st);
 int fast_grid(int parity);
 // The same kernels on FP32 3D grids of any x and y size and alignment (nz >= 8);
-// lc.tz > 0: CTAs take shares of that many planes.
+// lc.tz > 0: CTAs take shares of that many planes, except that any_default_tz planes
+// stand for the kernels' own division (plan_ctas).  A tuned shape of this family is
+// planes per work item, which the generic batched kernel takes too: its default, 32
+// planes, there and here leaves each kernel its default.
 bool any_eligible(const int64_t dims[3], int ndim, int dtype);
+int any_default_tz(const int64_t dims[3]);
 cudaError_t launch_cec_any(const void *in, void *out, const void *vel, const int64_t dims[3], const double s[3],
                            int parity, Launch lc, unsigned *status, const FieldSet &fs, cudaStream_t st);
 
