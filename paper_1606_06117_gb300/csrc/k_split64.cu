@@ -392,12 +392,7 @@ cudaError_t by_order(int parity, const Geo &g, const Launch &lc, const void *in,
         return (parity & 1) ? go<T, 16, 256, true, VEC, true>(g, lc, in, out, vel, fs, st)
                             : go<T, 16, 256, true, VEC, false>(g, lc, in, out, vel, fs, st);
     } else {
-        // Small planes take 4-row tiles, which spread them over more SMs: the
-        // 32 x 16 tiles of a 128^2 plane would leave 120 of 152 SMs idle, and the
-        // wider halo (about 38 double operations per cell in place of 24) costs less than that
-        // until the larger tiles give every SM two CTAs.
-        const int64_t big = (int64_t)((g.nx + TX - 1) / TX) * ((g.ny + 15) / 16) * fs.n;
-        if (big < 2 * 152)
+        if (split64_tile_y(false, g.nx, g.ny, fs.n) == 4)
             return (parity & 1) ? go<T, 4, 128, false, VEC, true>(g, lc, in, out, vel, fs, st)
                                 : go<T, 4, 128, false, VEC, false>(g, lc, in, out, vel, fs, st);
         return (parity & 1) ? go<T, 16, 256, false, VEC, true>(g, lc, in, out, vel, fs, st)
@@ -406,6 +401,15 @@ cudaError_t by_order(int parity, const Geo &g, const Launch &lc, const void *in,
 }
 
 }  // namespace
+
+// Small planes take 4-row tiles, which spread them over more SMs: the 32 x 16 tiles of
+// a 128^2 plane would leave 120 of 152 SMs idle, and the wider halo (about 38 double
+// operations per cell in place of 24) costs less than that until the larger tiles
+// give every SM two CTAs.
+int split64_tile_y(bool has_z, int64_t nx, int64_t ny, int fields)
+{
+    return !has_z && (nx + TX - 1) / TX * ((ny + 15) / 16) * fields < 2 * 152 ? 4 : 16;
+}
 
 cudaError_t launch_split_cec64(bool f32_storage, Geo g, int parity, Launch lc, bool has_z, const void *in, void *out,
                                const void *vel, const FieldSet &fs, cudaStream_t st)

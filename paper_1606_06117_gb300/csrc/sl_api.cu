@@ -149,11 +149,11 @@ int family_of(int scheme, int dtype, int ndim, const int64_t dims[3], bool align
 }
 
 // Tile height of a family's launch with no height chosen (the kernels' defaults).
-int default_ty(int fam, int dtype)
+int default_ty(int fam, int dtype, int ndim, const int64_t dims[3])
 {
     switch (fam) {
     case SL_KERNEL_CEC_FAST: return 32;
-    case SL_KERNEL_CEC_SPLIT: return dtype == SL_F64 ? 16 : 32;
+    case SL_KERNEL_CEC_SPLIT: return dtype == SL_F32 ? 32 : split64_tile_y(ndim == 3, dims[0], dims[1], 1);
     case SL_KERNEL_CIR_GROUPS: return 16;
     default: return dtype == SL_F64 ? 8 : 16;
     }
@@ -887,7 +887,7 @@ int sl_autotune_scheme(void *out, const void *in, const void *vel, int ndim, con
     sl_tuning t;
     t.kernel = fam;
     t.tile_x = 32;
-    t.tile_y = pick.ty > 0 ? pick.ty : default_ty(fam, dtype);
+    t.tile_y = pick.ty > 0 ? pick.ty : default_ty(fam, dtype, ndim, dims);
     if (fam == SL_KERNEL_CIR_GROUPS && t.tile_y == 32 && dims[1] < 32) t.tile_y = 16;
     t.tile_z = pick.tz;
     t.ctas_per_sm = pick.ctas;
@@ -981,7 +981,10 @@ int sl_tuning_load(const char *path)
         const bool ok = n == 11 && nx >= 1 && ny >= 1 && nz >= 1 && nx <= (1ll << 30) && ny <= (1ll << 30) &&
                         nz <= (1ll << 30) && scheme >= SL_CIR && scheme <= SL_CEC && dtype >= SL_F32 &&
                         dtype <= SL_F32_D64 && kernel >= SL_KERNEL_CEC_FAST && kernel <= SL_KERNEL_UNSPLIT &&
-                        tx == 32 && (ty == 8 || ty == 16 || ty == 32) && tz >= 0 && tz <= (1 << 30) && ctas >= 0 &&
+                        tx == 32 &&
+                        (ty == 8 || ty == 16 || ty == 32 ||
+                         (ty == 4 && kernel == SL_KERNEL_CEC_SPLIT && dtype != SL_F32)) &&   // its small planes
+                        tz >= 0 && tz <= (1 << 30) && ctas >= 0 &&
                         ctas <= 32 && std::isfinite(ms);
         if (!ok) {
             std::fclose(f);

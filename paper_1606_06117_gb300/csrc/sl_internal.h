@@ -88,6 +88,7 @@ cudaError_t launch_split_cec(int dtype, const void *in, void *out, const void *v
 // shares), its tiles are set by the launch (k_split64.cu).
 cudaError_t launch_split_cec64(bool f32_storage, Geo g, int parity, Launch lc, bool has_z, const void *in, void *out,
                                const void *vel, const FieldSet &fs, cudaStream_t st);
+int split64_tile_y(bool has_z, int64_t nx, int64_t ny, int fields);   // its tile height
 cudaError_t launch_unsplit(int dtype, int scheme, const void *in, void *out, const void *vel,
                            int ndim, const int64_t dims[3], const double s[3], Launch lc,
                            unsigned *status, cudaStream_t st, FieldSet fs = FieldSet());

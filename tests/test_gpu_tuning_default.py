@@ -89,3 +89,20 @@ def test_planes_filed_for_batch_plans_are_no_fewer_than_those_tried():
     phi, vel, sp, dt = inputs(shape, sl.F32)
     t = sl.sl_autotune_scheme(torch.empty_like(phi), phi, vel, 3, list(shape[::-1]), sp, dt, sl.CEC, sl.F32)
     assert t.kernel == 2 and t.tile_z in (8, 16, 24)
+
+
+@pytest.mark.parametrize("shape,dtype,tile_y", [((20, 40, 50), sl.F32_D64, 16), ((20, 40, 50), sl.F64, 16),
+                                                ((128, 128), sl.F64, 4), ((128, 128), sl.F32_D64, 4),
+                                                ((600, 520), sl.F64, 16)])
+def test_double_cec_files_the_tile_height_it_runs(tmp_path, shape, dtype, tile_y):
+    t = torch.float64 if dtype == sl.F64 else torch.float32
+    dims = (list(shape[::-1]) + [1])[:3]
+    phi = torch.rand(shape, device=DEV, dtype=t)
+    vel = torch.rand((len(shape),) + shape, device=DEV, dtype=t)
+    args = (phi, vel, len(shape), dims, [1.0] * 3, 0.5)
+    got = sl.sl_autotune_scheme(torch.empty_like(phi), *args, sl.CEC, dtype)
+    assert (got.kernel, got.tile_y) == (2, tile_y)
+    sl.sl_tuning_save(str(tmp_path / "t.txt"))
+    sl.sl_tuning_clear()
+    sl.sl_tuning_load(str(tmp_path / "t.txt"))
+    assert sl.sl_tuning_get(dims, sl.CEC, dtype).tile_y == tile_y
