@@ -46,7 +46,6 @@
 // small boxes only.
 #include <cmath>
 #include <new>
-#include <vector>
 
 #include "sl.h"
 #include "sl_internal.h"
@@ -241,7 +240,7 @@ __host__ __device__ constexpr int64_t rb_pad(int64_t n)
 // (lam_kj = lz[k] + lx[j]; the constant mode F[0] of k = 0 is 0); phi = C_z^T G is
 // left to the projection.  The last two are one linear map of a row, so
 //   G[k] = R M_k,  M_k[i][i'] = sum_{j, lam_kj != 0} C_x[j][i] C_x[j][i'] / lam_kj
-// with the matrices M_k computed once per box: a third of the FP64 sums and all
+// with the matrices M_k made once per box (k_rb_green): a third of the FP64 sums and all
 // divisions less per step (FP64 CEC, 50 x 50: 17.8 -> 16.3 us per step, 128 x 128: 58 ->
 // 51, 400 x 50: 175 -> 110).  Forms:
 //   kLarge   M would take more than kRbGreenMax, or FP32 boxes that are not staged
@@ -283,22 +282,93 @@ k_rb_modes(const T *D, const T *cz, const T *cx, const T *cxT, const T *M, const
                  [&](int, int i, T v) { Gk[i] = v; });
 }
 
-// M of one box, summed in double: thread (i, i') of mode k = blockIdx.y; the CTA's
-// 1 / lam_kj once in shared memory (a division per term took most of the time).
+// The tables of a box, made on the device.  Measured, ms to create an FP64 box with host
+// tables and no M, with host tables and M as a sum over the modes, and now: 50 x 50
+// 0.12 / 0.17 / 0.06, 300 x 200 1.6 / 20.8 / 0.6, 1024 x 32 13 / 134 / 0.8, 48 x 4096
+// 157 / 320 / 5.7.
+//
+// Element (j, i) of the orthonormal DCT-II matrix, s_j cos(pi j (i + 1/2) / n); the
+// angle in units of pi / (2 n) is an integer, reduced to [0, n] exactly.
+__device__ __forceinline__ double rb_cosine(int j, int i, int n)
+{
+    int r = (int)((int64_t)j * (2 * i + 1) % (4 * n));
+    if (r > 2 * n) r = 4 * n - r;
+    const bool neg = r > n;
+    if (neg) r = 2 * n - r;
+    const double c = sqrt((j == 0 ? 1.0 : 2.0) / n) * cospi((double)r / (2.0 * n));
+    return neg ? -c : c;
+}
+
+// C (row j), and where they are wanted its transpose and, transposed, the differences
+// of the rows around each (k_rb_project); the eigenvalues per axis.
 template <typename T>
-__global__ void k_rb_green(const T *cx, const T *lx, const T *lz, T *M, int nx)
+__global__ void k_rb_tables(T *c, T *ct, T *zt, T *lam, int n, double h)
+{
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= (int64_t)n * n) return;
+    const int a = (int)(e / n), b = (int)(e % n);
+    c[e] = T(rb_cosine(a, b, n));
+    if (ct) ct[e] = T(rb_cosine(b, a, n));
+    if (zt) zt[e] = T(rb_cosine(b, a + 1 < n ? a + 1 : a, n) - rb_cosine(b, a > 0 ? a - 1 : a, n));
+    if (a == 0) {
+        const double s = sinpi((double)b / (2.0 * n));
+        lam[b] = T(-4.0 / (h * h) * (s * s));
+    }
+}
+
+// M of one box.  M_k inverts the tridiagonal matrix lap_x + lz_k, so it has a closed form:
+// with s = dx / dz sin(pi k / (2 nz)), theta = 2 asinh(s), i <= i' (and symmetric)
+//   M_k[i][i'] = -dx^2 cosh((i + 1/2) theta) cosh((nx - i' - 1/2) theta) / (sinh(theta) sinh(nx theta)),
+// written with decaying exponentials; for k = 0 the inverse on vectors of zero mean,
+//   dx^2 (max(x, x') - (x^2 + x'^2) / (2 nx) - nx / 3 + 1 / (12 nx)),   x = i + 1/2.
+// (Its error against extended precision is a few units in the last place, that of the
+// sum over the modes up to thirty.)  One CTA of mode k = blockIdx.y takes every
+// gridDim.x-th row.
+template <typename T>
+__global__ void k_rb_green(T *M, int nx, int nz, double dx, double dz)
 {
     extern __shared__ __align__(16) unsigned char rb_smem[];
-    double *inv = reinterpret_cast<double *>(rb_smem);
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nn = (int64_t)nx * nx;
-    const int k = blockIdx.y, i = (int)(e / nx), i2 = (int)(e % nx);
-    for (int j = threadIdx.x; j < nx; j += blockDim.x)
-        inv[j] = k == 0 && j == 0 ? 0.0 : 1.0 / ((double)lz[k] + (double)lx[j]);
+    double *decay = reinterpret_cast<double *>(rb_smem);   // exp(-i theta)
+    __shared__ double mode[3];
+    const int k = blockIdx.y;
+    if (k && threadIdx.x == 0) {   // once: every thread would wait for the FP64 pipe
+        const double sn = sinpi((double)k / (2.0 * nz)), s = dx / dz * sn, theta = 2.0 * asinh(s);
+        mode[0] = theta;
+        mode[1] = dz / (2.0 * sn) * (dx / (2.0 * hypot(1.0, s))) / expm1(-2.0 * nx * theta);
+        mode[2] = exp(-theta);
+    }
     __syncthreads();
-    if (e >= nn) return;
-    double acc = 0.0;
-    for (int j = 0; j < nx; ++j) acc += (double)cx[(int64_t)j * nx + i] * inv[j] * (double)cx[(int64_t)j * nx + i2];
-    M[k * rb_pad<T>(nn) + e] = T(acc);
+    if (k)
+        for (int i = threadIdx.x; i < nx; i += blockDim.x) decay[i] = exp(-i * mode[0]);
+    __syncthreads();
+    const double scale = mode[1], half = mode[2];
+    T *Mk = M + k * rb_pad<T>((int64_t)nx * nx);
+    for (int i = blockIdx.x; i < nx; i += gridDim.x)
+        for (int i2 = threadIdx.x; i2 < nx; i2 += blockDim.x) {
+            const int lo = min(i, i2), hi = max(i, i2);
+            double v;
+            if (k) {
+                const double p = decay[lo], q = decay[nx - 1 - hi];
+                v = scale * decay[hi - lo] * (1.0 + p * p * half) * (1.0 + q * q * half);
+            } else {
+                const double x = lo + 0.5, y = hi + 0.5;
+                v = dx * dx * (y - (x * x + y * y) / (2.0 * nx) - (nx / 3.0 - 1.0 / (12.0 * nx)));
+            }
+            Mk[(int64_t)i * nx + i2] = T(v);
+        }
+}
+
+template <typename T>
+cudaError_t rb_tables(void *cx, void *cxT, void *cz, void *czT, void *zT, void *lx, void *lz, void *M, int nx, int nz,
+                      double dx, double dz)
+{
+    auto blocks = [](int n) { return (unsigned)(((int64_t)n * n + 63) / 64); };   // small, to spread over the SMs
+    k_rb_tables<T><<<blocks(nx), 64>>>(static_cast<T *>(cx), static_cast<T *>(cxT), static_cast<T *>(nullptr),
+                                        static_cast<T *>(lx), nx, dx);
+    k_rb_tables<T><<<blocks(nz), 64>>>(static_cast<T *>(cz), static_cast<T *>(czT), static_cast<T *>(zT),
+                                        static_cast<T *>(lz), nz, dz);
+    if (M) k_rb_green<T><<<dim3(nx < 256 ? (nx + 7) / 8 : 32, nz), 256, sizeof(double) * nx>>>(static_cast<T *>(M), nx, nz, dx, dz);
+    return cudaGetLastError();
 }
 
 // Projection, one CTA per row m: phi[m][i] = sum_k C_z[k][m] G[k][i] and the
@@ -552,15 +622,6 @@ int rb_graph(sl_rb *r, double dt)
     return SL_OK;
 }
 
-// orthonormal DCT-II matrix, row j: s_j cos(pi j (i + 1/2) / n)
-void dct_matrix(std::vector<double> &c, int n)
-{
-    c.resize((size_t)n * n);
-    for (int j = 0; j < n; ++j)
-        for (int i = 0; i < n; ++i)
-            c[(size_t)j * n + i] = std::sqrt((j == 0 ? 1.0 : 2.0) / n) * std::cos(M_PI * j * (i + 0.5) / n);
-}
-
 }  // namespace
 
 extern "C" {
@@ -638,50 +699,13 @@ int sl_rb_create(sl_rb **out, int nx, int nz, double Lx, double Lz, double Ra, d
     r->zT = take((int64_t)nz * nz);
     if (melems) r->M = take(melems);
     r->signs = reinterpret_cast<int *>(p);
-    std::vector<double> cxm, czm, cxt((size_t)nx * nx), lxv(nx), lzv(nz);
-    dct_matrix(cxm, nx);
-    for (int j = 0; j < nx; ++j)
-        for (int i = 0; i < nx; ++i) cxt[(size_t)i * nx + j] = cxm[(size_t)j * nx + i];
-    dct_matrix(czm, nz);
-    std::vector<double> czt((size_t)nz * nz), zt((size_t)nz * nz);
-    for (int k = 0; k < nz; ++k)
-        for (int m = 0; m < nz; ++m) {
-            const double *row = czm.data() + (size_t)k * nz;
-            czt[(size_t)m * nz + k] = row[m];
-            zt[(size_t)m * nz + k] = row[m + 1 < nz ? m + 1 : m] - row[m > 0 ? m - 1 : m];
-        }
     const double dx = Lx / nx, dz = Lz / nz;
-    for (int j = 0; j < nx; ++j) lxv[j] = -4.0 / (dx * dx) * std::pow(std::sin(M_PI * j / (2.0 * nx)), 2);
-    for (int k = 0; k < nz; ++k) lzv[k] = -4.0 / (dz * dz) * std::pow(std::sin(M_PI * k / (2.0 * nz)), 2);
     const int signs[6] = {-1, -1, 1, -1, -1, -1};   // sx of u, w, theta; sz of u, w, theta
     cudaError_t e = cudaMemset(r->mem, 0, r->esz * elems);
-    auto up = [&](void *dst, const std::vector<double> &v) {
-        if (e != cudaSuccess) return;
-        if (dtype == SL_F64) {
-            e = cudaMemcpy(dst, v.data(), 8 * v.size(), cudaMemcpyHostToDevice);
-        } else {
-            const std::vector<float> f(v.begin(), v.end());
-            e = cudaMemcpy(dst, f.data(), 4 * f.size(), cudaMemcpyHostToDevice);
-        }
-    };
-    up(r->cx, cxm);
-    if (!melems) up(r->cxT, cxt);
-    up(r->lx, lxv);
-    up(r->lz, lzv);
-    up(r->cz, czm);
-    up(r->czT, czt);
-    up(r->zT, zt);
-    if (e == cudaSuccess && r->M) {
-        const dim3 grid((unsigned)(((int64_t)nx * nx + 255) / 256), (unsigned)nz);
-        if (dtype == SL_F64)
-            k_rb_green<<<grid, 256, 8 * nx>>>(static_cast<const double *>(r->cx), static_cast<const double *>(r->lx),
-                                              static_cast<const double *>(r->lz), static_cast<double *>(r->M), nx);
-        else
-            k_rb_green<<<grid, 256, 8 * nx>>>(static_cast<const float *>(r->cx), static_cast<const float *>(r->lx),
-                                              static_cast<const float *>(r->lz), static_cast<float *>(r->M), nx);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
-    }
+    if (e == cudaSuccess)
+        e = dtype == SL_F64 ? rb_tables<double>(r->cx, r->cxT, r->cz, r->czT, r->zT, r->lx, r->lz, r->M, nx, nz, dx, dz)
+                            : rb_tables<float>(r->cx, r->cxT, r->cz, r->czT, r->zT, r->lx, r->lz, r->M, nx, nz, dx, dz);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e == cudaSuccess) e = cudaMemcpy(r->signs, signs, sizeof signs, cudaMemcpyHostToDevice);
     // small boxes stage the transforms' operands in shared memory; the kernels'
     // limit is per function, not per box, so it is raised to the cap that every

@@ -70,3 +70,21 @@ def test_a_form_matches_the_oracle(nx, nz, dtype):
         g.close()
     for name, a, b in zip(("u", "w", "theta"), got, (box.u, box.w, box.theta)):
         assert_parity(a, b, dtype, f"{nx}x{nz} {name}", T.allowance(nx, nz, steps, f64=dtype == "f64"))
+
+
+@pytest.mark.parametrize("nx,nz", [(1024, 32), (2800, 4), (48, 2048)])
+def test_creating_a_box_costs_no_more_than_a_few_hundred_steps(nx, nz):
+    """The tables of a box are a few passes over nx^2 nz (where it keeps them) and nz^2
+    elements, below 0.3 GB: a millisecond or two on the device, no host loops over
+    them (134 and 402 ms for the first two with host tables and a sum per element).  The
+    bound is several times that, for the allocation and a busy host."""
+    import time
+    best = 1e9
+    for _ in range(5):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        h = sl.sl_rb_create(nx, nz, scheme="CEC", dtype=sl.F64)
+        torch.cuda.synchronize()
+        best = min(best, time.perf_counter() - t)
+        sl.sl_rb_destroy(h)
+    assert best < 0.02, best
