@@ -355,9 +355,14 @@ bool unsplit32_serves(int scheme, int ndim, const int64_t dims[3], bool vec)
     if (!vec) return true;
     // by the (column tile, plane) pairs of the grid: FEC crosses over between 2600
     // (48 x 200 x 100: 20.4 against 21.6 us) and 4096 (128^3: 25.4 against 24.9), BEC
-    // between 8000 (160^3: 61.3 against 62.6) and 11200 (256 x 100 x 200: 91 against 87)
-    const int64_t pairs = ((dims[0] + TX - 1) / TX) * ((dims[1] + TY - 1) / TY) * dims[2];
-    return pairs < (scheme == 2 ? 9000 : 3000);
+    // between 8000 (160^3: 61.3 against 62.6) and 11200 (256 x 100 x 200: 91 against 87).
+    // Not where the tiles alone fill the SMs and have few planes: the equal shares then
+    // cut most tiles, and each cut warms up again (FEC 300 x 300 x 7 16.1 against 13.7 us,
+    // 512 x 512 x 5 27.4 against 18.0; BEC 512 x 512 x 8 50.8 against 48.3, x 11 59.5
+    // against 62.2, 2048 x 2048 x 1 263 against 224).
+    const int64_t tiles = ((dims[0] + TX - 1) / TX) * ((dims[1] + TY - 1) / TY);
+    const bool few_tiles = tiles < 152;
+    return scheme == 2 ? tiles * dims[2] < 9000 && (few_tiles || dims[2] >= 10) : tiles * dims[2] < 3000 && few_tiles;
 }
 
 cudaError_t launch_unsplit32(int scheme, Geo g, int grid, const void *in, void *out, const void *vel,
