@@ -468,6 +468,11 @@ __device__ __forceinline__ bool wg_or(int g, bool v)
 // One learned step over the grid; one cell per thread per tile.  wb points at
 // the BF16 operand images of W1 and W2 (already in the core-matrix layout, biases
 // included) followed by w3, b3 in FP32.
+// A CTA's warpgroups take neighbouring tiles; SPREAD, for grids of at most a tile per
+// warpgroup of the GPU: the CTAs take tiles in turn first, so that all SMs get some (32 x 16
+// x 8: 7.2 us by neighbours, 5.4 in turn).  Two kernels: chosen at run time the order
+// costs registers that spill (256^3 557 -> 614 us).
+template <bool SPREAD>
 __global__ void __launch_bounds__(NT_STEP, 1)
 k_learned_step(const float *__restrict__ phi, float *__restrict__ out, const float *__restrict__ vel, int nx, int ny,
                int nz, float sx, float sy, float sz, const unsigned char *__restrict__ wb, unsigned *status)
@@ -510,7 +515,7 @@ k_learned_step(const float *__restrict__ phi, float *__restrict__ out, const flo
     // tile (tx, ty, z) of this warpgroup, and the step to its next one
     const int tiles_x = nx / BX, tiles_y = ny / BY;
     const int64_t ntiles = (int64_t)tiles_x * tiles_y * nz, hop = (int64_t)gridDim.x * WGS;
-    const int64_t first = (int64_t)blockIdx.x * WGS + wg;
+    const int64_t first = SPREAD ? (int64_t)wg * gridDim.x + blockIdx.x : (int64_t)blockIdx.x * WGS + wg;
     const int hx = (int)(hop % tiles_x), hy = (int)(hop / tiles_x % tiles_y), hz = (int)(hop / ((int64_t)tiles_x * tiles_y));
     int tx = (int)(first % tiles_x), ty = (int)(first / tiles_x % tiles_y), z = (int)(first / ((int64_t)tiles_x * tiles_y));
     auto advance = [&](int &x, int &y, int &zz) {
@@ -926,19 +931,15 @@ int sl_advect_learned(sl_corrector *c, void *out, const void *in, const void *ve
     if (!ctx) return lfail(SL_ERR_CUDA, "no device context");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     auto learned = [&](void *dst) {
-        static int smem_set[64] = {};
-        if (!smem_set[ctx->device]) {
-            if (cudaFuncSetAttribute(k_learned_step, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess)
-                return cudaErrorInvalidValue;
-            // all of the SM's unified L1 / shared memory as shared
-            if (cudaFuncSetAttribute(k_learned_step, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
-                return cudaErrorInvalidValue;
-            smem_set[ctx->device] = 1;
-        }
         const int64_t tiles = (dims[0] / BX) * (dims[1] / BY) * dims[2];
-        const int64_t ctas = (tiles + WGS - 1) / WGS;
-        const int grid = ctas < ctx->num_sms ? (int)ctas : ctx->num_sms;   // one per SM: each holds its TMEM
-        k_learned_step<<<grid, NT_STEP, SMEM_BYTES, st>>>(
+        const bool spread = tiles <= (int64_t)ctx->num_sms * WGS;
+        const auto kern = spread ? k_learned_step<true> : k_learned_step<false>;
+        static ResidencyCache cache[2];
+        Residency res;
+        const cudaError_t e = residency(cache[spread], kern, NT_STEP, SMEM_BYTES, true, res);
+        if (e != cudaSuccess) return e;
+        const int grid = tiles < res.sms ? (int)tiles : res.sms;   // one per SM: each holds its TMEM
+        kern<<<grid, NT_STEP, SMEM_BYTES, st>>>(
             static_cast<const float *>(in), static_cast<float *>(dst), static_cast<const float *>(vel), (int)dims[0],
             (int)dims[1], (int)dims[2], (float)(dt / spacing[0]), (float)(dt / spacing[1]), (float)(dt / spacing[2]),
             c->wb, ctx->status);
