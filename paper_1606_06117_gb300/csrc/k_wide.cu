@@ -266,7 +266,10 @@ __device__ __forceinline__ bool below(double c, int n)
 // Persistent CTAs; the loads of a CTA's next tile are issued before it works on
 // the current one, so that DRAM latency runs under the three gathers (without
 // that the y and z sweeps stalled on their loads).
-template <typename T, int AX, int LW, int NT>
+// PART: tiles of so few cells that a thread has none in its last turns; these are
+// skipped, which pays where double operations bound (8^3 SL_F64, a step of each order:
+// 50.7 -> 21.5 us; with the test in full tiles, 256^3, 3438 -> 3871).
+template <typename T, int AX, int LW, int NT, bool PART>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 1024 / NT : 1)
 k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict__ vel, WideGeo g, T sc, int rows,
              int tiles)
@@ -292,6 +295,8 @@ k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict
     // place.  Cells beyond the tile's lines go to the spare place, and cells of a
     // partial tile beyond the grid work on zeros in places of their own.
     const int count = AX == 0 ? rows * n : n << LW;
+    const int turns = (count + NT - 1) / NT;
+    auto has = [&](int k) { return !PART || k < turns; };
     int pos[E], line[E], own[E];
     bool rep[E];                                       // repeated at its line's end
     if constexpr (AX == 0) {
@@ -344,6 +349,7 @@ k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict
         }
 #pragma unroll
         for (int k = 0; k < E; ++k) {
+            if (!has(k)) break;
             const bool ok = k * NT < limit;
             v[k] = ok ? src[q0 + k * hop] : T(0);
             c[k] = ok ? va[q0 + k * hop] : T(0);
@@ -356,6 +362,7 @@ k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict
         bool far = false;
 #pragma unroll
         for (int k = 0; k < E; ++k) {
+            if (!has(k)) break;
             c[k] *= sc;
             far |= !below(c[k], n);
         }
@@ -363,6 +370,7 @@ k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict
         if (!__any_sync(0xffffffffu, far)) {
 #pragma unroll
             for (int k = 0; k < E; ++k) {
+            if (!has(k)) break;
                 const T f = trunc(c[k]);
                 m[k] = (int)f;
                 r[k] = c[k] - f;
@@ -370,6 +378,7 @@ k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict
         } else {   // a period or more somewhere, or a number that cannot be used
 #pragma unroll
             for (int k = 0; k < E; ++k) {
+            if (!has(k)) break;
                 if (!(fabs(c[k]) < T(1073741824.0))) {
                     bad = true;
                     c[k] = T(0);
@@ -381,6 +390,7 @@ k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict
         }
 #pragma unroll
         for (int k = 0; k < E; ++k) {
+            if (!has(k)) break;
             const int d = m[k] * step;
             lo[k] = line[k] + wrap3(pos[k] - d - (positive(r[k]) ? step : 0), period);
             back[k] = LB + line[k] + wrap3(pos[k] + d - (positive(-r[k]) ? step : 0), period);
@@ -390,27 +400,33 @@ k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict
         const int climit = limit;
         __syncthreads();   // the previous tile's delta has been read
 #pragma unroll
-        for (int k = 0; k < E; ++k) put(0, k, phi[k]);
+        for (int k = 0; k < E; ++k)
+            if (has(k)) put(0, k, phi[k]);
         if (b + (int)gridDim.x < tiles) load(b + gridDim.x);
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < E; ++k) {                                     // L_U[Phi]
+            if (!has(k)) break;
             const T a = lds(lo[k]), d = lds(lo[k] + step);
             L[k] = a + ((positive(r[k]) ? T(1) : T(0)) - r[k]) * (d - a);
         }
 #pragma unroll
-        for (int k = 0; k < E; ++k) put(LB, k, L[k]);
+        for (int k = 0; k < E; ++k)
+            if (has(k)) put(LB, k, L[k]);
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < E; ++k) {                                     // delta = Phi - L_{-U}[L_U[Phi]]
+            if (!has(k)) break;
             const T a = lds(back[k]), d = lds(back[k] + step);
             phi[k] -= a + ((positive(-r[k]) ? T(1) : T(0)) + r[k]) * (d - a);
         }
 #pragma unroll
-        for (int k = 0; k < E; ++k) put(0, k, phi[k]);
+        for (int k = 0; k < E; ++k)
+            if (has(k)) put(0, k, phi[k]);
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < E; ++k) {                                     // departure-cell correction
+            if (!has(k)) break;
             const T a = lds(lo[k]), d = lds(lo[k] + step);
             const T dj = positive(r[k]) ? d : a;
             const T du = positive(-r[k]) ? d : a;                             // r = 0: the cell itself
@@ -421,30 +437,30 @@ k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict
     flag_cfl(g.status, bad);
 }
 
-template <typename T, int AX, int LW, int NT>
+template <typename T, int AX, int LW, int NT, bool PART>
 cudaError_t go_sweep(T *dst, const T *src, const T *vel, const WideGeo &g, int rows, unsigned tiles, cudaStream_t st)
 {
     // at most NT kSweepCells cells and their repeated elements, in two arrays
     constexpr size_t cap = 2 * sizeof(T) * (size_t)(NT * kSweepCells + 1 + (AX == 0 ? 256 : 1 << LW));
-    static int ready[64] = {};   // resident CTAs of the GPU
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static ResidencyCache cache;
+    Residency res;
+    const cudaError_t e = residency(cache, k_wide_sweep<T, AX, LW, NT, PART>, NT, cap, false, res);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!ready[dev]) {
-        e = cudaFuncSetAttribute(k_wide_sweep<T, AX, LW, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wide_sweep<T, AX, LW, NT>, NT, cap);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        ready[dev] = sms * (per_sm > 0 ? per_sm : 1);
-    }
     const size_t lines = AX == 0 ? (size_t)rows : (size_t)1 << LW;
     const size_t smem = 2 * sizeof(T) * (lines * (size_t)(g.n[AX] + 1) + 1);
-    const unsigned grid = std::min(tiles, (unsigned)ready[dev]);
-    k_wide_sweep<T, AX, LW, NT><<<grid, NT, smem, st>>>(dst, src, vel, g, T(g.s[AX]), rows, (int)tiles);
+    const unsigned grid = std::min(tiles, (unsigned)(res.sms * res.per_sm));
+    k_wide_sweep<T, AX, LW, NT, PART><<<grid, NT, smem, st>>>(dst, src, vel, g, T(g.s[AX]), rows, (int)tiles);
     return cudaGetLastError();
+}
+
+template <typename T, int AX, int LW, int NT>
+cudaError_t sweep_tiles(T *dst, const T *src, const T *vel, const WideGeo &g, int rows, unsigned tiles, cudaStream_t st)
+{
+    if constexpr (sizeof(T) == 8) {
+        const int64_t count = AX == 0 ? (int64_t)rows * g.n[0] : (int64_t)g.n[AX] << LW;
+        if (count <= NT * (kSweepCells - 1)) return go_sweep<T, AX, LW, NT, true>(dst, src, vel, g, rows, tiles, st);
+    }
+    return go_sweep<T, AX, LW, NT, false>(dst, src, vel, g, rows, tiles, st);
 }
 
 // The fused sweep, with 512 threads (2048 cells); lines over 256 cells along y or
@@ -459,25 +475,30 @@ bool sweep_fused(T *dst, const T *src, const T *vel, const WideGeo &g, cudaStrea
     const int64_t lines = g.ncell / n;
     if constexpr (AX == 0) {
         const int nt = n > 512 * kSweepCells ? 1024 : 512;
-        const int rows = (int)std::min<int64_t>(std::min(256, nt * kSweepCells / n), lines);
+        int rows = (int)std::min<int64_t>(std::min(256, nt * kSweepCells / n), lines);
+        // few lines in double precision, which the FP64 pipes bound: over all SMs, but a
+        // cell for every thread (16^3: two tiles of 128 rows, 51.2 us a step of each order;
+        // eight of 32, 27.6)
+        if (const DevCtx *c = sizeof(T) == 8 ? ctx_get() : nullptr)
+            rows = (int)std::min<int64_t>(rows, std::max<int64_t>((lines + c->num_sms - 1) / c->num_sms, std::max(1, nt / n)));
         const int64_t blocks = (lines + rows - 1) / rows;
         if (blocks > 0x7fffffff) return false;
-        e = nt == 1024 ? go_sweep<T, 0, 0, 1024>(dst, src, vel, g, rows, (unsigned)blocks, st)
-                       : go_sweep<T, 0, 0, 512>(dst, src, vel, g, rows, (unsigned)blocks, st);
+        e = nt == 1024 ? sweep_tiles<T, 0, 0, 1024>(dst, src, vel, g, rows, (unsigned)blocks, st)
+                       : sweep_tiles<T, 0, 0, 512>(dst, src, vel, g, rows, (unsigned)blocks, st);
     } else {
         const int lw = n <= 64 ? 5 : n <= 128 ? 4 : n <= 512 ? 3 : n <= 1024 ? 2 : n <= 2048 ? 1 : 0;
         const int64_t blocks = (((int64_t)g.n[0] + (1 << lw) - 1) >> lw) * (lines / g.n[0]);
         if (blocks > 0x7fffffff) return false;
         const unsigned b = (unsigned)blocks;
         switch (lw) {
-        case 5: e = n <= 32 ? go_sweep<T, AX, 5, 256>(dst, src, vel, g, 0, b, st)
-                            : go_sweep<T, AX, 5, 512>(dst, src, vel, g, 0, b, st); break;
-        case 4: e = go_sweep<T, AX, 4, 512>(dst, src, vel, g, 0, b, st); break;
-        case 3: e = n <= 256 ? go_sweep<T, AX, 3, 512>(dst, src, vel, g, 0, b, st)
-                             : go_sweep<T, AX, 3, 1024>(dst, src, vel, g, 0, b, st); break;
-        case 2: e = go_sweep<T, AX, 2, 1024>(dst, src, vel, g, 0, b, st); break;
-        case 1: e = go_sweep<T, AX, 1, 1024>(dst, src, vel, g, 0, b, st); break;
-        default: e = go_sweep<T, AX, 0, 1024>(dst, src, vel, g, 0, b, st); break;
+        case 5: e = n <= 32 ? sweep_tiles<T, AX, 5, 256>(dst, src, vel, g, 0, b, st)
+                            : sweep_tiles<T, AX, 5, 512>(dst, src, vel, g, 0, b, st); break;
+        case 4: e = sweep_tiles<T, AX, 4, 512>(dst, src, vel, g, 0, b, st); break;
+        case 3: e = n <= 256 ? sweep_tiles<T, AX, 3, 512>(dst, src, vel, g, 0, b, st)
+                             : sweep_tiles<T, AX, 3, 1024>(dst, src, vel, g, 0, b, st); break;
+        case 2: e = sweep_tiles<T, AX, 2, 1024>(dst, src, vel, g, 0, b, st); break;
+        case 1: e = sweep_tiles<T, AX, 1, 1024>(dst, src, vel, g, 0, b, st); break;
+        default: e = sweep_tiles<T, AX, 0, 1024>(dst, src, vel, g, 0, b, st); break;
         }
     }
     return true;
