@@ -266,9 +266,9 @@ __device__ __forceinline__ bool below(double c, int n)
 // Persistent CTAs; the loads of a CTA's next tile are issued before it works on
 // the current one, so that DRAM latency runs under the three gathers (without
 // that the y and z sweeps stalled on their loads).
-// PART: tiles of so few cells that a thread has none in its last turns; these are
-// skipped, which pays where double operations bound (8^3 SL_F64, a step of each order:
-// 50.7 -> 21.5 us; with the test in full tiles, 256^3, 3438 -> 3871).
+// PART: tiles of so few cells that some warps have none in some turns; they skip these,
+// which pays where double operations bound (8^3 SL_F64, a step of each order: 50.7 ->
+// 17.9 us; with the test in full tiles, 256^3, 3438 -> 3871).
 template <typename T, int AX, int LW, int NT, bool PART>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 1024 / NT : 1)
 k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict__ vel, WideGeo g, T sc, int rows,
@@ -295,7 +295,7 @@ k_wide_sweep(T *__restrict__ out, const T *__restrict__ src, const T *__restrict
     // place.  Cells beyond the tile's lines go to the spare place, and cells of a
     // partial tile beyond the grid work on zeros in places of their own.
     const int count = AX == 0 ? rows * n : n << LW;
-    const int turns = (count + NT - 1) / NT;
+    const int turns = (count - (tid & ~31) + NT - 1) / NT;   // of this warp
     auto has = [&](int k) { return !PART || k < turns; };
     int pos[E], line[E], own[E];
     bool rep[E];                                       // repeated at its line's end
@@ -473,21 +473,24 @@ bool sweep_fused(T *dst, const T *src, const T *vel, const WideGeo &g, cudaStrea
     const int n = g.n[AX];
     if (n > 1024 * kSweepCells) return false;
     const int64_t lines = g.ncell / n;
+    // Few tiles in double precision, which the FP64 pipes bound: smaller ones, over all
+    // SMs (16^3: two tiles of 128 rows and 16 column blocks, 51.2 us a step of each order,
+    // now 18.5; a 512 x 300 plane 72.2, now 34.8).
+    const DevCtx *const ctx = sizeof(T) == 8 ? ctx_get() : nullptr;
+    const int sms = ctx ? ctx->num_sms : 0;
     if constexpr (AX == 0) {
         const int nt = n > 512 * kSweepCells ? 1024 : 512;
         int rows = (int)std::min<int64_t>(std::min(256, nt * kSweepCells / n), lines);
-        // few lines in double precision, which the FP64 pipes bound: over all SMs, but a
-        // cell for every thread (16^3: two tiles of 128 rows, 51.2 us a step of each order;
-        // eight of 32, 27.6)
-        if (const DevCtx *c = sizeof(T) == 8 ? ctx_get() : nullptr)
-            rows = (int)std::min<int64_t>(rows, std::max<int64_t>((lines + c->num_sms - 1) / c->num_sms, std::max(1, nt / n)));
+        if ((lines + rows - 1) / rows * 2 <= sms) rows = (int)((lines + sms - 1) / sms);
         const int64_t blocks = (lines + rows - 1) / rows;
         if (blocks > 0x7fffffff) return false;
         e = nt == 1024 ? sweep_tiles<T, 0, 0, 1024>(dst, src, vel, g, rows, (unsigned)blocks, st)
                        : sweep_tiles<T, 0, 0, 512>(dst, src, vel, g, rows, (unsigned)blocks, st);
     } else {
-        const int lw = n <= 64 ? 5 : n <= 128 ? 4 : n <= 512 ? 3 : n <= 1024 ? 2 : n <= 2048 ? 1 : 0;
-        const int64_t blocks = (((int64_t)g.n[0] + (1 << lw) - 1) >> lw) * (lines / g.n[0]);
+        int lw = n <= 64 ? 5 : n <= 128 ? 4 : n <= 512 ? 3 : n <= 1024 ? 2 : n <= 2048 ? 1 : 0;
+        auto tiles = [&] { return (((int64_t)g.n[0] + (1 << lw) - 1) >> lw) * (lines / g.n[0]); };
+        while (lw > 1 && tiles() * 2 <= sms) --lw;   // 16 bytes of a row at least
+        const int64_t blocks = tiles();
         if (blocks > 0x7fffffff) return false;
         const unsigned b = (unsigned)blocks;
         switch (lw) {
