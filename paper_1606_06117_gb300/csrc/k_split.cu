@@ -26,7 +26,7 @@
 namespace sl {
 namespace {
 
-template <typename T, int TX, int TY>
+template <int TX, int TY>
 struct Shape {
     static constexpr int HW = TX + 8;                    // staged x in [-4, TX+4)
     static constexpr int PW = HW + 4;   // row stride
@@ -34,10 +34,10 @@ struct Shape {
 };
 
 // N consecutive elements from 16-byte aligned shared memory.
-template <typename T, int N>
-__device__ __forceinline__ void lds_vec(const T *src, T (&dst)[N])
+template <int N>
+__device__ __forceinline__ void lds_vec(const float *src, float (&dst)[N])
 {
-    static_assert(sizeof(T) == 4 && N % 4 == 0, "");
+    static_assert(N % 4 == 0, "");
 #pragma unroll
     for (int i = 0; i < N / 4; ++i) {
         const float4 v = reinterpret_cast<const float4 *>(src)[i];
@@ -45,8 +45,8 @@ __device__ __forceinline__ void lds_vec(const T *src, T (&dst)[N])
     }
 }
 
-template <typename T, int N>
-__device__ __forceinline__ void sts_vec(T *dst, const T (&src)[N])
+template <int N>
+__device__ __forceinline__ void sts_vec(float *dst, const float (&src)[N])
 {
 #pragma unroll
     for (int i = 0; i < N / 4; ++i)
@@ -62,9 +62,9 @@ __device__ __forceinline__ void sts_vec(T *dst, const T (&src)[N])
 // once per work item; wrapping every element of every plane again took most of
 // the time on grids whose rows are no multiple of 16 bytes (187 x 150 x 131,
 // x,y,z / z,y,x: 123 / 173 us before, 55 / 79 after, when this kernel served it).
-template <typename T, int NT, int NR, int NC, int LD, bool VEC>
+template <int NT, int NR, int NC, int LD, bool VEC>
 struct Stager {
-    static constexpr int V = VEC ? 16 / sizeof(T) : 1;
+    static constexpr int V = VEC ? 16 / sizeof(float) : 1;
     static constexpr int CPR = VEC ? NC / V : LD;
     static constexpr int N = NR * CPR;
     static constexpr int K = (N + NT - 1) / NT;
@@ -86,7 +86,7 @@ struct Stager {
         }
     }
 
-    __device__ __forceinline__ void issue(int tid, T *dst, const T *src) const
+    __device__ __forceinline__ void issue(int tid, float *dst, const float *src) const
     {
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -116,9 +116,9 @@ __device__ __forceinline__ void decode_item(int item, const Geo &g, int TX, int 
 }
 
 // ============================================================ order x, y, z
-template <typename T, typename D, int TX, int TY, bool HAS_Z, bool VEC>
+template <int TX, int TY, bool HAS_Z, bool VEC>
 struct XYZ {
-    using S = Shape<T, TX, TY>;
+    using S = Shape<TX, TY>;
     static constexpr int RX = 8, RY = 4;
     static constexpr int NT = TX * (TY / RY);
     static constexpr int NB = 2;
@@ -126,28 +126,28 @@ struct XYZ {
     static constexpr int SZ_CY = (TY + 4) * TX;
     static constexpr int SZ_CZ = HAS_Z ? TY * TX : 0;
     static constexpr int SZ_S1 = S::PH * TX;
-    static constexpr size_t smem() { return sizeof(T) * (size_t)(NB * (2 * SZ_PHI + SZ_CY + SZ_CZ) + SZ_S1); }
+    static constexpr size_t smem() { return sizeof(float) * (size_t)(NB * (2 * SZ_PHI + SZ_CY + SZ_CZ) + SZ_S1); }
 };
 
-template <typename T, typename D, int TX, int TY, bool HAS_Z, bool VEC>
-__device__ __forceinline__ void xyz_item(const Geo &g, int item, const T *__restrict__ in, T *__restrict__ out,
-                                         const T *__restrict__ vel, unsigned char *smem_raw, bool &bad)
+template <int TX, int TY, bool HAS_Z, bool VEC>
+__device__ __forceinline__ void xyz_item(const Geo &g, int item, const float *__restrict__ in, float *__restrict__ out,
+                                         const float *__restrict__ vel, unsigned char *smem_raw, bool &bad)
 {
-    using K = XYZ<T, D, TX, TY, HAS_Z, VEC>;
+    using K = XYZ<TX, TY, HAS_Z, VEC>;
     using S = typename K::S;
     constexpr int RX = K::RX, RY = K::RY, NT = K::NT, NB = K::NB;
-    T *sPhi = reinterpret_cast<T *>(smem_raw);
-    T *sCx = sPhi + NB * K::SZ_PHI;
-    T *sCy = sCx + NB * K::SZ_PHI;
-    T *sCz = sCy + NB * K::SZ_CY;
-    T *sS1 = sCz + NB * K::SZ_CZ;
+    float *sPhi = reinterpret_cast<float *>(smem_raw);
+    float *sCx = sPhi + NB * K::SZ_PHI;
+    float *sCy = sCx + NB * K::SZ_PHI;
+    float *sCz = sCy + NB * K::SZ_CY;
+    float *sS1 = sCz + NB * K::SZ_CZ;
 
     const int tid = threadIdx.x;
-    const D sx = D(g.sx), sy = D(g.sy), sz = D(g.sz);
+    const float sx = (float)g.sx, sy = (float)g.sy, sz = (float)g.sz;
 
-    Stager<T, NT, S::PH, S::HW, S::PW, VEC> stPhi;     // Phi and u_x: rows [-3,TY+3), cols [-4,TX+4)
-    Stager<T, NT, TY + 4, TX, TX, VEC> stCy;           // u_y: rows [-2,TY+2), cols [0,TX)
-    Stager<T, NT, TY, TX, TX, VEC> stCz;               // u_z: rows [0,TY), cols [0,TX)
+    Stager<NT, S::PH, S::HW, S::PW, VEC> stPhi;     // Phi and u_x: rows [-3,TY+3), cols [-4,TX+4)
+    Stager<NT, TY + 4, TX, TX, VEC> stCy;           // u_y: rows [-2,TY+2), cols [0,TX)
+    Stager<NT, TY, TX, TX, VEC> stCz;               // u_z: rows [0,TY), cols [0,TX)
 
     int x0, y0, z0, z1;
     decode_item(item, g, TX, TY, x0, y0, z0, z1);
@@ -170,7 +170,7 @@ __device__ __forceinline__ void xyz_item(const Geo &g, int item, const T *__rest
     };
 
     const int cx = tid % TX, yr = (tid / TX) * RY;     // y-sweep run / z columns of this thread
-    ZWin<T, D> win[RY];
+    ZWin win[RY];
 #pragma unroll
     for (int i = 0; i < RY; ++i) win[i].init();
 
@@ -182,49 +182,49 @@ __device__ __forceinline__ void xyz_item(const Geo &g, int item, const T *__rest
         if (p < plast) issue(p + 1, slot ^ 1);
 
         // ---- x sweep: rows [-3, TY+3) x cols [0, TX) -> sS1
-        const T *phiP = sPhi + slot * K::SZ_PHI;
-        const T *cxP = sCx + slot * K::SZ_PHI;
+        const float *phiP = sPhi + slot * K::SZ_PHI;
+        const float *cxP = sCx + slot * K::SZ_PHI;
         constexpr int XR = TX / RX;
         for (int r = tid; r < S::PH * XR; r += NT) {
             const int row = r / XR, xr = (r - (r / XR) * XR) * RX;
-            T blk[RX + 8];
-            lds_vec<T, RX + 8>(phiP + row * S::PW + xr, blk);
-            T pv[RX + 6];
+            float blk[RX + 8];
+            lds_vec<RX + 8>(phiP + row * S::PW + xr, blk);
+            float pv[RX + 6];
 #pragma unroll
             for (int k = 0; k < RX + 6; ++k) pv[k] = blk[k + 1];
-            lds_vec<T, RX + 8>(cxP + row * S::PW + xr, blk);
-            D cv[RX + 4];
+            lds_vec<RX + 8>(cxP + row * S::PW + xr, blk);
+            float cv[RX + 4];
 #pragma unroll
-            for (int k = 0; k < RX + 4; ++k) cv[k] = D(blk[k + 2]) * sx;
+            for (int k = 0; k < RX + 4; ++k) cv[k] = blk[k + 2] * sx;
 #pragma unroll
-            for (int k = 2; k < RX + 2; ++k) bad |= fabs(cv[k]) > D(1);
-            T o[RX];
-            cec_line<T, D, RX>(pv, cv, o);
-            sts_vec<T, RX>(sS1 + row * TX + xr, o);
+            for (int k = 2; k < RX + 2; ++k) bad |= fabs(cv[k]) > 1.f;
+            float o[RX];
+            cec_line<RX>(pv, cv, o);
+            sts_vec<RX>(sS1 + row * TX + xr, o);
         }
         __syncthreads();
 
         // ---- y sweep of this thread's run, then z windows
-        const T *cyP = sCy + slot * K::SZ_CY;
-        T pv[RY + 6];
+        const float *cyP = sCy + slot * K::SZ_CY;
+        float pv[RY + 6];
 #pragma unroll
         for (int k = 0; k < RY + 6; ++k) pv[k] = sS1[(yr + k) * TX + cx];
-        D cv[RY + 4];
+        float cv[RY + 4];
 #pragma unroll
-        for (int k = 0; k < RY + 4; ++k) cv[k] = D(cyP[(yr + k) * TX + cx]) * sy;
+        for (int k = 0; k < RY + 4; ++k) cv[k] = cyP[(yr + k) * TX + cx] * sy;
 #pragma unroll
-        for (int k = 2; k < RY + 2; ++k) bad |= fabs(cv[k]) > D(1);
-        T o[RY];
-        cec_line<T, D, RY>(pv, cv, o);
+        for (int k = 2; k < RY + 2; ++k) bad |= fabs(cv[k]) > 1.f;
+        float o[RY];
+        cec_line<RY>(pv, cv, o);
         const int gx = x0 + cx;
         if constexpr (HAS_Z) {
-            const T *czP = sCz + slot * K::SZ_CZ;
+            const float *czP = sCz + slot * K::SZ_CZ;
             const int kz = p - 3;
 #pragma unroll
             for (int i = 0; i < RY; ++i) {
-                const D c = D(czP[(yr + i) * TX + cx]) * sz;
-                bad |= fabs(c) > D(1);
-                const T v = win[i].push(o[i], c);
+                const float c = czP[(yr + i) * TX + cx] * sz;
+                bad |= fabs(c) > 1.f;
+                const float v = win[i].push(o[i], c);
                 const int gy = y0 + yr + i;
                 if (kz >= z0 && gx < g.nx && gy < g.ny) out[(int64_t)kz * g.plane + (int64_t)gy * g.nx + gx] = v;
             }
@@ -239,9 +239,9 @@ __device__ __forceinline__ void xyz_item(const Geo &g, int item, const T *__rest
     __syncthreads();   // shared buffers are reused by the next item
 }
 
-template <typename T, typename D, int TX, int TY, bool HAS_Z, bool VEC>
-__global__ void __launch_bounds__(XYZ<T, D, TX, TY, HAS_Z, VEC>::NT)
-k_cec_xyz(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel, Geo g, int64_t fin,
+template <int TX, int TY, bool HAS_Z, bool VEC>
+__global__ void __launch_bounds__(XYZ<TX, TY, HAS_Z, VEC>::NT)
+k_cec_xyz(const float *__restrict__ in, float *__restrict__ out, const float *__restrict__ vel, Geo g, int64_t fin,
           int64_t fout)
 {
     in += (int64_t)blockIdx.y * fin;   // field of this CTA (FieldSet)
@@ -250,14 +250,14 @@ k_cec_xyz(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
     const int nitems = g.tiles_x * g.tiles_y * g.chunks;
     bool bad = false;
     for (int item = blockIdx.x; item < nitems; item += gridDim.x)
-        xyz_item<T, D, TX, TY, HAS_Z, VEC>(g, item, in, out, vel, smem_raw, bad);
+        xyz_item<TX, TY, HAS_Z, VEC>(g, item, in, out, vel, smem_raw, bad);
     flag_cfl(g.status, bad);
 }
 
 // ============================================================ order z, y, x
-template <typename T, typename D, int TX, int TY, bool HAS_Z, bool VEC>
+template <int TX, int TY, bool HAS_Z, bool VEC>
 struct ZYX {
-    using S = Shape<T, TX, TY>;
+    using S = Shape<TX, TY>;
     static constexpr int RX = 4, RY = 4;
     static constexpr int NT = 256;
     static constexpr int NB = 2;
@@ -271,30 +271,30 @@ struct ZYX {
     static constexpr int SZ_CX = TY * S::PW;
     static constexpr size_t smem()
     {
-        return sizeof(T) * (size_t)(NB * (SZ_PHI + SZ_CZ + SZ_CY + SZ_CX) + SZ_Z + SZ_S2);
+        return sizeof(float) * (size_t)(NB * (SZ_PHI + SZ_CZ + SZ_CY + SZ_CX) + SZ_Z + SZ_S2);
     }
 };
 
-template <typename T, typename D, int TX, int TY, bool HAS_Z, bool VEC>
-__device__ __forceinline__ void zyx_item(const Geo &g, int item, const T *__restrict__ in, T *__restrict__ out,
-                                         const T *__restrict__ vel, unsigned char *smem_raw, bool &bad)
+template <int TX, int TY, bool HAS_Z, bool VEC>
+__device__ __forceinline__ void zyx_item(const Geo &g, int item, const float *__restrict__ in, float *__restrict__ out,
+                                         const float *__restrict__ vel, unsigned char *smem_raw, bool &bad)
 {
-    using K = ZYX<T, D, TX, TY, HAS_Z, VEC>;
+    using K = ZYX<TX, TY, HAS_Z, VEC>;
     using S = typename K::S;
     constexpr int RX = K::RX, RY = K::RY, NT = K::NT, NB = K::NB, NCOL = K::NCOL;
-    T *sPhi = reinterpret_cast<T *>(smem_raw);
-    T *sCz = sPhi + NB * K::SZ_PHI;
-    T *sCy = sCz + NB * K::SZ_CZ;
-    T *sCx = sCy + NB * K::SZ_CY;
-    T *sZ = sCx + NB * K::SZ_CX;
-    T *sS2 = sZ + K::SZ_Z;
+    float *sPhi = reinterpret_cast<float *>(smem_raw);
+    float *sCz = sPhi + NB * K::SZ_PHI;
+    float *sCy = sCz + NB * K::SZ_CZ;
+    float *sCx = sCy + NB * K::SZ_CY;
+    float *sZ = sCx + NB * K::SZ_CX;
+    float *sS2 = sZ + K::SZ_Z;
 
     const int tid = threadIdx.x;
-    const D sx = D(g.sx), sy = D(g.sy), sz = D(g.sz);
+    const float sx = (float)g.sx, sy = (float)g.sy, sz = (float)g.sz;
 
-    Stager<T, NT, S::PH, S::HW, S::PW, VEC> stPhi;     // Phi, u_z: rows [-3,TY+3), cols [-4,TX+4)
-    Stager<T, NT, TY + 4, S::HW, S::PW, VEC> stCy;     // u_y: rows [-2,TY+2)
-    Stager<T, NT, TY, S::HW, S::PW, VEC> stCx;         // u_x: rows [0,TY)
+    Stager<NT, S::PH, S::HW, S::PW, VEC> stPhi;     // Phi, u_z: rows [-3,TY+3), cols [-4,TX+4)
+    Stager<NT, TY + 4, S::HW, S::PW, VEC> stCy;     // u_y: rows [-2,TY+2)
+    Stager<NT, TY, S::HW, S::PW, VEC> stCx;         // u_x: rows [0,TY)
 
     int x0, y0, z0, z1;
     decode_item(item, g, TX, TY, x0, y0, z0, z1);
@@ -318,7 +318,7 @@ __device__ __forceinline__ void zyx_item(const Geo &g, int item, const T *__rest
         cp_async_commit();
     };
 
-    ZWin<T, D> win[NCOL];
+    ZWin win[NCOL];
 #pragma unroll
     for (int j = 0; j < NCOL; ++j) win[j].init();
 
@@ -329,20 +329,20 @@ __device__ __forceinline__ void zyx_item(const Geo &g, int item, const T *__rest
         __syncthreads();
         if (p < plast) issue(p + 1, slot ^ 1);
 
-        const T *zsrc = sPhi + slot * K::SZ_PHI;
+        const float *zsrc = sPhi + slot * K::SZ_PHI;
         int kz = 0;
         if constexpr (HAS_Z) {
             // ---- z sweep over columns x in [-3, TX+3), y in [-3, TY+3)
-            const T *czP = sCz + slot * K::SZ_CZ;
+            const float *czP = sCz + slot * K::SZ_CZ;
 #pragma unroll
             for (int j = 0; j < NCOL; ++j) {
                 const int r = tid + j * NT;
                 if (r < K::NZC) {
                     const int row = r / (TX + 6), col = r - (r / (TX + 6)) * (TX + 6) + 1;
-                    const D c = D(czP[row * S::PW + col]) * sz;
-                    const T v = win[j].push(zsrc[row * S::PW + col], c);
+                    const float c = czP[row * S::PW + col] * sz;
+                    const float v = win[j].push(zsrc[row * S::PW + col], c);
                     sZ[row * S::PW + col] = v;
-                    if (row >= 3 && row < TY + 3 && col >= 4 && col < TX + 4) bad |= fabs(c) > D(1);
+                    if (row >= 3 && row < TY + 3 && col >= 4 && col < TX + 4) bad |= fabs(c) > 1.f;
                 }
             }
             __syncthreads();
@@ -352,47 +352,47 @@ __device__ __forceinline__ void zyx_item(const Geo &g, int item, const T *__rest
         }
 
         // ---- y sweep: columns x in [-3, TX+3), rows [0, TY) -> sS2
-        const T *cyP = sCy + slot * K::SZ_CY;
+        const float *cyP = sCy + slot * K::SZ_CY;
         for (int r = tid; r < (TX + 6) * (TY / RY); r += NT) {
             const int col = r % (TX + 6) + 1, yr = (r / (TX + 6)) * RY;
-            T pv[RY + 6];
+            float pv[RY + 6];
 #pragma unroll
             for (int k = 0; k < RY + 6; ++k) pv[k] = zsrc[(yr + k) * S::PW + col];
-            D cv[RY + 4];
+            float cv[RY + 4];
 #pragma unroll
-            for (int k = 0; k < RY + 4; ++k) cv[k] = D(cyP[(yr + k) * S::PW + col]) * sy;
+            for (int k = 0; k < RY + 4; ++k) cv[k] = cyP[(yr + k) * S::PW + col] * sy;
             if (col >= 4 && col < TX + 4) {
 #pragma unroll
-                for (int k = 2; k < RY + 2; ++k) bad |= fabs(cv[k]) > D(1);
+                for (int k = 2; k < RY + 2; ++k) bad |= fabs(cv[k]) > 1.f;
             }
-            T o[RY];
-            cec_line<T, D, RY>(pv, cv, o);
+            float o[RY];
+            cec_line<RY>(pv, cv, o);
 #pragma unroll
             for (int i = 0; i < RY; ++i) sS2[(yr + i) * S::PW + col] = o[i];
         }
         __syncthreads();
 
         // ---- x sweep: rows [0, TY), cols [0, TX) -> global plane kz
-        const T *cxP = sCx + slot * K::SZ_CX;
+        const float *cxP = sCx + slot * K::SZ_CX;
         constexpr int XR = TX / RX;
         for (int r = tid; r < TY * XR; r += NT) {
             const int row = r / XR, xr = (r - (r / XR) * XR) * RX;
-            T blk[RX + 8];
-            lds_vec<T, RX + 8>(sS2 + row * S::PW + xr, blk);
-            T pv[RX + 6];
+            float blk[RX + 8];
+            lds_vec<RX + 8>(sS2 + row * S::PW + xr, blk);
+            float pv[RX + 6];
 #pragma unroll
             for (int k = 0; k < RX + 6; ++k) pv[k] = blk[k + 1];
-            lds_vec<T, RX + 8>(cxP + row * S::PW + xr, blk);
-            D cv[RX + 4];
+            lds_vec<RX + 8>(cxP + row * S::PW + xr, blk);
+            float cv[RX + 4];
 #pragma unroll
-            for (int k = 0; k < RX + 4; ++k) cv[k] = D(blk[k + 2]) * sx;
+            for (int k = 0; k < RX + 4; ++k) cv[k] = blk[k + 2] * sx;
 #pragma unroll
-            for (int k = 2; k < RX + 2; ++k) bad |= fabs(cv[k]) > D(1);
-            T o[RX];
-            cec_line<T, D, RX>(pv, cv, o);
+            for (int k = 2; k < RX + 2; ++k) bad |= fabs(cv[k]) > 1.f;
+            float o[RX];
+            cec_line<RX>(pv, cv, o);
             const int gy = y0 + row;
             if (gy < g.ny) {
-                T *dst = out + (int64_t)kz * g.plane + (int64_t)gy * g.nx + x0 + xr;
+                float *dst = out + (int64_t)kz * g.plane + (int64_t)gy * g.nx + x0 + xr;
                 if (VEC && x0 + xr + RX <= g.nx) {
                     reinterpret_cast<float4 *>(dst)[0] = make_float4(o[0], o[1], o[2], o[3]);
                 } else {
@@ -406,9 +406,9 @@ __device__ __forceinline__ void zyx_item(const Geo &g, int item, const T *__rest
     __syncthreads();
 }
 
-template <typename T, typename D, int TX, int TY, bool HAS_Z, bool VEC>
+template <int TX, int TY, bool HAS_Z, bool VEC>
 __global__ void __launch_bounds__(256)
-k_cec_zyx(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ vel, Geo g, int64_t fin,
+k_cec_zyx(const float *__restrict__ in, float *__restrict__ out, const float *__restrict__ vel, Geo g, int64_t fin,
           int64_t fout)
 {
     in += (int64_t)blockIdx.y * fin;   // field of this CTA (FieldSet)
@@ -417,28 +417,28 @@ k_cec_zyx(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
     const int nitems = g.tiles_x * g.tiles_y * g.chunks;
     bool bad = false;
     for (int item = blockIdx.x; item < nitems; item += gridDim.x)
-        zyx_item<T, D, TX, TY, HAS_Z, VEC>(g, item, in, out, vel, smem_raw, bad);
+        zyx_item<TX, TY, HAS_Z, VEC>(g, item, in, out, vel, smem_raw, bad);
     flag_cfl(g.status, bad);
 }
 
-template <typename T, typename D, int TX, int TY, bool HAS_Z, bool VEC>
+template <int TX, int TY, bool HAS_Z, bool VEC>
 cudaError_t dispatch_order(int parity, const Geo &g, int grid, const void *in, void *out, const void *vel,
                            const FieldSet &fs, cudaStream_t st)
 {
-    const T *i = static_cast<const T *>(in);
-    const T *v = static_cast<const T *>(vel);
-    T *o = static_cast<T *>(out);
+    const float *i = static_cast<const float *>(in);
+    const float *v = static_cast<const float *>(vel);
+    float *o = static_cast<float *>(out);
     if ((parity & 1) == 0) {
-        using K = XYZ<T, D, TX, TY, HAS_Z, VEC>;
-        auto kern = k_cec_xyz<T, D, TX, TY, HAS_Z, VEC>;
+        using K = XYZ<TX, TY, HAS_Z, VEC>;
+        auto kern = k_cec_xyz<TX, TY, HAS_Z, VEC>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem());
         if (e != cudaSuccess) return e;
         const int nitems = g.tiles_x * g.tiles_y * g.chunks;
         const int gr = grid > 0 && grid < nitems ? grid : nitems;
         kern<<<dim3(gr, fs.n), K::NT, K::smem(), st>>>(i, o, v, g, fs.fin, fs.fout);
     } else {
-        using K = ZYX<T, D, TX, TY / 2, HAS_Z, VEC>;
-        auto kern = k_cec_zyx<T, D, TX, TY / 2, HAS_Z, VEC>;
+        using K = ZYX<TX, TY / 2, HAS_Z, VEC>;
+        auto kern = k_cec_zyx<TX, TY / 2, HAS_Z, VEC>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem());
         if (e != cudaSuccess) return e;
         Geo g2 = g;
@@ -453,7 +453,7 @@ cudaError_t dispatch_order(int parity, const Geo &g, int grid, const void *in, v
 // ------------------------------------------------------------ batched
 // Persistent CTAs take (instance, tile, z-chunk) items from a device counter
 // until the batch is exhausted; every item is the same fused step as above.
-template <typename T, int TX, int TY, int PAR>
+template <int TX, int TY, int PAR>
 __global__ void __launch_bounds__(256)
 k_cec_batched(const BatchRec *__restrict__ recs, int ninst, int nitems, unsigned *counter, unsigned *status)
 {
@@ -473,13 +473,13 @@ k_cec_batched(const BatchRec *__restrict__ recs, int ninst, int nitems, unsigned
         }
         const BatchRec &r = recs[lo];
         const Geo g = r.g[PAR];
-        const T *in = static_cast<const T *>(PAR ? r.b : r.a);
-        T *out = static_cast<T *>(PAR ? r.a : r.b);
-        const T *vel = static_cast<const T *>(r.vel);
+        const float *in = static_cast<const float *>(PAR ? r.b : r.a);
+        float *out = static_cast<float *>(PAR ? r.a : r.b);
+        const float *vel = static_cast<const float *>(r.vel);
         if constexpr (PAR == 0)
-            xyz_item<T, T, TX, TY, true, true>(g, it - r.item0[0], in, out, vel, smem_raw, bad);
+            xyz_item<TX, TY, true, true>(g, it - r.item0[0], in, out, vel, smem_raw, bad);
         else
-            zyx_item<T, T, TX, TY / 2, true, true>(g, it - r.item0[1], in, out, vel, smem_raw, bad);
+            zyx_item<TX, TY / 2, true, true>(g, it - r.item0[1], in, out, vel, smem_raw, bad);
     }
     flag_cfl(status, bad);
 }
@@ -549,15 +549,15 @@ cudaError_t launch_split_cec(int dtype, const void *in, void *out, const void *v
     g.tiles_y = (g.ny + TY - 1) / TY;
     const bool vec = lc.aligned && g.nx % 4 == 0;
     if (has_z)
-        return vec ? dispatch_order<float, float, TX, TY, true, true>(parity, g, lc.grid, in, out, vel, fs, st)
-                   : dispatch_order<float, float, TX, TY, true, false>(parity, g, lc.grid, in, out, vel, fs, st);
-    return vec ? dispatch_order<float, float, TX, TY, false, true>(parity, g, lc.grid, in, out, vel, fs, st)
-               : dispatch_order<float, float, TX, TY, false, false>(parity, g, lc.grid, in, out, vel, fs, st);
+        return vec ? dispatch_order<TX, TY, true, true>(parity, g, lc.grid, in, out, vel, fs, st)
+                   : dispatch_order<TX, TY, true, false>(parity, g, lc.grid, in, out, vel, fs, st);
+    return vec ? dispatch_order<TX, TY, false, true>(parity, g, lc.grid, in, out, vel, fs, st)
+               : dispatch_order<TX, TY, false, false>(parity, g, lc.grid, in, out, vel, fs, st);
 }
 
 size_t batched_smem(int parity)
 {
-    return parity ? ZYX<float, float, 32, 16, true, true>::smem() : XYZ<float, float, 32, 32, true, true>::smem();
+    return parity ? ZYX<32, 16, true, true>::smem() : XYZ<32, 32, true, true>::smem();
 }
 
 void batched_tiles(int parity, int &tx, int &ty)
@@ -571,12 +571,12 @@ cudaError_t launch_batched_cec(const BatchRec *dev_recs, int ninst, int nitems, 
 {
     const size_t smem = batched_smem(parity);
     if (parity) {
-        auto kern = k_cec_batched<float, 32, 32, 1>;
+        auto kern = k_cec_batched<32, 32, 1>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         kern<<<grid, 256, smem, st>>>(dev_recs, ninst, nitems, counter, status);
     } else {
-        auto kern = k_cec_batched<float, 32, 32, 0>;
+        auto kern = k_cec_batched<32, 32, 0>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         kern<<<grid, 256, smem, st>>>(dev_recs, ninst, nitems, counter, status);
@@ -590,11 +590,11 @@ int batched_blocks_per_sm(int parity)
     const size_t smem = batched_smem(parity);
     cudaError_t e;
     if (parity) {
-        auto kern = k_cec_batched<float, 32, 32, 1>;
+        auto kern = k_cec_batched<32, 32, 1>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 256, smem);
     } else {
-        auto kern = k_cec_batched<float, 32, 32, 0>;
+        auto kern = k_cec_batched<32, 32, 0>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 256, smem);
     }

@@ -85,8 +85,7 @@ __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.lau
 //           = L_i + delta_i / 2 + (1 + U_i)/6 (delta_{i-s_i} - delta_i),
 // exact algebra on the definitions without 1/U.  Constant fields stay exact
 // (every difference is zero), C = +-1 is an exact shift (W = 0) and C = 0
-// keeps the cell.  D is the arithmetic type (float, or double with float
-// storage for SL_F32_D64).
+// keeps the cell.  In FP32; k_split64.cu has the forms in double arithmetic.
 
 // GB300 issues about two double operations per clock and SM, comparisons and
 // float-to-double conversions included, so double signs, bounds and widenings go
@@ -140,28 +139,28 @@ __device__ __forceinline__ V by_sign(D C, V pos, V neg, V zero)
 
 // Outputs o[0..R) of a line segment from p[0..R+6) = Phi at offsets -3..R+2
 // and c[0..R+4) = Courant numbers at offsets -2..R+1.
-template <typename T, typename D, int R>
-__device__ __forceinline__ void cec_line(const T (&p)[R + 6], const D (&c)[R + 4], T (&o)[R])
+template <int R>
+__device__ __forceinline__ void cec_line(const float (&p)[R + 6], const float (&c)[R + 4], float (&o)[R])
 {
-    D L[R + 4];                  // offsets -2..R+1 (index m <-> offset m-2, Phi at p[m+1])
+    float L[R + 4];                  // offsets -2..R+1 (index m <-> offset m-2, Phi at p[m+1])
 #pragma unroll
     for (int m = 0; m < R + 4; ++m) {
-        const D nb = by_sign(c[m], D(p[m]), D(p[m + 2]), D(p[m + 1]));
-        L[m] = nb + (D(1) - fabs(c[m])) * (D(p[m + 1]) - nb);
+        const float nb = by_sign(c[m], p[m], p[m + 2], p[m + 1]);
+        L[m] = nb + (1.f - fabs(c[m])) * (p[m + 1] - nb);
     }
-    D del[R + 2];                // offsets -1..R (index q <-> offset q-1)
+    float del[R + 2];                // offsets -1..R (index q <-> offset q-1)
 #pragma unroll
     for (int q = 0; q < R + 2; ++q) {
         const int m = q + 1;
-        const D Ln = by_sign(c[m], L[m + 1], L[m - 1], L[m]);
-        del[q] = (D(p[m + 1]) - L[m]) - fabs(c[m]) * (Ln - L[m]);
+        const float Ln = by_sign(c[m], L[m + 1], L[m - 1], L[m]);
+        del[q] = (p[m + 1] - L[m]) - fabs(c[m]) * (Ln - L[m]);
     }
 #pragma unroll
     for (int i = 0; i < R; ++i) {
         const int m = i + 2, q = i + 1;
-        const D U = fabs(c[m]);
-        const D dn = by_sign(c[m], del[q - 1], del[q + 1], del[q]);
-        o[i] = T(L[m] + D(0.5) * del[q] + (D(1) + U) * D(1.0 / 6.0) * (dn - del[q]));
+        const float U = fabs(c[m]);
+        const float dn = by_sign(c[m], del[q - 1], del[q + 1], del[q]);
+        o[i] = L[m] + 0.5f * del[q] + (1.f + U) * (1.f / 6.f) * (dn - del[q]);
     }
 }
 
@@ -169,33 +168,31 @@ __device__ __forceinline__ void cec_line(const T (&p)[R + 6], const D (&c)[R + 4
 // order with push(); after plane p is pushed, the result is the value at p - 3.
 // State after a push of plane p: Phi at p-1, p; L at p-2, p-1; Courant at p-2,
 // p-1; delta at p-3, p-2.
-template <typename T, typename D>
 struct ZWin {
-    D ph[2];   // Phi at p-2 (ph[0]), p-1 (ph[1])
-    D L[2];    // L at p-3, p-2
-    D c[2];    // Courant at p-3, p-2
-    D dl[2];   // delta at p-4, p-3
+    float ph[2];   // Phi at p-2 (ph[0]), p-1 (ph[1])
+    float L[2];    // L at p-3, p-2
+    float c[2];    // Courant at p-3, p-2
+    float dl[2];   // delta at p-4, p-3
 
     __device__ __forceinline__ void init()
     {
-        ph[0] = ph[1] = L[0] = L[1] = c[0] = c[1] = dl[0] = dl[1] = D(0);
+        ph[0] = ph[1] = L[0] = L[1] = c[0] = c[1] = dl[0] = dl[1] = 0.f;
     }
 
-    // phi_p: Phi at plane p; c_pm1: Courant number at plane p-1.
-    __device__ __forceinline__ T push(T phi_p, D c_pm1)
+    // phi: Phi at plane p; c_pm1: Courant number at plane p-1.
+    __device__ __forceinline__ float push(float phi, float c_pm1)
     {
-        const D phi = D(phi_p);
         // L at p-1 (Phi at p-2, p-1, p; Courant at p-1)
-        const D nb = by_sign(c_pm1, ph[0], phi, ph[1]);
-        const D Ln = nb + (D(1) - fabs(c_pm1)) * (ph[1] - nb);
+        const float nb = by_sign(c_pm1, ph[0], phi, ph[1]);
+        const float Ln = nb + (1.f - fabs(c_pm1)) * (ph[1] - nb);
         // delta at p-2 (Phi at p-2; L at p-3, p-2, p-1; Courant at p-2)
-        const D C2 = c[1];
-        const D Lb = by_sign(C2, Ln, L[0], L[1]);
-        const D dn = (ph[0] - L[1]) - fabs(C2) * (Lb - L[1]);
+        const float C2 = c[1];
+        const float Lb = by_sign(C2, Ln, L[0], L[1]);
+        const float dn = (ph[0] - L[1]) - fabs(C2) * (Lb - L[1]);
         // CEC at p-3 (L at p-3; delta at p-4, p-3, p-2; Courant at p-3)
-        const D C3 = c[0];
-        const D dd = by_sign(C3, dl[0], dn, dl[1]);
-        const T out = T(L[0] + D(0.5) * dl[1] + (D(1) + fabs(C3)) * D(1.0 / 6.0) * (dd - dl[1]));
+        const float C3 = c[0];
+        const float dd = by_sign(C3, dl[0], dn, dl[1]);
+        const float out = L[0] + 0.5f * dl[1] + (1.f + fabs(C3)) * (1.f / 6.f) * (dd - dl[1]);
         ph[0] = ph[1];
         ph[1] = phi;
         L[0] = L[1];
