@@ -110,13 +110,15 @@ int sl_advect(void *out, const void *in, const void *vel, int ndim,
  * bit to one sl_advect call per field.  Same arguments and errors as
  * sl_advect; every outs[f] must differ from every ins[g] and from the other
  * outs.  Since L_U is linear in Phi for a fixed velocity (Sec. 2), every field
- * shares the departure points and CEC weights; an SL_CEC step in FP32 on a 3D
- * grid of 8 planes or more advances up to 4 fields per launch: the launch's CTAs form groups, one CTA per field, that walk the
- * same (column tile, plane) sequence, so that a group's velocity reads can be
- * served from L2 after the first one.  Otherwise fields stored at uniform
- * strides (ins[f] = ins[0] + f * a, outs[f] = outs[0] + f * b, whole elements)
- * whose buffers share one 16-byte alignment run in one launch of the generic
- * kernels, a row of CTAs per field; other field sets take a launch per field.
+ * shares the departure points and CEC weights; an SL_CEC step in FP32 on the
+ * geometry of the persistent kernel (SL_KERNEL_CEC_FAST, see sl_autotune) advances
+ * up to 4 fields per launch, wherever they are: the launch's CTAs form groups, one
+ * CTA per field, that walk the same (column tile, plane) sequence, so that a
+ * group's velocity reads can be served from L2 after the first one.  Otherwise
+ * fields stored at uniform strides (ins[f] = ins[0] + f * a, outs[f] = outs[0] +
+ * f * b, whole elements) whose buffers share one 16-byte alignment run in one launch
+ * (SL_CEC in FP32 on other 3D grids of 8 planes or more: in such groups of up to 4
+ * fields); other field sets take a launch per field.
  */
 int sl_advect_multi(void *const *outs, const void *const *ins, int nfields,
                     const void *vel, int ndim, const int64_t dims[3],
@@ -497,8 +499,9 @@ int sl_advect_learned(sl_corrector *c, void *out, const void *in, const void *ve
  *   scheme sl_scheme; dtype SL_F64 or SL_F32 (the arithmetic of every step).
  *   Allocates all device buffers on the current device (about
  *   12 (nx + 6)(nz + 6) + 2 nx nz + 2 nx^2 + 3 nz^2 elements, and nx^2 nz more for small
- *   FP32 boxes and for FP64 boxes where these stay below 256 MB and the device has them); the state starts at
- *   rest (U = 0, theta = 0).  Errors: SL_ERR_ARG, SL_ERR_UNSUPPORTED,
+ *   boxes and for FP64 boxes where these stay below 256 MB and the device has them) and
+ *   fills their tables there (0.06 ms at 50 x 50, 6 ms at 48 x 4096); the state starts
+ *   at rest (U = 0, theta = 0).  Errors: SL_ERR_ARG, SL_ERR_UNSUPPORTED,
  *   SL_ERR_NOMEM, SL_ERR_CUDA.
  * sl_rb_set_state / sl_rb_get_state: DEVICE arrays of nz x nx elements of the
  *   box's dtype (row-major, x fastest) for u, w and theta, copied in / out on
