@@ -15,8 +15,9 @@
 //
 // Kernels: feature extraction for training samples, an FP32 minibatch
 // forward/backward kernel with an Adam update, and the inference step whose
-// two GEMMs run on the tensor cores (tcgen05.mma, BF16 operands staged in
-// shared memory, FP32 accumulators in tensor memory).
+// two GEMMs run on the tensor cores (tcgen05.mma, BF16; the weights and the last 16 K
+// columns of the activations in shared memory, the activations' first 64 columns and
+// the FP32 accumulators in tensor memory).
 #include <cuda_bf16.h>
 
 #include <cmath>

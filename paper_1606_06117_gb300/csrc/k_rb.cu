@@ -43,7 +43,8 @@
 // k_split64.cu, 23.0 (108) with four launches that overlap from their start, 21.5
 // (100) with the forces' terms on warps of their own, 17.8 (58) with the late release,
 // 16.3 (51) with one matrix per z mode for its x solve, 16.3 (42.5) with the overlap on
-// small boxes only.
+// small boxes only, 15.9 (42.6) now.  Boxes of one size differ by up to 3 % with where
+// their memory lies.
 #include <cmath>
 #include <new>
 

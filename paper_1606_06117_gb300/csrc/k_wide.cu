@@ -240,7 +240,7 @@ dim3 wide_grid(const WideGeo &g)
 // or more take a remainder first.
 // Measured (256^3 FP32 at CFL 3.64, us per step of three sweeps): 291 with the
 // Courant numbers in shared memory and three separate departure calculations
-// (170-179 instructions per cell and sweep), 178 now.
+// (170-179 instructions per cell and sweep), 187 now (178 replayed from a graph).
 // Cells per thread: with 4 a thread keeps to 64 registers, so that 32 warps fit an
 // SM (8 took 98).
 constexpr int kSweepCells = 4;
