@@ -240,7 +240,9 @@ k_unsplit(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ v
             t = (int)(w / nzz);
             const int64_t tile_w = (int64_t)t * nzz;
             const int o = (int)(w - tile_w);
-            const int rot = (int)(fmod((double)tile_w, share) + 0.5) % nzz;
+            // few planes stay in L2 in any order, and the remainder costs a tile of few
+            // planes a sixth of its time (CIR SL_F64, 2048 x 2048 x 1: 273 us with, 215 without)
+            const int rot = nzz < 8 ? 0 : (int)(fmod((double)tile_w, share) + 0.5) % nzz;
             const int64_t e = wend < tile_w + nzz ? wend : tile_w + nzz;
             z0 = o + rot;                   // in [0, 2 nz)
             z1 = z0 + (int)(e - w);

@@ -201,7 +201,7 @@ k_unsplit32(const float *__restrict__ in, float *__restrict__ out, const float *
         if (shares) {
             t = (int)(w / g.nz);
             const int64_t tile_w = (int64_t)t * g.nz;
-            const int rot = (int)(fmod((double)tile_w, share) + 0.5) % g.nz;
+            const int rot = g.nz < 8 ? 0 : (int)(fmod((double)tile_w, share) + 0.5) % g.nz;   // as k_unsplit.cu
             const int64_t e = wend < tile_w + g.nz ? wend : tile_w + g.nz;
             z0 = (int)(w - tile_w) + rot;   // planes are taken modulo nz
             z1 = z0 + (int)(e - w);
